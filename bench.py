@@ -41,7 +41,7 @@ FP64_PEAK_TFLOPS = SM_COUNT * 2 * 2 * SM_MAX_MHZ * 1e6 / 1e12
 FP32_PEAK_TFLOPS = SM_COUNT * 128 * 2 * SM_MAX_MHZ * 1e6 / 1e12
 
 
-KERNEL_SOURCES = ["include/nhmf.h", "paper_2505_15535_gb300/csrc/operators.cu",
+KERNEL_SOURCES = ["include/nhmf.h", "paper_2505_15535_gb300/csrc/operators.cuh",
                   "paper_2505_15535_gb300/csrc/sumfact.cuh", "paper_2505_15535_gb300/csrc/df64.cuh",
                   "paper_2505_15535_gb300/csrc/internal.h"]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_apply_fp64_cached_q2_64.traffic.json")

@@ -98,6 +98,7 @@ struct nhmf_ctx {
   nhmf::Geometry g;
   nhmf::Tables1D tab;
   int device = 0;
+  int sms = 1;                // SMs of the device
   double* ubar = nullptr;     // linearisation point, FP64
   float* ubar32 = nullptr;    // its FP32 copy (FP32 on-the-fly apply)
   double* cache64 = nullptr;  // [10][nq]
@@ -158,6 +159,15 @@ nhmf_status unet_record(nhmf_ctx* c, const double* r, const double* e, cudaStrea
 void unet_smooth_field(nhmf_ctx* c, double* e, unsigned long long seed, cudaStream_t s);
 int unet_snapshot_begin(nhmf_ctx* c, const double* r, const double* xj, cudaStream_t s);
 void unet_snapshot_finish(nhmf_ctx* c, int slot, const double* xstar, cudaStream_t s);
+
+// The operators of one degree (operators.cuh); operators.cu dispatches on the context's degree.
+template <int P>
+struct Operators {
+  static nhmf_status apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw, cudaStream_t s);
+  static nhmf_status cache(nhmf_ctx* c, cudaStream_t s);
+  static nhmf_status residual(nhmf_ctx* c, const double* u, double* r, cudaStream_t s);
+  static nhmf_status diagonal(nhmf_ctx* c, double* d, cudaStream_t s);
+};
 
 // raw = true applies the unconstrained operator K (no Dirichlet masking or identity rows).
 nhmf_status launch_apply(nhmf_ctx* c, int precision, int strategy, const void* du, void* v,

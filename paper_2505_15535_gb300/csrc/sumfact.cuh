@@ -62,6 +62,23 @@ template <> struct LaunchCfg<2, double, NHMF_ON_THE_FLY> {
   static constexpr int NE = NHMF_Q2D_OTF_NE, THREADS = NHMF_Q2D_OTF_THREADS;
 };
 
+// Block shapes: the launch shape above, and for the FP64 and double-float kernels (issue bound
+// within an SM) small blocks of one to four elements for meshes whose normal blocks would not give
+// every SM `per_sm` of them: a block of 27 Q2 elements keeps one SM's FP64 pipe busy for 34 us
+// while the others idle.  The line: FP64 cached apply, small / normal blocks, Q2 12^3 40 / 87 us,
+// 24^3 142 / 146, 32^3 312 / 306; Q4 12^3 113 / 119, 32^3 1819 / 1721.  Double-float blocks take
+// less time each: Q2 16^3 50 / 75 us, 24^3 101 / 94; Q4 8^3 49 / 67, 12^3 91 / 87.
+struct df64;
+template <typename T> struct SmallRule { static constexpr int per_sm = 4; };
+template <> struct SmallRule<df64> { static constexpr int per_sm = 2; };
+template <int P> struct SmallCfg;
+template <> struct SmallCfg<1> { static constexpr int NE = 4, THREADS = 32; };
+template <> struct SmallCfg<2> { static constexpr int NE = 3, THREADS = 96; };
+template <> struct SmallCfg<3> { static constexpr int NE = 1, THREADS = 64; };
+template <> struct SmallCfg<4> { static constexpr int NE = 1, THREADS = 128; };
+template <int P, typename T, int STRAT, bool SMALL> struct Shape : LaunchCfg<P, T, STRAT> {};
+template <int P, typename T, int STRAT> struct Shape<P, T, STRAT, true> : SmallCfg<P> {};
+
 // Coefficients of one n x n operator in even-odd form (odd n <= 5): S, A ((h+1) x h each) and C
 // (h+1), h = n / 2.
 constexpr int kEoSlots = 16;
@@ -142,6 +159,12 @@ __device__ __forceinline__ void st_policy(float* a, float v, unsigned long long 
   *a = v;
 #endif
 }
+// Programmatic dependent launch: let the stream's next launch start once every block of this one
+// has started; wait until the launches before this one are complete and their writes visible.
+// Both do nothing where a kernel is launched without the attribute.
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ bool is_constrained(int bc, int c, int gi, int gk, int M) {
   if (bc == NHMF_BC_CLAMP_X0) return gi == 0;
   if (bc == NHMF_BC_COMPRESSION) return gk == 0 || (c == 2 && gk == M - 1);
