@@ -204,6 +204,7 @@ void gmg_free(nhmf_ctx* c) {
     free_map(l.I);
     if (i + 1 < c->gmg->L.size()) nhmf_destroy(l.ctx);
   }
+  coarse_free(*c->gmg);
   delete c->gmg;
   c->gmg = nullptr;
 }
@@ -308,6 +309,10 @@ nhmf_status gmg_build(nhmf_ctx* c) {
       return fail(c, NHMF_ERR_OOM, "gmg: transfer maps");
     }
   }
+  if (!coarse_setup(G)) {
+    gmg_free(c);
+    return fail(c, NHMF_ERR_OOM, "gmg: coarse matrix");
+  }
   return NHMF_OK;
 }
 
@@ -369,6 +374,7 @@ nhmf_status gmg_prepare(nhmf_ctx* c, int strategy, bool fp32, cudaStream_t s, bo
                                             : power_iteration<double>(c, L, strategy, s);
     if (st != NHMF_OK) return st;
   }
+  if (G.coarse.blocks > 0 && (st = coarse_assemble(G, s)) != NHMF_OK) return st;
   return cuda_check(c, cudaGetLastError(), "gmg prepare");
 }
 

@@ -28,7 +28,18 @@ struct GmgLevel {
   Map1D I;   // interpolation of the linearisation point from this level to the coarser one
 };
 
+// The coarsest level's matrix and solve (coarse.cu).
+constexpr int kCoarseMaxN = 15;  // elements per direction up to which the level is a matrix
+struct CoarseSolve {
+  int blocks = 0;            // blocks of the solve's cluster; 0: the level is solved by pcg() on its operator
+  int R = 0, Rpad = 0;       // rows per block, padded
+  double *Ke = nullptr, *A64 = nullptr;
+  float* A32 = nullptr;
+  unsigned long long* words = nullptr;  // device: iterations since zeroed, status flags met
+};
+
 struct Gmg {
+  CoarseSolve coarse;
   std::vector<GmgLevel> L;  // L.back() mirrors the fine context (its ctx pointer is not owned)
 };
 
@@ -70,6 +81,13 @@ nhmf_status chebyshev(GmgLevel& L, int strat, const T* b, T* x, int degree, doub
 template <typename T> void gmg_restrict(GmgLevel& F, const T* r_fine, T* r_coarse, cudaStream_t s);
 template <typename T> void gmg_prolong_add(GmgLevel& F, const T* e_coarse, T* x_fine, T* scratch, cudaStream_t s);
 template <typename T> void gmg_bminus(long long n, const T* b, T* y, cudaStream_t s);
+bool coarse_setup(Gmg& G);
+void coarse_free(Gmg& G);
+// The coarsest operator's matrix at its level's linearisation point.
+nhmf_status coarse_assemble(Gmg& G, cudaStream_t s);
+// Jacobi-CG on it from x = 0, as pcg() does it; asynchronous, see CoarseSolve::words.
+template <typename T>
+nhmf_status coarse_cg(Gmg& G, const T* b, T* x, double rtol, int maxit, int check, cudaStream_t s);
 void gmg_start_vector(long long n, double* v, cudaStream_t s);
 
 }  // namespace nhmf

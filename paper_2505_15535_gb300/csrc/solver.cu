@@ -4,6 +4,7 @@
 // only every `check_every` iterations.
 #include <chrono>
 #include <cmath>
+#include <cstring>
 #include <limits>
 #include <type_traits>
 #include <vector>
@@ -86,6 +87,14 @@ nhmf_status read_scalar(Ctx& x, const double* dev, double* out) {
   nhmf_status st = cuda_check(x.c, cudaMemcpyAsync(x.w.host, dev, sizeof(double), cudaMemcpyDeviceToHost, x.s), "scalar read");
   if (st == NHMF_OK) st = cuda_check(x.c, cudaStreamSynchronize(x.s), "scalar sync");
   *out = x.w.host[0];
+  return st;
+}
+
+// The two counters of the multigrid coarse solves (CoarseSolve::words).
+nhmf_status read_words(Ctx& x, const unsigned long long* dev, unsigned long long (&h)[2]) {
+  nhmf_status st = cuda_check(x.c, cudaMemcpyAsync(x.w.host + 1, dev, sizeof(h), cudaMemcpyDeviceToHost, x.s), "counter read");
+  if (st == NHMF_OK) st = cuda_check(x.c, cudaStreamSynchronize(x.s), "counter sync");
+  std::memcpy(h, x.w.host + 1, sizeof(h));
   return st;
 }
 
@@ -218,9 +227,12 @@ nhmf_status pcg(Ctx& x, int strat, const T* b, T* sol, const T* dinv, T* r, T* z
 //   z = M(r); p = z - (z.q_prev / p_prev.q_prev) p_prev; alpha = p.r / p.q.
 // Returns NHMF_ERR_NOT_CONVERGED (with sol, w.r the current iterate and residual) when the
 // residual drops by less than stall_factor over stall_window iterations or maxit is reached.
+// `words`: the counters of the multigrid coarse solves inside precond (CoarseSolve::words), whose
+// status flags are read with p.q, or null.
 template <class Precond>
 nhmf_status fcg(Ctx& x, int strat, const double* b, double* sol, double rtol, int maxit, Precond&& precond,
-                long long* iters, double* relres, int stall_window = 0, double stall_factor = 1.0) {
+                long long* iters, double* relres, int stall_window = 0, double stall_factor = 1.0,
+                const unsigned long long* words = nullptr) {
   nhmf_ctx* c = x.c;
   SolverWork& w = x.w;
   double* sc = w.sc;
@@ -257,7 +269,15 @@ nhmf_status fcg(Ctx& x, int strat, const double* b, double* sol, double rtol, in
     std::swap(q, qprev);
     ++k;
     double pqh;
+    w.host[2] = 0.0;
+    if (words) cudaMemcpyAsync(w.host + 1, words, 2 * sizeof(double), cudaMemcpyDeviceToHost, x.s);
     if ((st = read_scalar(x, sc + PQ, &pqh)) != NHMF_OK) return st;
+    if (words) {
+      unsigned long long flags;
+      std::memcpy(&flags, w.host + 2, sizeof(flags));
+      if (flags & kStatusNonFinite) return fail(c, NHMF_ERR_NONFINITE, "multigrid coarse solve: non-finite residual");
+      if (flags & kStatusBreakdown) return fail(c, NHMF_ERR_BREAKDOWN, "multigrid coarse solve: p^T A p <= 0");
+    }
     if (!(pqh > 0.0)) return fail(c, NHMF_ERR_BREAKDOWN, "fcg: p^T A p <= 0");
     if ((st = norm(x, w.r, RNORM, &rn)) != NHMF_OK) return st;
     if (!std::isfinite(rn)) return fail(c, NHMF_ERR_NONFINITE, "fcg: non-finite residual");
@@ -424,6 +444,8 @@ nhmf_status vcycle(nhmf_ctx* c, int l, const nhmf_solve_opts& o, const T* b, T* 
   const bool fp32 = sizeof(T) == 4;
   const int strat = (fp32 && o.strategy == NHMF_SPATIAL) ? NHMF_ON_THE_FLY : o.strategy;
   nhmf_status st;
+  if (l == 0 && G.coarse.blocks > 0)  // one launch; iterations and failures are read by the caller
+    return coarse_cg<T>(G, b, x, fp32 ? 1e-4 : 1e-6, 5000, 10, s);
   if (l == 0) {
     Ctx cx{L.ctx, s, L.n, *L.ctx->work};
     long long it = 0;
@@ -543,8 +565,19 @@ nhmf_status linear(Ctx& x, const nhmf_solve_opts& o, const double* b, double* so
         gmg_start_vector(C0.n, C0.b, x.s);
         long long it = 0;
         double rel = 0.0;
-        nhmf_status ps = pcg<double>(cx, o.strategy, C0.b, C0.x, C0.dinv, C0.r, C0.d, C0.t1, C0.t2, 1e-6, 300, 10, RZ0,
-                                     &it, &rel);
+        nhmf_status ps = NHMF_OK;
+        if (x.c->gmg->coarse.blocks > 0) {
+          unsigned long long* words = x.c->gmg->coarse.words;
+          cudaMemsetAsync(words, 0, 2 * sizeof(unsigned long long), x.s);
+          if ((st = coarse_cg<double>(*x.c->gmg, C0.b, C0.x, 1e-6, 300, 10, x.s)) != NHMF_OK) return st;
+          unsigned long long h[2] = {0, 0};
+          if ((st = read_words(x, words, h)) != NHMF_OK) return st;
+          ps = (h[1] & kStatusNonFinite)   ? fail(C0.ctx, NHMF_ERR_NONFINITE, "coarse probe: non-finite residual")
+               : (h[1] & kStatusBreakdown) ? NHMF_ERR_BREAKDOWN
+                                           : NHMF_OK;
+        } else {
+          ps = pcg<double>(cx, o.strategy, C0.b, C0.x, C0.dinv, C0.r, C0.d, C0.t1, C0.t2, 1e-6, 300, 10, RZ0, &it, &rel);
+        }
         if (ps == NHMF_ERR_BREAKDOWN) {
           if ((st = gmg_prepare(x.c, o.strategy, f32, x.s, true, w.diag)) != NHMF_OK) return st;
         } else if (ps != NHMF_OK) {
@@ -552,6 +585,15 @@ nhmf_status linear(Ctx& x, const nhmf_solve_opts& o, const double* b, double* so
         }
       }
     }
+    unsigned long long* words = x.c->gmg->coarse.blocks > 0 ? x.c->gmg->coarse.words : nullptr;
+    if (words) cudaMemsetAsync(words, 0, 2 * sizeof(unsigned long long), x.s);
+    auto count_inner = [&](nhmf_status v) -> nhmf_status {  // the coarse solves' iterations
+      unsigned long long h[2] = {0, 0};
+      if (!words) return v;
+      const nhmf_status r = read_words(x, words, h);
+      *inner += (long long)h[0];
+      return v != NHMF_OK ? v : r;
+    };
     GmgLevel& top = x.c->gmg->L.back();
     const int ltop = (int)x.c->gmg->L.size() - 1;
     const int strat32 = o.strategy == NHMF_SPATIAL ? NHMF_ON_THE_FLY : o.strategy;
@@ -596,12 +638,12 @@ nhmf_status linear(Ctx& x, const nhmf_solve_opts& o, const double* b, double* so
       return cuda_check(x.c, cudaGetLastError(), "mixed gmg");
     };
     if (learned) {
-      st = fcg(x, o.strategy, b, sol, o.linear_rtol, std::max(1, o.linear_max_iter / 4), precond, outer, relres,
-               o.learned_stall_window, o.learned_stall_factor);
+      st = count_inner(fcg(x, o.strategy, b, sol, o.linear_rtol, std::max(1, o.linear_max_iter / 4), precond, outer,
+                           relres, o.learned_stall_window, o.learned_stall_factor, words));
       if (st == NHMF_ERR_BREAKDOWN) return restart_cg();
       return st == NHMF_ERR_NOT_CONVERGED ? fallback_cg() : st;
     }
-    st = fcg(x, o.strategy, b, sol, o.linear_rtol, o.linear_max_iter, precond, outer, relres);
+    st = count_inner(fcg(x, o.strategy, b, sol, o.linear_rtol, o.linear_max_iter, precond, outer, relres, 0, 1.0, words));
     if (st == NHMF_OK && !slots.empty()) {
       for (int slot : slots) unet_snapshot_finish(x.c, slot, sol, x.s);
       return cuda_check(x.c, cudaGetLastError(), "pair recording");
