@@ -220,11 +220,21 @@ nhmf_status nhmf_check_status(nhmf_ctx* c, void* stream) {
 }
 
 nhmf_status nhmf_set_linearization(nhmf_ctx* c, const double* u, int mask, void* stream) {
+  const nhmf_status st = set_linearization_async(c, u, mask, as_stream(stream));
+  if (st != NHMF_OK) return st;
+  c->have_lin = false;
+  const nhmf_status check = nhmf_check_status(c, stream);
+  c->have_lin = check == NHMF_OK;
+  return check;
+}
+
+}  // extern "C"
+
+nhmf_status nhmf::set_linearization_async(nhmf_ctx* c, const double* u, int mask, cudaStream_t s) {
   if (!c || !u || mask < 0 || mask > 15) return fail(c, NHMF_ERR_ARG, "set_linearization: bad argument");
   if (c->prm.model == NHMF_MODEL_SPLIT && (mask & (NHMF_CACHE_FP64 | NHMF_CACHE_FP32 | NHMF_CACHE_DF64)))
     return fail(c, NHMF_ERR_ARG, "set_linearization: the split model has only the spatial (Algorithm 2) cache");
   NvtxRange range("nhmf_set_linearization");
-  cudaStream_t s = as_stream(stream);
   const size_t n = 3 * c->g.M3;
   c->have_lin = false;
   nhmf_status st = cuda_check(c, cudaMemcpyAsync(c->ubar, u, n * sizeof(double), cudaMemcpyDeviceToDevice, s), "ubar copy");
@@ -253,10 +263,11 @@ nhmf_status nhmf_set_linearization(nhmf_ctx* c, const double* u, int mask, void*
   if (mask) {
     if ((st = launch_cache_build(c, s)) != NHMF_OK) return st;
   }
-  if ((st = nhmf_check_status(c, stream)) != NHMF_OK) return st;
   c->have_lin = true;
   return NHMF_OK;
 }
+
+extern "C" {
 
 nhmf_status nhmf_tangent_apply(nhmf_ctx* c, int precision, int strategy, const void* du, void* v, void* stream) {
   if (!c) return NHMF_ERR_ARG;

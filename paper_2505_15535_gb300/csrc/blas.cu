@@ -1,7 +1,7 @@
 // Vector kernels of the Krylov solvers (Section 2.3: CG on the matrix-free operator).
-// Reductions are deterministic: a fixed grid of kRedBlocks blocks accumulates FP64 partial
-// sums with a fixed grid-stride order and a fixed shuffle tree; one block then reduces the
-// partials in a fixed order.  Results stay on the device.
+// Reductions are deterministic: a grid that depends on the length alone accumulates FP64 partial
+// sums with a fixed grid-stride order and a fixed shuffle tree; the last block to finish reduces
+// the partials in a fixed order.  Results stay on the device.
 #include "blas.h"
 
 namespace nhmf {
@@ -13,66 +13,77 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Block-reduce NS accumulators and write partials[s * kRedBlocks + blockIdx.x].
+// Sums of NS values per thread over the grid: every block writes its partial sums, and the block
+// that comes last (a counter behind the partials, back at zero afterwards) adds them in block
+// order, so the sums do not depend on timing.  True, with the sums in `tot`, in that block's thread
+// 0 alone.  (A second launch for the final sum cost 3-4 us on every dot product.)
 template <int NS>
-__device__ __forceinline__ void block_partials(double (&acc)[NS], double* partials) {
+__device__ __forceinline__ bool grid_sum(double (&acc)[NS], double* partials, double (&tot)[NS]) {
   __shared__ double sh[NS][kRedThreads / 32];
+  __shared__ bool last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    double v = warp_sum(acc[s]);
-    if (lane == 0) sh[s][wid] = v;
-  }
-  __syncthreads();
-  if (wid == 0) {
+  auto block_sum = [&](double (&v)[NS]) {  // in warp 0's lane 0
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
-      double v = lane < kRedThreads / 32 ? sh[s][lane] : 0.0;
-      v = warp_sum(v);
-      if (lane == 0) partials[s * kRedBlocks + blockIdx.x] = v;
-    }
-  }
-}
-
-// out[s] = sum over partials of slot s; one block of kRedThreads threads.
-__global__ void k_final(const double* partials, int ns, double* out0, double* out1, double* out2) {
-  __shared__ double sh[kRedThreads / 32];
-  double* outs[3] = {out0, out1, out2};
-  for (int s = 0; s < ns; ++s) {
-    double v = 0.0;
-    for (int i = threadIdx.x; i < kRedBlocks; i += kRedThreads) v += partials[s * kRedBlocks + i];
-    v = warp_sum(v);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      double w = threadIdx.x < kRedThreads / 32 ? sh[threadIdx.x] : 0.0;
-      w = warp_sum(w);
-      if (threadIdx.x == 0 && outs[s]) *outs[s] = w;
+      v[s] = warp_sum(v[s]);
+      if (lane == 0) sh[s][wid] = v[s];
     }
     __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+      for (int s = 0; s < NS; ++s) v[s] = warp_sum(lane < kRedThreads / 32 ? sh[s][lane] : 0.0);
+    }
+  };
+  block_sum(acc);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) partials[s * kRedBlocks + blockIdx.x] = acc[s];
+    __threadfence();
+    last = atomicInc(reinterpret_cast<unsigned*>(partials + kRedBlocks * 3), gridDim.x - 1) == gridDim.x - 1;
   }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    tot[s] = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedThreads) tot[s] += __ldcg(partials + s * kRedBlocks + i);
+  }
+  block_sum(tot);
+  return threadIdx.x == 0;
 }
 
+// Blocks of a reduction over n values: at least four values a thread, at most kRedBlocks.
+unsigned red_blocks(long long n) {
+  const long long b = (n + 4 * kRedThreads - 1) / (4 * kRedThreads);
+  return (unsigned)(b < 1 ? 1 : (b > kRedBlocks ? kRedBlocks : b));
+}
+
+// *out = x . y, its square root if `root`; with `den`, also *quot = sign * *out / *den.
 template <typename TX, typename TY>
-__global__ void __launch_bounds__(kRedThreads) k_dot(long long n, const TX* x, const TY* y, double* partials) {
-  double acc[1] = {0.0};
-  for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)kRedBlocks * kRedThreads)
+__global__ void __launch_bounds__(kRedThreads) k_dot(long long n, const TX* x, const TY* y, double* partials, double* out,
+                                                     bool root, const double* den, double sign, double* quot) {
+  double acc[1] = {0.0}, tot[1];
+  for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads)
     acc[0] = fma(double(x[i]), double(y[i]), acc[0]);
-  block_partials<1>(acc, partials);
+  if (!grid_sum<1>(acc, partials, tot)) return;
+  const double v = root ? sqrt(tot[0]) : tot[0];
+  *out = v;
+  if (den) *quot = sign * (v / *den);
 }
 
 // PCG update (Jacobi): alpha = rz/pq; x += alpha p; r -= alpha q; z = dinv r;
-// partial sums of r.z and r.r.  A non-positive p.q is a breakdown: alpha = 0 and flag.
+// r.z and r.r.  A non-positive p.q is a breakdown: alpha = 0 and flag.
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_pcg_update(long long n, const double* rz, const double* pq, T* x, T* r,
-                                                            const T* p, const T* q, const T* dinv, T* z,
-                                                            double* partials, unsigned* flag) {
+                                                            const T* p, const T* q, const T* dinv, T* z, double* partials,
+                                                            double* rz_new, double* rr, unsigned* flag) {
   const double pqv = *pq;
   const bool ok = pqv > 0.0 && isfinite(pqv);
   const T alpha = ok ? T(*rz / pqv) : T(0);
   if (!ok && blockIdx.x == 0 && threadIdx.x == 0) atomicOr(flag, 4u);
-  double acc[2] = {0.0, 0.0};
-  for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)kRedBlocks * kRedThreads) {
+  double acc[2] = {0.0, 0.0}, tot[2];
+  for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads) {
     x[i] = fma(alpha, p[i], x[i]);
     const T ri = fma(-alpha, q[i], r[i]);
     r[i] = ri;
@@ -81,7 +92,37 @@ __global__ void __launch_bounds__(kRedThreads) k_pcg_update(long long n, const d
     acc[0] = fma(double(ri), double(zi), acc[0]);
     acc[1] = fma(double(ri), double(ri), acc[1]);
   }
-  block_partials<2>(acc, partials);
+  if (!grid_sum<2>(acc, partials, tot)) return;
+  *rz_new = tot[0];
+  *rr = tot[1];
+}
+
+// Flexible CG: *pq = p.q, *alpha = p.r / p.q.
+__global__ void __launch_bounds__(kRedThreads) k_fcg_alpha(long long n, const double* p, const double* q, const double* r,
+                                                           double* partials, double* pq, double* alpha) {
+  double acc[2] = {0.0, 0.0}, tot[2];
+  for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads) {
+    acc[0] = fma(p[i], q[i], acc[0]);
+    acc[1] = fma(p[i], r[i], acc[1]);
+  }
+  if (!grid_sum<2>(acc, partials, tot)) return;
+  *pq = tot[0];
+  *alpha = tot[1] / tot[0];
+}
+
+// x += alpha p, r -= alpha q, *rnorm = ||r||.
+__global__ void __launch_bounds__(kRedThreads) k_fcg_update(long long n, const double* alpha, const double* p,
+                                                            const double* q, double* x, double* r, double* partials,
+                                                            double* rnorm) {
+  const double al = *alpha;
+  double acc[1] = {0.0}, tot[1];
+  for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads) {
+    x[i] = fma(al, p[i], x[i]);
+    const double ri = fma(-al, q[i], r[i]);
+    r[i] = ri;
+    acc[0] = fma(ri, ri, acc[0]);
+  }
+  if (grid_sum<1>(acc, partials, tot)) *rnorm = sqrt(tot[0]);
 }
 
 // p = z + beta p with beta = rz_new / rz_old (beta = 0 when rz_old is null).
@@ -92,17 +133,20 @@ __global__ void k_pcg_direction(long long n, const double* rz_new, const double*
     p[i] = rz_old ? fma(beta, p[i], z[i]) : z[i];
 }
 
-// z = dinv r and partial sums of r.z, r.r (start of PCG).
+// z = dinv r, r.z and r.r (start of PCG).
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_jacobi(long long n, const T* r, const T* dinv, T* z, double* partials) {
-  double acc[2] = {0.0, 0.0};
-  for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)kRedBlocks * kRedThreads) {
+__global__ void __launch_bounds__(kRedThreads) k_jacobi(long long n, const T* r, const T* dinv, T* z, double* partials,
+                                                        double* rz, double* rr) {
+  double acc[2] = {0.0, 0.0}, tot[2];
+  for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads) {
     const T zi = dinv[i] * r[i];
     z[i] = zi;
     acc[0] = fma(double(r[i]), double(zi), acc[0]);
     acc[1] = fma(double(r[i]), double(r[i]), acc[1]);
   }
-  block_partials<2>(acc, partials);
+  if (!grid_sum<2>(acc, partials, tot)) return;
+  *rz = tot[0];
+  *rr = tot[1];
 }
 
 // y = a x + b y with scalars a = sa * (*pa) (pa may be null -> sa), same for b.
@@ -156,37 +200,40 @@ __global__ void k_mul(long long n, const double* d, double* x) {
     x[i] *= d[i];
 }
 
-__global__ void k_sqrt(double* x) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *x = sqrt(*x);
-}
-
 constexpr int kEwBlocks = 1216;  // 8 blocks per SM for element-wise kernels
 constexpr int kEwThreads = 256;
 
 }  // namespace
 
 void dot(long long n, const double* x, const double* y, double* out, double* partials, cudaStream_t s) {
-  k_dot<<<kRedBlocks, kRedThreads, 0, s>>>(n, x, y, partials);
-  k_final<<<1, kRedThreads, 0, s>>>(partials, 1, out, nullptr, nullptr);
+  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, y, partials, out, false, nullptr, 0.0, nullptr);
 }
 void dot(long long n, const float* x, const float* y, double* out, double* partials, cudaStream_t s) {
-  k_dot<<<kRedBlocks, kRedThreads, 0, s>>>(n, x, y, partials);
-  k_final<<<1, kRedThreads, 0, s>>>(partials, 1, out, nullptr, nullptr);
+  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, y, partials, out, false, nullptr, 0.0, nullptr);
+}
+void dot_ratio(long long n, const double* x, const double* y, double* out, const double* den, double sign, double* quot,
+               double* partials, cudaStream_t s) {
+  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, y, partials, out, false, den, sign, quot);
 }
 void norm2(long long n, const double* x, double* out, double* partials, cudaStream_t s) {
-  dot(n, x, x, out, partials, s);
-  k_sqrt<<<1, 32, 0, s>>>(out);
+  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, x, partials, out, true, nullptr, 0.0, nullptr);
 }
 void norm2(long long n, const float* x, double* out, double* partials, cudaStream_t s) {
-  dot(n, x, x, out, partials, s);
-  k_sqrt<<<1, 32, 0, s>>>(out);
+  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, x, partials, out, true, nullptr, 0.0, nullptr);
+}
+void fcg_alpha(long long n, const double* p, const double* q, const double* r, double* pq, double* alpha,
+               double* partials, cudaStream_t s) {
+  k_fcg_alpha<<<red_blocks(n), kRedThreads, 0, s>>>(n, p, q, r, partials, pq, alpha);
+}
+void fcg_update(long long n, const double* alpha, const double* p, const double* q, double* x, double* r, double* rnorm,
+                double* partials, cudaStream_t s) {
+  k_fcg_update<<<red_blocks(n), kRedThreads, 0, s>>>(n, alpha, p, q, x, r, partials, rnorm);
 }
 
 template <typename T>
 void pcg_update(long long n, const double* rz, const double* pq, T* x, T* r, const T* p, const T* q, const T* dinv, T* z,
                 double* rz_new, double* rr, double* partials, unsigned* flag, cudaStream_t s) {
-  k_pcg_update<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, rz, pq, x, r, p, q, dinv, z, partials, flag);
-  k_final<<<1, kRedThreads, 0, s>>>(partials, 2, rz_new, rr, nullptr);
+  k_pcg_update<T><<<red_blocks(n), kRedThreads, 0, s>>>(n, rz, pq, x, r, p, q, dinv, z, partials, rz_new, rr, flag);
 }
 template <typename T>
 void pcg_direction(long long n, const double* rz_new, const double* rz_old, const T* z, T* p, cudaStream_t s) {
@@ -194,8 +241,7 @@ void pcg_direction(long long n, const double* rz_new, const double* rz_old, cons
 }
 template <typename T>
 void jacobi(long long n, const T* r, const T* dinv, T* z, double* rz, double* rr, double* partials, cudaStream_t s) {
-  k_jacobi<T><<<kRedBlocks, kRedThreads, 0, s>>>(n, r, dinv, z, partials);
-  k_final<<<1, kRedThreads, 0, s>>>(partials, 2, rz, rr, nullptr);
+  k_jacobi<T><<<red_blocks(n), kRedThreads, 0, s>>>(n, r, dinv, z, partials, rz, rr);
 }
 template void pcg_update<double>(long long, const double*, const double*, double*, double*, const double*, const double*,
                                  const double*, double*, double*, double*, double*, unsigned*, cudaStream_t);

@@ -4,12 +4,22 @@
 
 namespace nhmf {
 
-constexpr int kRedBlocks = 1024;   // fixed reduction grid: results do not depend on timing
+constexpr int kRedBlocks = 1024;   // largest reduction grid
 constexpr int kRedThreads = 256;
-constexpr int kPartialSlots = 3 * kRedBlocks;  // scratch doubles a reduction needs
+// Scratch doubles that a reduction needs: three partial sums per block and a counter, which is
+// zero before the first use.  Reductions that share it run one after another.
+constexpr int kPartialSlots = 3 * kRedBlocks + 2;
 
 void dot(long long n, const double* x, const double* y, double* out, double* partials, cudaStream_t s);
 void dot(long long n, const float* x, const float* y, double* out, double* partials, cudaStream_t s);
+// *out = x . y and *quot = sign * *out / *den
+void dot_ratio(long long n, const double* x, const double* y, double* out, const double* den, double sign, double* quot,
+               double* partials, cudaStream_t s);
+// flexible CG: *pq = p . q and *alpha = p . r / p . q; x += alpha p, r -= alpha q and *rnorm = ||r||
+void fcg_alpha(long long n, const double* p, const double* q, const double* r, double* pq, double* alpha,
+               double* partials, cudaStream_t s);
+void fcg_update(long long n, const double* alpha, const double* p, const double* q, double* x, double* r, double* rnorm,
+                double* partials, cudaStream_t s);
 void norm2(long long n, const double* x, double* out, double* partials, cudaStream_t s);
 void norm2(long long n, const float* x, double* out, double* partials, cudaStream_t s);
 template <typename T>

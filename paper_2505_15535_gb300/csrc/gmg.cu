@@ -9,6 +9,7 @@
 // of 1D maps applied as three passes.
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <vector>
 
 #include "blas.h"
@@ -19,26 +20,40 @@ namespace nhmf {
 namespace {
 
 // ------------------------------------------------------------------ kernels
-// One 1D pass along `dir` of a [3][nz][ny][nx] field: out(.., i_dir, ..) = sum_k w_k in(.., col_k, ..).
+__device__ __forceinline__ bool constrained(int bc, int c, int i, int k, int M) {
+  if (bc == NHMF_BC_CLAMP_X0) return i == 0;
+  if (bc == NHMF_BC_COMPRESSION) return k == 0 || (c == 2 && k == M - 1);
+  return false;
+}
+
+// One 1D pass along `dir` of a [3][nz][ny][nx] field: out(.., i_dir, ..) = sum_k w_k in(.., col_k, ..),
+// added to out if `add`, and zero on the constrained DoFs of preset `bc` on an ox^3 grid.  Grid: x
+// covers an output z-plane, y the planes, z the components.
 template <typename T>
-__global__ void k_map1d(const T* __restrict__ in, T* __restrict__ out, int dir, int nx, int ny, int nz, int mout,
-                        const int* __restrict__ ptr, const int* __restrict__ col, const T* __restrict__ w) {
+__global__ void __launch_bounds__(256) k_map1d(const T* __restrict__ in, T* __restrict__ out, int dir, int nx, int ny,
+                                               int nz, int mout, const int* __restrict__ ptr,
+                                               const int* __restrict__ col, const T* __restrict__ w, bool add, int bc) {
   const int ox = dir == 0 ? mout : nx, oy = dir == 1 ? mout : ny, oz = dir == 2 ? mout : nz;
-  const long long plane = (long long)ox * oy * oz;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < 3 * plane;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int c = int(idx / plane);
-    const long long rem = idx % plane;
-    const int i = int(rem % ox), j = int((rem / ox) % oy), k = int(rem / ((long long)ox * oy));
-    const int row = dir == 0 ? i : (dir == 1 ? j : k);
-    T s = T(0);
-    for (int e = ptr[row]; e < ptr[row + 1]; ++e) {
-      const int cc = col[e];
-      const int ii = dir == 0 ? cc : i, jj = dir == 1 ? cc : j, kk = dir == 2 ? cc : k;
-      s = fma(w[e], in[(long long)c * nx * ny * nz + ii + (long long)nx * (jj + (long long)ny * kk)], s);
-    }
-    out[idx] = s;
+  const int ij = blockIdx.x * 256 + threadIdx.x, k = blockIdx.y, c = blockIdx.z;
+  if (ij >= ox * oy) return;
+  const int j = ij / ox, i = ij - j * ox, row = dir == 0 ? i : (dir == 1 ? j : k);
+  const T* src = in + (long long)c * nx * ny * nz;
+  long long step;  // of the contracted index
+  if (dir == 0) {
+    src += (long long)nx * (j + (long long)ny * k);
+    step = 1;
+  } else if (dir == 1) {
+    src += i + (long long)nx * ny * k;
+    step = nx;
+  } else {
+    src += i + (long long)nx * j;
+    step = (long long)nx * ny;
   }
+  T s = T(0);
+  for (int e = ptr[row]; e < ptr[row + 1]; ++e) s = fma(w[e], src[step * col[e]], s);
+  if (bc != NHMF_BC_NONE && constrained(bc, c, i, k, ox)) s = T(0);
+  T* o = out + (long long)c * ox * oy * oz + (long long)ox * oy * k + ij;
+  *o = add ? *o + s : s;
 }
 
 // Chebyshev step: d = c_old d + c_new D^-1 (b - q), x += d (q null: q = 0).
@@ -60,13 +75,6 @@ __global__ void k_bminus(long long n, const T* __restrict__ b, T* __restrict__ y
     y[i] = b[i] - y[i];
 }
 
-// x += y
-template <typename T>
-__global__ void k_add(long long n, const T* __restrict__ y, T* __restrict__ x) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    x[i] += y[i];
-}
-
 // deterministic start vector of the power iteration: values in [0.5, 1.5) from a hash of i
 __global__ void k_start(long long n, double* v) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -76,18 +84,11 @@ __global__ void k_start(long long n, double* v) {
   }
 }
 
-// x *= 1 / *nrm (x stays as it is when *nrm is not positive)
+// x = D^-1 q / 4, a power-iteration step from q = A x
 template <typename T>
-__global__ void k_scale_inv(long long n, const double* __restrict__ nrm, T* __restrict__ x) {
-  const double s = *nrm > 0.0 ? 1.0 / *nrm : 1.0;
+__global__ void k_power(long long n, const T* __restrict__ dinv, const T* __restrict__ q, T* __restrict__ x) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    x[i] = T(x[i] * s);
-}
-
-template <typename T>
-__global__ void k_mul_t(long long n, const T* __restrict__ a, T* __restrict__ x) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    x[i] *= a[i];
+    x[i] = T(0.25) * dinv[i] * q[i];
 }
 
 template <typename T>
@@ -181,13 +182,15 @@ template <typename T> const T* wts(const Map1D& m);
 template <> const double* wts<double>(const Map1D& m) { return m.w64; }
 template <> const float* wts<float>(const Map1D& m) { return m.w32; }
 
-// out (M_out^3) = (map x map x map) in (M_in^3), using two temporaries
+// out (M_out^3) (+)= (map x map x map) in (M_in^3), using two temporaries; zero on the constrained
+// DoFs of preset `bc`
 template <typename T>
-void map3d(const Map1D& m, const T* in, T* out, T* t1, T* t2, cudaStream_t s) {
+void map3d(const Map1D& m, const T* in, T* out, T* t1, T* t2, cudaStream_t s, bool add = false, int bc = NHMF_BC_NONE) {
   const int mi = m.cols, mo = m.rows;
-  k_map1d<T><<<kB, kT, 0, s>>>(in, t1, 0, mi, mi, mi, mo, m.ptr, m.col, wts<T>(m));
-  k_map1d<T><<<kB, kT, 0, s>>>(t1, t2, 1, mo, mi, mi, mo, m.ptr, m.col, wts<T>(m));
-  k_map1d<T><<<kB, kT, 0, s>>>(t2, out, 2, mo, mo, mi, mo, m.ptr, m.col, wts<T>(m));
+  auto grid = [](int ox, int oy, int oz) { return dim3((unsigned)((ox * oy + 255) / 256), (unsigned)oz, 3u); };
+  k_map1d<T><<<grid(mo, mi, mi), 256, 0, s>>>(in, t1, 0, mi, mi, mi, mo, m.ptr, m.col, wts<T>(m), false, NHMF_BC_NONE);
+  k_map1d<T><<<grid(mo, mo, mi), 256, 0, s>>>(t1, t2, 1, mo, mi, mi, mo, m.ptr, m.col, wts<T>(m), false, NHMF_BC_NONE);
+  k_map1d<T><<<grid(mo, mo, mo), 256, 0, s>>>(t2, out, 2, mo, mo, mi, mo, m.ptr, m.col, wts<T>(m), add, bc);
 }
 
 }  // namespace
@@ -215,7 +218,7 @@ void gmg_free(nhmf_ctx* c) {
 nhmf_status gmg_build(nhmf_ctx* c) {
   if (c->gmg) return NHMF_OK;
   std::vector<int> Ns{c->g.N}, Ps{c->g.p};
-  while (Ns.back() % 2 == 0 && Ns.back() / 2 >= 2 && Ns.size() < 12) {
+  while (Ns.back() % 2 == 0 && Ns.back() / 2 >= 2 && (int)Ns.size() < kMaxLevels - 1) {
     Ns.push_back(Ns.back() / 2);
     Ps.push_back(c->g.p);
   }
@@ -316,33 +319,36 @@ nhmf_status gmg_build(nhmf_ctx* c) {
   return NHMF_OK;
 }
 
-// Power iteration for the largest eigenvalue of D^-1 A on level L in precision T (12 steps).
-// The vector is normalised on the device; the host reads the two norms once at the end.
+// Enqueues the power iteration for the largest eigenvalue of D^-1 A on level L in precision T (12
+// steps of x <- D^-1 A x / 4: the factor is exact and keeps 12 steps far from overflow, so no step
+// normalises), and the norms of its last two vectors into sc[40], sc[41].
 template <typename T>
-nhmf_status power_iteration(nhmf_ctx* c, GmgLevel& L, int strategy, cudaStream_t s) {
+nhmf_status power_iteration(GmgLevel& L, int strategy, cudaStream_t s) {
   T* x = Buf<T>::x(L);
   T* q = Buf<T>::q(L);
   const T* dinv = Buf<T>::dinv(L);
-  double* sc = L.ctx->work->sc;
+  SolverWork& w = *L.ctx->work;
   nhmf_status st;
   k_start<<<kB, kT, 0, s>>>(L.n, L.x);
   if constexpr (sizeof(T) == 4) k_to<float><<<kB, kT, 0, s>>>(L.n, L.x, L.x32);
   for (int it = 0; it < 12; ++it) {
-    if ((st = launch_apply(L.ctx, sizeof(T) == 8 ? NHMF_FP64 : NHMF_FP32, strategy, x, q, s)) != NHMF_OK) return st;
-    k_mul_t<T><<<kB, kT, 0, s>>>(L.n, dinv, q);
-    norm2(L.n, x, sc + 40, L.ctx->work->partials, s);
-    norm2(L.n, q, sc + 41, L.ctx->work->partials, s);
-    cudaMemcpyAsync(x, q, L.n * sizeof(T), cudaMemcpyDeviceToDevice, s);
-    k_scale_inv<T><<<kB, kT, 0, s>>>(L.n, sc + 41, x);
+    if (it == 11) norm2(L.n, x, w.sc + 40, w.partials, s);
+    if constexpr (sizeof(T) == 4) {
+      Gather32 g;
+      g.mode = Gather32::kPower;
+      g.dinv = dinv;
+      if ((st = launch_apply32(L.ctx, strategy, x, x, g, s)) != NHMF_OK) return st;
+    } else {
+      if ((st = launch_apply(L.ctx, NHMF_FP64, strategy, x, q, s)) != NHMF_OK) return st;
+      k_power<T><<<kB, kT, 0, s>>>(L.n, dinv, q, x);
+    }
   }
-  double h[2];
-  cudaMemcpyAsync(h, sc + 40, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
-  if ((st = cuda_check(c, cudaStreamSynchronize(s), "gmg power iteration")) != NHMF_OK) return st;
-  L.lmax = (h[0] > 0.0 && h[1] > 0.0) ? h[1] / h[0] : 2.0;
+  norm2(L.n, x, w.sc + 41, w.partials, s);
   return NHMF_OK;
 }
 
-// Level linearisation points, diagonals and eigenvalue estimates at the fine point c->ubar.
+// Level linearisation points, diagonals and eigenvalue estimates at the fine point c->ubar.  All
+// of it is enqueued before the host reads the levels' status words and norms, in one wait.
 nhmf_status gmg_prepare(nhmf_ctx* c, int strategy, bool fp32, cudaStream_t s, bool coarse_at_zero,
                         const double* fine_diag) {
   nhmf_status st = gmg_build(c);
@@ -351,6 +357,8 @@ nhmf_status gmg_prepare(nhmf_ctx* c, int strategy, bool fp32, cudaStream_t s, bo
   const int nl = (int)G.L.size();
   const int mask = strategy == NHMF_CACHED ? (NHMF_CACHE_FP64 | (fp32 ? NHMF_CACHE_FP32 : 0))
                    : strategy == NHMF_SPATIAL ? NHMF_CACHE_SPATIAL : 0;
+  double* host = c->work->host;
+  static_assert(3 * kMaxLevels <= kHostSlots, "status words and norms of the levels fit the pinned slots");
   for (int l = nl - 2; l >= 0; --l) {
     GmgLevel& F = G.L[l + 1];
     GmgLevel& C = G.L[l];
@@ -358,8 +366,11 @@ nhmf_status gmg_prepare(nhmf_ctx* c, int strategy, bool fp32, cudaStream_t s, bo
       cudaMemsetAsync(C.x, 0, C.n * sizeof(double), s);  // linear elasticity on the coarse levels
     else
       map3d<double>(F.I, F.ctx->ubar, C.x, F.t1, F.t2, s);
-    if ((st = nhmf_set_linearization(C.ctx, C.x, mask, s)) != NHMF_OK)
+    if ((st = set_linearization_async(C.ctx, C.x, mask, s)) != NHMF_OK)
       return fail(c, st, std::string("gmg: coarse linearisation: ") + nhmf_last_error(C.ctx));
+    host[l] = 0.0;
+    cudaMemcpyAsync(host + l, C.ctx->status, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+    cudaMemsetAsync(C.ctx->status, 0, sizeof(unsigned), s);
   }
   for (int l = 0; l < nl; ++l) {
     GmgLevel& L = G.L[l];
@@ -370,15 +381,26 @@ nhmf_status gmg_prepare(nhmf_ctx* c, int strategy, bool fp32, cudaStream_t s, bo
     reciprocal(L.n, L.diag, L.dinv, L.dinv32, s);
     if (l == 0) continue;  // the coarsest level is solved, not smoothed
     // in the precision of the V-cycle (Algorithm 2 has no FP32 apply)
-    st = (fp32 && strategy != NHMF_SPATIAL) ? power_iteration<float>(c, L, strategy, s)
-                                            : power_iteration<double>(c, L, strategy, s);
+    st = (fp32 && strategy != NHMF_SPATIAL) ? power_iteration<float>(L, strategy, s)
+                                            : power_iteration<double>(L, strategy, s);
     if (st != NHMF_OK) return st;
+    cudaMemcpyAsync(host + kMaxLevels + 2 * l, L.ctx->work->sc + 40, 2 * sizeof(double), cudaMemcpyDeviceToHost, s);
   }
   if (G.coarse.blocks > 0 && (st = coarse_assemble(G, s)) != NHMF_OK) return st;
+  if ((st = cuda_check(c, cudaStreamSynchronize(s), "gmg prepare")) != NHMF_OK) return st;
+  for (int l = nl - 2; l >= 0; --l) {
+    unsigned flags = 0;
+    std::memcpy(&flags, host + l, sizeof(flags));
+    if (flags & kStatusNonPosJ)
+      return fail(c, NHMF_ERR_NONPOS_J, "gmg: coarse linearisation: det F <= 0 at a quadrature point");
+    if (flags & kStatusNonFinite) return fail(c, NHMF_ERR_NONFINITE, "gmg: coarse linearisation: non-finite value");
+  }
+  for (int l = 1; l < nl; ++l) {
+    const double h0 = host[kMaxLevels + 2 * l], h1 = host[kMaxLevels + 2 * l + 1];
+    G.L[l].lmax = (h0 > 0.0 && h1 > 0.0) ? 4.0 * h1 / h0 : 2.0;
+  }
   return cuda_check(c, cudaGetLastError(), "gmg prepare");
 }
-
-
 
 // Chebyshev iteration of `degree` steps on D^-1 A for A x = b, on the interval
 // [lmax/range, lmax] (lmax = 1.2 x the power-iteration estimate); x = 0 on entry if zero_start.
@@ -393,11 +415,6 @@ nhmf_status chebyshev(GmgLevel& L, int strat, const T* b, T* x, int degree, doub
   nhmf_status st = NHMF_OK;
   for (int j = 0; j < degree; ++j) {
     const bool first = j == 0;
-    const T* qq = nullptr;
-    if (!(first && zero_start)) {
-      if ((st = launch_apply(L.ctx, Buf<T>::prec, strat, x, q, s)) != NHMF_OK) return st;
-      qq = q;
-    }
     T c_old, c_new;
     if (first) {
       c_old = T(0);
@@ -408,43 +425,63 @@ nhmf_status chebyshev(GmgLevel& L, int strat, const T* b, T* x, int degree, doub
       c_new = T(2.0 * rho_new / delta);
       rho = rho_new;
     }
-    if (first && !zero_start) {
-      // d = D^-1 (b - A x) / theta, x += d
-      k_cheb<T><<<kB, kT, 0, s>>>(L.n, b, qq, Buf<T>::dinv(L), d, x, T(0), c_new);
+    // d = c_old d + c_new D^-1 (b - A x), x += d, with A x = 0 in the first step from zero
+    if (first && zero_start) {
+      k_cheb<T><<<kB, kT, 0, s>>>(L.n, b, nullptr, Buf<T>::dinv(L), d, x, c_old, c_new);
+    } else if constexpr (sizeof(T) == 4) {
+      Gather32 g;
+      g.mode = Gather32::kChebyshev;
+      g.b = b;
+      g.dinv = Buf<T>::dinv(L);
+      g.d = d;
+      g.c_old = c_old;
+      g.c_new = c_new;
+      if ((st = launch_apply32(L.ctx, strat, x, x, g, s)) != NHMF_OK) return st;
     } else {
-      k_cheb<T><<<kB, kT, 0, s>>>(L.n, b, qq, Buf<T>::dinv(L), d, x, c_old, c_new);
+      if ((st = launch_apply(L.ctx, Buf<T>::prec, strat, x, q, s)) != NHMF_OK) return st;
+      k_cheb<T><<<kB, kT, 0, s>>>(L.n, b, q, Buf<T>::dinv(L), d, x, c_old, c_new);
     }
   }
   return cuda_check(L.ctx, cudaGetLastError(), "chebyshev");
 }
 
-// r_coarse = R r_fine (transpose of the prolongation), fine level `F`
+// r = b - A x on level L
 template <typename T>
-void gmg_restrict(GmgLevel& F, const T* r_fine, T* r_coarse, cudaStream_t s) {
-  map3d<T>(F.R, r_fine, r_coarse, Buf<T>::t1(F), Buf<T>::t2(F), s);
+nhmf_status gmg_residual(GmgLevel& L, int strat, const T* b, const T* x, T* r, cudaStream_t s) {
+  nhmf_status st;
+  if constexpr (sizeof(T) == 4) {
+    Gather32 g;
+    g.mode = Gather32::kResidual;
+    g.b = b;
+    return launch_apply32(L.ctx, strat, x, r, g, s);
+  } else {
+    if ((st = launch_apply(L.ctx, Buf<T>::prec, strat, x, r, s)) != NHMF_OK) return st;
+    k_bminus<T><<<kB, kT, 0, s>>>(L.n, b, r);
+    return cuda_check(L.ctx, cudaGetLastError(), "gmg residual");
+  }
 }
 
-// x_fine += P e_coarse, through the fine level's q buffer
+// r_coarse = R r_fine (transpose of the prolongation), zero on the coarse level's constrained rows
 template <typename T>
-void gmg_prolong_add(GmgLevel& F, const T* e_coarse, T* x_fine, T* scratch, cudaStream_t s) {
-  map3d<T>(F.P, e_coarse, scratch, Buf<T>::t1(F), Buf<T>::t2(F), s);
-  k_add<T><<<kB, kT, 0, s>>>(F.n, scratch, x_fine);
+void gmg_restrict(GmgLevel& F, GmgLevel& C, const T* r_fine, T* r_coarse, cudaStream_t s) {
+  map3d<T>(F.R, r_fine, r_coarse, Buf<T>::t1(F), Buf<T>::t2(F), s, false, C.ctx->prm.bc);
+}
+
+// x_fine += P e_coarse
+template <typename T>
+void gmg_prolong_add(GmgLevel& F, GmgLevel&, const T* e_coarse, T* x_fine, cudaStream_t s) {
+  map3d<T>(F.P, e_coarse, x_fine, Buf<T>::t1(F), Buf<T>::t2(F), s, true);
 }
 
 void gmg_start_vector(long long n, double* v, cudaStream_t s) { k_start<<<kB, kT, 0, s>>>(n, v); }
 
-template <typename T>
-void gmg_bminus(long long n, const T* b, T* y, cudaStream_t s) {
-  k_bminus<T><<<kB, kT, 0, s>>>(n, b, y);
-}
-
 template nhmf_status chebyshev<double>(GmgLevel&, int, const double*, double*, int, double, bool, cudaStream_t);
 template nhmf_status chebyshev<float>(GmgLevel&, int, const float*, float*, int, double, bool, cudaStream_t);
-template void gmg_restrict<double>(GmgLevel&, const double*, double*, cudaStream_t);
-template void gmg_restrict<float>(GmgLevel&, const float*, float*, cudaStream_t);
-template void gmg_prolong_add<double>(GmgLevel&, const double*, double*, double*, cudaStream_t);
-template void gmg_prolong_add<float>(GmgLevel&, const float*, float*, float*, cudaStream_t);
-template void gmg_bminus<double>(long long, const double*, double*, cudaStream_t);
-template void gmg_bminus<float>(long long, const float*, float*, cudaStream_t);
+template nhmf_status gmg_residual<double>(GmgLevel&, int, const double*, const double*, double*, cudaStream_t);
+template nhmf_status gmg_residual<float>(GmgLevel&, int, const float*, const float*, float*, cudaStream_t);
+template void gmg_restrict<double>(GmgLevel&, GmgLevel&, const double*, double*, cudaStream_t);
+template void gmg_restrict<float>(GmgLevel&, GmgLevel&, const float*, float*, cudaStream_t);
+template void gmg_prolong_add<double>(GmgLevel&, GmgLevel&, const double*, double*, cudaStream_t);
+template void gmg_prolong_add<float>(GmgLevel&, GmgLevel&, const float*, float*, cudaStream_t);
 
 }  // namespace nhmf

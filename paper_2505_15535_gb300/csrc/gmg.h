@@ -38,6 +38,8 @@ struct CoarseSolve {
   unsigned long long* words = nullptr;  // device: iterations since zeroed, status flags met
 };
 
+constexpr int kMaxLevels = 13;     // twelve meshes and the p-coarsened one
+
 struct Gmg {
   CoarseSolve coarse;
   std::vector<GmgLevel> L;  // L.back() mirrors the fine context (its ctx pointer is not owned)
@@ -78,9 +80,12 @@ template <> struct Buf<float> {
 template <typename T>
 nhmf_status chebyshev(GmgLevel& L, int strat, const T* b, T* x, int degree, double range, bool zero_start,
                       cudaStream_t s);
-template <typename T> void gmg_restrict(GmgLevel& F, const T* r_fine, T* r_coarse, cudaStream_t s);
-template <typename T> void gmg_prolong_add(GmgLevel& F, const T* e_coarse, T* x_fine, T* scratch, cudaStream_t s);
-template <typename T> void gmg_bminus(long long n, const T* b, T* y, cudaStream_t s);
+template <typename T>
+nhmf_status gmg_residual(GmgLevel& L, int strat, const T* b, const T* x, T* r, cudaStream_t s);
+template <typename T>
+void gmg_restrict(GmgLevel& F, GmgLevel& C, const T* r_fine, T* r_coarse, cudaStream_t s);
+template <typename T>
+void gmg_prolong_add(GmgLevel& F, GmgLevel& C, const T* e_coarse, T* x_fine, cudaStream_t s);
 bool coarse_setup(Gmg& G);
 void coarse_free(Gmg& G);
 // The coarsest operator's matrix at its level's linearisation point.

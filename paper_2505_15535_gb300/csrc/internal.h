@@ -73,6 +73,7 @@ struct Geometry {
 namespace nhmf {
 struct UNet;
 struct Gmg;
+constexpr int kHostSlots = 64;
 // Work vectors of the solvers, allocated on first use.
 struct SolverWork {
   long long n = 0;
@@ -82,7 +83,7 @@ struct SolverWork {
   float *r32 = nullptr, *z32 = nullptr, *p32 = nullptr, *q32 = nullptr, *x32 = nullptr, *b32 = nullptr, *dinv32 = nullptr;
   double* sc = nullptr;        // device scalars
   double* partials = nullptr;  // reduction scratch
-  double* host = nullptr;      // pinned host scalar
+  double* host = nullptr;      // pinned host scalars, kHostSlots of them
   cudaStream_t stream = nullptr;  // the solvers' own stream (graph capture needs a non-legacy stream)
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   // CUDA graphs of `check_every` CG iterations, keyed by the buffers they were captured with
@@ -160,10 +161,21 @@ void unet_smooth_field(nhmf_ctx* c, double* e, unsigned long long seed, cudaStre
 int unet_snapshot_begin(nhmf_ctx* c, const double* r, const double* xj, cudaStream_t s);
 void unet_snapshot_finish(nhmf_ctx* c, int slot, const double* xstar, cudaStream_t s);
 
+// What the FP32 apply's node gather writes from A du: v = A du; v = b - A du; the Chebyshev step
+// d = c_old d + c_new D^-1 (b - A du), v = du + d; or the power-iteration step v = D^-1 A du / 4.
+struct Gather32 {
+  enum Mode { kApply = 0, kResidual = 1, kChebyshev = 2, kPower = 3 };
+  int mode = kApply;
+  const float *b = nullptr, *dinv = nullptr;
+  float* d = nullptr;
+  float c_old = 0.f, c_new = 0.f;
+};
+
 // The operators of one degree (operators.cuh); operators.cu dispatches on the context's degree.
 template <int P>
 struct Operators {
-  static nhmf_status apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw, cudaStream_t s);
+  static nhmf_status apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw,
+                           const Gather32& g32, cudaStream_t s);
   static nhmf_status cache(nhmf_ctx* c, cudaStream_t s);
   static nhmf_status residual(nhmf_ctx* c, const double* u, double* r, cudaStream_t s);
   static nhmf_status diagonal(nhmf_ctx* c, double* d, cudaStream_t s);
@@ -172,6 +184,10 @@ struct Operators {
 // raw = true applies the unconstrained operator K (no Dirichlet masking or identity rows).
 nhmf_status launch_apply(nhmf_ctx* c, int precision, int strategy, const void* du, void* v,
                          cudaStream_t s, bool raw = false);
+// The FP32 apply of du with the gather's update `g32` into v (v == du is allowed but for kApply).
+nhmf_status launch_apply32(nhmf_ctx* c, int strategy, const float* du, float* v, const Gather32& g32, cudaStream_t s);
+// nhmf_set_linearization without reading the status word: the caller does (asynchronous).
+nhmf_status set_linearization_async(nhmf_ctx* c, const double* u, int mask, cudaStream_t s);
 // On every constrained DoF: out = src (mode 0) or out = value (mode 1).
 nhmf_status fix_rows64(nhmf_ctx* c, const double* src, double* out, int mode, double value, cudaStream_t s);
 nhmf_status fix_rows32(nhmf_ctx* c, const float* src, float* out, int mode, float value, cudaStream_t s);

@@ -45,14 +45,25 @@ nhmf_status fix_rows(nhmf_ctx* c, const T* src, T* out, int mode, T value, cudaS
 
 }  // namespace
 
-nhmf_status launch_apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, cudaStream_t s, bool raw) {
+namespace {
+nhmf_status apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw, const Gather32& g32,
+                  cudaStream_t s) {
   switch (c->g.p) {
-    case 1: return Operators<1>::apply(c, prec, strat, du, v, raw, s);
-    case 2: return Operators<2>::apply(c, prec, strat, du, v, raw, s);
-    case 3: return Operators<3>::apply(c, prec, strat, du, v, raw, s);
-    case 4: return Operators<4>::apply(c, prec, strat, du, v, raw, s);
+    case 1: return Operators<1>::apply(c, prec, strat, du, v, raw, g32, s);
+    case 2: return Operators<2>::apply(c, prec, strat, du, v, raw, g32, s);
+    case 3: return Operators<3>::apply(c, prec, strat, du, v, raw, g32, s);
+    case 4: return Operators<4>::apply(c, prec, strat, du, v, raw, g32, s);
   }
   return fail(c, NHMF_ERR_ARG, "degree out of range");
+}
+}  // namespace
+
+nhmf_status launch_apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, cudaStream_t s, bool raw) {
+  return apply(c, prec, strat, du, v, raw, Gather32{}, s);
+}
+
+nhmf_status launch_apply32(nhmf_ctx* c, int strat, const float* du, float* v, const Gather32& g32, cudaStream_t s) {
+  return apply(c, NHMF_FP32, strat, du, v, false, g32, s);
 }
 
 nhmf_status launch_cache_build(nhmf_ctx* c, cudaStream_t s) {

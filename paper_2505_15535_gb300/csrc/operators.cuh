@@ -583,10 +583,13 @@ __global__ void __launch_bounds__(kRegThreads, NHMF_REG_MINB) k_apply_reg(const 
 // v[c][node] = sum of vloc(e; c, q) over the elements e whose closure holds the node (1, 2, 4
 // or 8 of them; q the node's local index in e), always in increasing (ez, ey, ex) order, so
 // the result is bitwise deterministic without atomics.  Dirichlet rows (unless raw):
-// v = du there.  One thread per node.
-template <int P>
-__global__ void __launch_bounds__(256) k_gather_local(const float* __restrict__ vloc, const float* __restrict__ du,
-                                                     float* __restrict__ v, int N, int M, int bc) {
+// v = du there.  One thread per node.  The multigrid's vector updates ride on the gather (see
+// Gather32): a node's result is final here, so b - A x, a Chebyshev step or a power-iteration
+// step costs no further pass over A x and no launch.  v may be du in those forms: every thread
+// reads and writes its own node only.
+template <int P, int MODE>
+__global__ void __launch_bounds__(256) k_gather_local(const float* __restrict__ vloc, const float* du, float* v, int N,
+                                                     int M, int bc, const Gather32 g32) {
   constexpr int n = P + 1, n3 = n * n * n;
   static_assert(kTile == 32, "tile index by shift and mask");
   // grid: x covers the M^2 nodes of one z-plane, y the plane (32-bit index arithmetic; the
@@ -643,8 +646,20 @@ __global__ void __launch_bounds__(256) k_gather_local(const float* __restrict__ 
 #pragma unroll
         for (int x = 0; x < 2; ++x)
           if (has[2][z] && has[1][y] && has[0][x]) s += val[c][4 * z + 2 * y + x];
-    if (is_constrained(bc, c, g[0], g[2], M)) s = du[c * M3 + node];
-    v[c * M3 + node] = s;
+    const long long i = c * M3 + node;
+    if (is_constrained(bc, c, g[0], g[2], M)) s = du[i];
+    if constexpr (MODE == Gather32::kApply) {
+      v[i] = s;
+    } else if constexpr (MODE == Gather32::kResidual) {
+      v[i] = g32.b[i] - s;
+    } else if constexpr (MODE == Gather32::kChebyshev) {
+      const float t = g32.c_new * g32.dinv[i] * (g32.b[i] - s);
+      const float di = g32.c_old == 0.f ? t : fmaf(g32.c_old, g32.d[i], t);
+      g32.d[i] = di;
+      v[i] = du[i] + di;
+    } else {
+      v[i] = 0.25f * g32.dinv[i] * s;
+    }
   }
 }
 
@@ -1054,10 +1069,11 @@ nhmf_status run_colours(nhmf_ctx* c, KernelT kernel, OpArgs a, int NE, int threa
 }
 
 // The element-local FP32 apply: `kernel` once over the class of all elements (NE per block),
-// writing c->vloc, then k_gather_local<P> onto v with the Dirichlet rows (bc of `a`).
+// writing c->vloc, then k_gather_local<P> onto v with the Dirichlet rows (bc of `a`) and the
+// update `g32`.
 template <int P, typename KernelT>
 nhmf_status run_local(nhmf_ctx* c, KernelT kernel, OpArgs a, int NE, int threads, size_t smem, const float* du,
-                      float* v, cudaStream_t s) {
+                      float* v, const Gather32& g32, cudaStream_t s) {
   if (cudaError_t e = prepare(kernel, smem); e != cudaSuccess) return cuda_check(c, e, "apply");
   if (!c->vloc) return fail(c, NHMF_ERR_STATE, "apply: no element-local buffer (set_linearization first)");
   if (c->g.E > 0x7fffffffLL || (long long)c->g.M * c->g.M > 0x7fffffffLL)
@@ -1072,7 +1088,11 @@ nhmf_status run_local(nhmf_ctx* c, KernelT kernel, OpArgs a, int NE, int threads
   a.vloc = c->vloc;
   kernel<<<(unsigned)((c->g.E + NE - 1) / NE), threads, smem, s>>>(a);
   const dim3 gather_grid((unsigned)(((long long)c->g.M * c->g.M + 255) / 256), (unsigned)c->g.M);
-  k_gather_local<P><<<gather_grid, 256, 0, s>>>(c->vloc, du, v, c->g.N, c->g.M, a.bc);
+  auto* gather = g32.mode == Gather32::kApply       ? k_gather_local<P, Gather32::kApply>
+                 : g32.mode == Gather32::kResidual  ? k_gather_local<P, Gather32::kResidual>
+                 : g32.mode == Gather32::kChebyshev ? k_gather_local<P, Gather32::kChebyshev>
+                                                    : k_gather_local<P, Gather32::kPower>;
+  gather<<<gather_grid, 256, 0, s>>>(c->vloc, du, v, c->g.N, c->g.M, a.bc, g32);
   if (c->profiling) {
     cudaEventRecord(rec.b, s);
     c->prof.push_back(rec);
@@ -1098,7 +1118,7 @@ nhmf_status apply_colours(nhmf_ctx* c, const OpArgs& a, size_t slots_per_item, c
 }
 
 template <int P, typename T, int STRAT>
-nhmf_status apply_p(nhmf_ctx* c, const void* du, void* v, bool raw, cudaStream_t s) {
+nhmf_status apply_p(nhmf_ctx* c, const void* du, void* v, bool raw, const Gather32& g32, cudaStream_t s) {
   OpArgs a = base_args(c);
   if (raw) a.bc = NHMF_BC_NONE;  // unconstrained operator K: no masking, no identity rows
   a.u64 = c->u_at ? c->u_at : c->ubar;
@@ -1124,15 +1144,15 @@ nhmf_status apply_p(nhmf_ctx* c, const void* du, void* v, bool raw, cudaStream_t
         constexpr size_t n3 = (P + 1) * (P + 1) * (P + 1), n2 = (P + 1) * (P + 1);
         const size_t kin_smem = (3 * n3 + 10 * n2) * kRegThreads * sizeof(float);
         if (split)
-          return run_local<P>(c, k_apply_reg<P, STRAT, SPLIT>, a, kRegThreads, kRegThreads, 0, du32, v32, s);
+          return run_local<P>(c, k_apply_reg<P, STRAT, SPLIT>, a, kRegThreads, kRegThreads, 0, du32, v32, g32, s);
         return run_local<P>(c, k_apply_reg<P, STRAT, NHMF_MODEL_COMPRESSIBLE>, a, kRegThreads, kRegThreads,
-                            STRAT == NHMF_ON_THE_FLY ? kin_smem : 0, du32, v32, s);
+                            STRAT == NHMF_ON_THE_FLY ? kin_smem : 0, du32, v32, g32, s);
       }
     }
     using Sh = Shape<P, T, STRAT, false>;
     const size_t smem = (kTabSlots + per_item * Sh::NE * (P + 1) * (P + 1) * (P + 1)) * sizeof(T);
     auto* k = split ? k_apply<P, T, STRAT, SPLIT, false> : k_apply<P, T, STRAT, NHMF_MODEL_COMPRESSIBLE, false>;
-    return run_local<P>(c, k, a, Sh::NE, Sh::THREADS, smem, du32, v32, s);
+    return run_local<P>(c, k, a, Sh::NE, Sh::THREADS, smem, du32, v32, g32, s);
   } else {
     if (small_blocks<T, Shape<P, T, STRAT, false>::NE>(c))
       return split ? apply_colours<P, T, STRAT, SPLIT, true>(c, a, per_item, s)
@@ -1143,18 +1163,19 @@ nhmf_status apply_p(nhmf_ctx* c, const void* du, void* v, bool raw, cudaStream_t
 }
 
 template <int P>
-nhmf_status apply_dispatch_p(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw, cudaStream_t s) {
+nhmf_status apply_dispatch_p(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw,
+                             const Gather32& g32, cudaStream_t s) {
   if (prec == NHMF_DF64) {
     if (strat != NHMF_CACHED) return fail(c, NHMF_ERR_ARG, "df64 apply: cached strategy only");
-    return apply_p<P, df64, NHMF_CACHED>(c, du, v, raw, s);
+    return apply_p<P, df64, NHMF_CACHED>(c, du, v, raw, g32, s);
   }
   if (prec == NHMF_FP64) {
-    if (strat == NHMF_SPATIAL) return apply_p<P, double, NHMF_SPATIAL>(c, du, v, raw, s);
-    return strat == NHMF_CACHED ? apply_p<P, double, NHMF_CACHED>(c, du, v, raw, s)
-                                : apply_p<P, double, NHMF_ON_THE_FLY>(c, du, v, raw, s);
+    if (strat == NHMF_SPATIAL) return apply_p<P, double, NHMF_SPATIAL>(c, du, v, raw, g32, s);
+    return strat == NHMF_CACHED ? apply_p<P, double, NHMF_CACHED>(c, du, v, raw, g32, s)
+                                : apply_p<P, double, NHMF_ON_THE_FLY>(c, du, v, raw, g32, s);
   }
-  return strat == NHMF_CACHED ? apply_p<P, float, NHMF_CACHED>(c, du, v, raw, s)
-                              : apply_p<P, float, NHMF_ON_THE_FLY>(c, du, v, raw, s);
+  return strat == NHMF_CACHED ? apply_p<P, float, NHMF_CACHED>(c, du, v, raw, g32, s)
+                              : apply_p<P, float, NHMF_ON_THE_FLY>(c, du, v, raw, g32, s);
 }
 
 template <int P, bool SMALL>
@@ -1217,8 +1238,9 @@ nhmf_status diagonal_p(nhmf_ctx* c, double* d, cudaStream_t s) {
 }  // namespace
 
 template <int P>
-nhmf_status Operators<P>::apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw, cudaStream_t s) {
-  return apply_dispatch_p<P>(c, prec, strat, du, v, raw, s);
+nhmf_status Operators<P>::apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw,
+                                const Gather32& g32, cudaStream_t s) {
+  return apply_dispatch_p<P>(c, prec, strat, du, v, raw, g32, s);
 }
 template <int P>
 nhmf_status Operators<P>::cache(nhmf_ctx* c, cudaStream_t s) {

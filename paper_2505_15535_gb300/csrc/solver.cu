@@ -43,7 +43,8 @@ __global__ void k_bc(int bc, int M, long long M3, double top_uz, double* u, doub
 }
 
 enum Slot { CT = 24, CAC = 25, OMEGA = 26, CNORM = 27,  // the learned correction's step length
-            RZ0 = 0, RZ1 = 1, PQ = 2, RR = 3, BN = 4, ALPHA = 5, BETA = 6, ZQ = 7, PR = 8, PQPREV = 9,
+            RZ0 = 0, RZ1 = 1, PQ = 2, RR = 3, BN = 4, ALPHA = 5, BETA = 6, ZQ = 7,
+            FPQ = 9,  // fcg's p.q (a one-level hierarchy's coarse pcg() uses slots 0..4 of the same context)
             RNORM = 10, TMP = 11, IN_RZ0 = 16, IN_RZ1 = 17, IN_PQ = 18, IN_RR = 19, IN_BN = 20 };
 
 struct Ctx {
@@ -72,7 +73,8 @@ nhmf_status ensure_work(nhmf_ctx* c) {
     if (cudaMalloc(p, n * sizeof(float)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "solver work alloc");
   if (cudaMalloc(&w.sc, 64 * sizeof(double)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "solver scalars");
   if (cudaMalloc(&w.partials, kPartialSlots * sizeof(double)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "partials");
-  if (cudaMallocHost(&w.host, 8 * sizeof(double)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "pinned scalar");
+  cudaMemset(w.partials, 0, kPartialSlots * sizeof(double));
+  if (cudaMallocHost(&w.host, kHostSlots * sizeof(double)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "pinned scalar");
   cudaMemset(w.sc, 0, 64 * sizeof(double));
   if (cudaStreamCreateWithFlags(&w.stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&w.ev_in, cudaEventDisableTiming) != cudaSuccess ||
@@ -237,7 +239,7 @@ nhmf_status fcg(Ctx& x, int strat, const double* b, double* sol, double rtol, in
   SolverWork& w = x.w;
   double* sc = w.sc;
   double bnh;
-  nhmf_status st = norm(x, b, BN, &bnh);
+  nhmf_status st = norm(x, b, RNORM, &bnh);  // RNORM holds ||r|| throughout
   if (st != NHMF_OK) return st;
   cudaMemsetAsync(sol, 0, x.n * sizeof(double), x.s);
   *iters = 0;
@@ -255,31 +257,26 @@ nhmf_status fcg(Ctx& x, int strat, const double* b, double* sol, double rtol, in
     if (k == 0) {
       cudaMemcpyAsync(w.p, w.z, x.n * sizeof(double), cudaMemcpyDeviceToDevice, x.s);
     } else {
-      dot(x.n, w.z, qprev, sc + ZQ, w.partials, x.s);
-      ratio(sc + ZQ, sc + PQPREV, -1.0, sc + BETA, x.s);
+      // beta = -(z . q_prev) / (p_prev . q_prev); FPQ still holds the previous p . q
+      dot_ratio(x.n, w.z, qprev, sc + ZQ, sc + FPQ, -1.0, sc + BETA, w.partials, x.s);
       axpby(x.n, 1.0, nullptr, w.z, 1.0, sc + BETA, w.p, x.s);
     }
     if ((st = launch_apply(c, x.outer, strat, w.p, q, x.s)) != NHMF_OK) return st;
-    dot(x.n, w.p, q, sc + PQ, w.partials, x.s);
-    dot(x.n, w.p, w.r, sc + PR, w.partials, x.s);
-    ratio(sc + PR, sc + PQ, 1.0, sc + ALPHA, x.s);
-    axpby(x.n, 1.0, sc + ALPHA, w.p, 1.0, nullptr, sol, x.s);
-    axpby(x.n, -1.0, sc + ALPHA, q, 1.0, nullptr, w.r, x.s);
-    cudaMemcpyAsync(sc + PQPREV, sc + PQ, sizeof(double), cudaMemcpyDeviceToDevice, x.s);
+    fcg_alpha(x.n, w.p, q, w.r, sc + FPQ, sc + ALPHA, w.partials, x.s);
+    fcg_update(x.n, sc + ALPHA, w.p, q, sol, w.r, sc + RNORM, w.partials, x.s);
     std::swap(q, qprev);
     ++k;
-    double pqh;
-    w.host[2] = 0.0;
-    if (words) cudaMemcpyAsync(w.host + 1, words, 2 * sizeof(double), cudaMemcpyDeviceToHost, x.s);
-    if ((st = read_scalar(x, sc + PQ, &pqh)) != NHMF_OK) return st;
-    if (words) {
-      unsigned long long flags;
-      std::memcpy(&flags, w.host + 2, sizeof(flags));
-      if (flags & kStatusNonFinite) return fail(c, NHMF_ERR_NONFINITE, "multigrid coarse solve: non-finite residual");
-      if (flags & kStatusBreakdown) return fail(c, NHMF_ERR_BREAKDOWN, "multigrid coarse solve: p^T A p <= 0");
-    }
-    if (!(pqh > 0.0)) return fail(c, NHMF_ERR_BREAKDOWN, "fcg: p^T A p <= 0");
-    if ((st = norm(x, w.r, RNORM, &rn)) != NHMF_OK) return st;
+    // p . q, ||r|| and the coarse solves' flags in one read
+    unsigned long long flags = 0;
+    if (words) cudaMemcpyAsync(w.host + 16, words, 2 * sizeof(double), cudaMemcpyDeviceToHost, x.s);
+    st = cuda_check(c, cudaMemcpyAsync(w.host, sc, 16 * sizeof(double), cudaMemcpyDeviceToHost, x.s), "fcg read");
+    if (st == NHMF_OK) st = cuda_check(c, cudaStreamSynchronize(x.s), "fcg sync");
+    if (st != NHMF_OK) return st;
+    if (words) std::memcpy(&flags, w.host + 17, sizeof(flags));
+    if (flags & kStatusNonFinite) return fail(c, NHMF_ERR_NONFINITE, "multigrid coarse solve: non-finite residual");
+    if (flags & kStatusBreakdown) return fail(c, NHMF_ERR_BREAKDOWN, "multigrid coarse solve: p^T A p <= 0");
+    if (!(w.host[FPQ] > 0.0)) return fail(c, NHMF_ERR_BREAKDOWN, "fcg: p^T A p <= 0");
+    rn = w.host[RNORM];
     if (!std::isfinite(rn)) return fail(c, NHMF_ERR_NONFINITE, "fcg: non-finite residual");
     hist.push_back(rn);
     if (rn <= rtol * bnh) break;
@@ -460,16 +457,10 @@ nhmf_status vcycle(nhmf_ctx* c, int l, const nhmf_solve_opts& o, const T* b, T* 
   const int deg = o.smoother_degree > 0 ? o.smoother_degree : 3;
   const double range = o.smoother_range > 1.0 ? o.smoother_range : 15.0;
   if ((st = chebyshev<T>(L, strat, b, x, deg, range, true, s)) != NHMF_OK) return st;
-  if ((st = launch_apply(L.ctx, Buf<T>::prec, strat, x, Buf<T>::r(L), s)) != NHMF_OK) return st;
-  gmg_bminus<T>(L.n, b, Buf<T>::r(L), s);
-  gmg_restrict<T>(L, Buf<T>::r(L), Buf<T>::b(C), s);
-  if (fp32)
-    st = fix_rows32(C.ctx, nullptr, reinterpret_cast<float*>(Buf<T>::b(C)), 1, 0.f, s);
-  else
-    st = fix_rows64(C.ctx, nullptr, reinterpret_cast<double*>(Buf<T>::b(C)), 1, 0.0, s);
-  if (st != NHMF_OK) return st;
+  if ((st = gmg_residual<T>(L, strat, b, x, Buf<T>::r(L), s)) != NHMF_OK) return st;
+  gmg_restrict<T>(L, C, Buf<T>::r(L), Buf<T>::b(C), s);  // zero on C's constrained rows
   if ((st = vcycle<T>(c, l - 1, o, Buf<T>::b(C), Buf<T>::x(C), s, coarse_iters)) != NHMF_OK) return st;
-  gmg_prolong_add<T>(L, Buf<T>::x(C), x, Buf<T>::q(L), s);
+  gmg_prolong_add<T>(L, C, Buf<T>::x(C), x, s);
   return chebyshev<T>(L, strat, b, x, deg, range, false, s);
 }
 
@@ -600,17 +591,17 @@ nhmf_status linear(Ctx& x, const nhmf_solve_opts& o, const double* b, double* so
     auto precond = [&](const double* r, double* z) -> nhmf_status {
       if (stall) return zero(z);
       if (!f32) return vcycle<double>(x.c, ltop, o, r, z, x.s, inner);
-      norm2(x.n, r, w.sc + TMP, w.partials, x.s);
-      to_fp32_scaled(x.n, r, w.sc + TMP, true, top.b32, x.s);
+      // fcg keeps ||r|| in RNORM: the FP32 cycle runs on r / ||r||
+      to_fp32_scaled(x.n, r, w.sc + RNORM, true, top.b32, x.s);
       nhmf_status s2 = vcycle<float>(x.c, ltop, o, top.b32, top.x32, x.s, inner);
       if (s2 != NHMF_OK) return s2;
-      to_fp64_scaled(x.n, top.x32, w.sc + TMP, z, x.s);
+      to_fp64_scaled(x.n, top.x32, w.sc + RNORM, z, x.s);
       const bool rec_now = record && un->npairs < un->cap && jprec < rec_iters;
       ++jprec;
       if (learned || rec_now) {
         // residual the V-cycle leaves, t = r - A z, from an FP32 apply to its FP32 output
         if ((s2 = launch_apply(x.c, NHMF_FP32, strat32, top.x32, top.r32, x.s)) != NHMF_OK) return s2;
-        to_fp64_scaled(x.n, top.r32, w.sc + TMP, w.t, x.s);
+        to_fp64_scaled(x.n, top.r32, w.sc + RNORM, w.t, x.s);
         axpby(x.n, 1.0, nullptr, r, -1.0, nullptr, w.t, x.s);
         if (rec_now) {
           // pair (t, x* - (x_j + z)): the error left after the V-cycle, A (x* - x_j - z) = t
