@@ -41,8 +41,9 @@ __device__ __forceinline__ void load_tables(const OpArgs& a, T* sB, T* sDc, T* s
 
 // The apply's tables: B and Dc (forward), BW and DcW (transposed, carrying w, mu, h), Dch and
 // the even-odd coefficient sets, laid out as in k_apply.
+// `deriv`: the even-odd set in the place of Dc's (the residual takes physical gradients), or null.
 template <int P, typename T>
-__device__ __forceinline__ void load_apply_tables(const OpArgs& a, T* tab) {
+__device__ __forceinline__ void load_apply_tables(const OpArgs& a, T* tab, const double* deriv = nullptr) {
   constexpr int n = P + 1, S = kMaxN * kMaxN;
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
     tab[i] = T(a.B[i]);
@@ -52,7 +53,7 @@ __device__ __forceinline__ void load_apply_tables(const OpArgs& a, T* tab) {
     tab[4 * S + i] = T(a.Dch[i]);
   }
   for (int i = threadIdx.x; i < 4 * kEoSlots; i += blockDim.x)
-    tab[5 * S + i] = T(a.eo[i / kEoSlots][i % kEoSlots]);
+    tab[5 * S + i] = T(deriv && i / kEoSlots == 1 ? deriv[i % kEoSlots] : a.eo[i / kEoSlots][i % kEoSlots]);
 }
 
 // Gather three components of a global vector into dst[c][t] for the block's elements,
@@ -88,10 +89,10 @@ __device__ __forceinline__ float to_store(float x) { return x; }
 __device__ __forceinline__ double to_store(df64 x) { return to_double(x); }
 
 // Adds the block's element results to `out` once the launches before this one are complete
-// (rows of constrained DoFs keep what k_init_rows wrote).
+// (rows of constrained DoFs keep what k_init_rows wrote), scaled by a per-element factor fac[e].
 template <int P, int NI, typename T>
 __device__ __forceinline__ void scatter_add(const OpArgs& a, const T* src, long long e0, int nvalid,
-                                            typename Store<T>::type* __restrict__ out) {
+                                            typename Store<T>::type* __restrict__ out, const T* fac = nullptr) {
   constexpr int n3 = (P + 1) * (P + 1) * (P + 1);
   pdl_wait();
   for (int t = threadIdx.x; t < NI; t += blockDim.x) {
@@ -102,7 +103,8 @@ __device__ __forceinline__ void scatter_add(const OpArgs& a, const T* src, long 
     const long long node = gi + (long long)a.M * (gj + (long long)a.M * gk);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-      if (!is_constrained(a.bc, c, gi, gk, a.M)) out[c * a.M3 + node] += to_store(src[c * NI + t]);
+      if (!is_constrained(a.bc, c, gi, gk, a.M))
+        out[c * a.M3 + node] += to_store(fac ? src[c * NI + t] * fac[e] : src[c * NI + t]);
   }
 }
 
@@ -148,15 +150,31 @@ __device__ __forceinline__ void from_points(const T* sB, const T* sDc, T* G, T* 
   __syncthreads();
 }
 
+// The transposed passes of the apply and the residual: fluxes G[3c+d] with the weighted tables BW,
+// DcW (kBW: even-odd coefficients of BW^T) to nodal values in G[3..5].
+template <int n, int NI, int TH, bool EO, typename T, typename MAP = NoLineMap>
+__device__ __forceinline__ void transposed(const T* sBW, const T* sDcW, const T* kBW, T* G, T* Vq, int nitems,
+                                           int nlines, const MAP& lm = MAP()) {
+  if constexpr (EO) {
+    colloc_grad_T<n, NI>(sDcW, G, Vq, nitems);
+    __syncthreads();
+    eo_pass<n, NI, 3, 0, false, kEoCentreCol, TH>(kBW, Vq, G, nlines, lm);
+    __syncthreads();
+    eo_pass<n, NI, 3, 1, false, kEoCentreCol, TH>(kBW, G, Vq, nlines, lm);
+    __syncthreads();
+    eo_pass<n, NI, 3, 2, false, kEoCentreCol, TH>(kBW, Vq, G + 3 * NI, nlines, lm);
+    __syncthreads();
+  } else {
+    from_points<n, NI>(sBW, sDcW, G, Vq, G + 3 * NI, nitems);
+  }
+}
+
 // ------------------------------------------------------------------ tangent application
 // The quadrature weight, mu and h ride on the transposed tables (BW, DcW) and the element's
 // material factor on the gathered du (the operator is linear in du), so the point code returns
 // dP / mu without any scaling.  For odd n (Q2, Q4) every non-accumulating pass (forward B,
 // forward collocation derivative, transposed B) runs one thread per line in even-odd form, and
 // the gradient of du reaches the point code through shared memory.
-#ifndef NHMF_EO_GRADT
-#define NHMF_EO_GRADT 1
-#endif
 #ifndef NHMF_LINEMAP
 #define NHMF_LINEMAP 1
 #endif
@@ -266,15 +284,24 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
       for (int k = 0; k < 9; ++k) G[k * NI + t] = g[k];
       continue;
     }
-    T Fi[9], lnJ, Jm1 = T(0), F[9];
     if constexpr (STRAT == NHMF_ON_THE_FLY) {
       T H[9];
       colloc_grad<n, NI>(sDch, U, t, H);  // physical gradient: Dch = Dc / h
-      Jm1 = kinematics(H, Fi, lnJ);
-      bad |= !(Jm1 > T(-1));
+      const Kinematics<T> kin(H);
+      bad |= !(kin.Jm1 > T(-1));
+      if constexpr (MODEL == NHMF_MODEL_SPLIT) {
+        T F[9], Fi[9];
 #pragma unroll
-      for (int k = 0; k < 9; ++k) F[k] = (k % 4 == 0 ? T(1) : T(0)) + H[k];
+        for (int k = 0; k < 9; ++k) {
+          F[k] = (k % 4 == 0 ? T(1) : T(0)) + H[k];
+          Fi[k] = kin.A[k] * kin.invJ;
+        }
+        split_stress_dP(F, Fi, kin.lnJ, kin.Jm1, dH, T(a.mu), T(a.lam), inv_mu, g);
+      } else {
+        linearised_stress_unit(kin, dH, r2, g);
+      }
     } else {
+      T Fi[9], lnJ;
       if (t / n3 < nvalid) {
         if constexpr (std::is_same<T, df64>::value) {
           const float2* cdf = static_cast<const float2*>(a.cache);
@@ -303,27 +330,20 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
         for (int k = 0; k < 9; ++k) Fi[k] = (k % 4 == 0) ? T(1) : T(0);
         lnJ = T(0);
       }
-    }
-    if constexpr (STRAT == NHMF_ON_THE_FLY && MODEL == NHMF_MODEL_SPLIT)
-      split_stress_dP(F, Fi, lnJ, Jm1, dH, T(a.mu), T(a.lam), inv_mu, g);
-    else
       linearised_stress_unit(Fi, lnJ, dH, r2, g);
+    }
 #pragma unroll
     for (int k = 0; k < 9; ++k) G[k * NI + t] = g[k];
   }
   if (bad) atomicOr(a.status, kStatusNonPosJ);
   __syncthreads();
-  if constexpr (EO) {
-    if constexpr (std::is_same<T, float>::value && NHMF_EO_GRADT) {
-      // FP32: the transposed derivative as three even-odd line passes, Vq[c] = sum_d DcW^T_d G[3c+d]
-      eo_pass<n, NI, 3, 0, true, kEoGeneral, TH, 1, 0, 3, 0, false>(kDcWT, G, Vq, nlines, lm);
-      __syncthreads();
-      eo_pass<n, NI, 3, 1, true, kEoGeneral, TH, 1, 0, 3, 1, true>(kDcWT, G, Vq, nlines, lm);
-      __syncthreads();
-      eo_pass<n, NI, 3, 2, true, kEoGeneral, TH, 1, 0, 3, 2, true>(kDcWT, G, Vq, nlines, lm);
-    } else {
-      colloc_grad_T<n, NI>(sDcW, G, Vq, nitems);
-    }
+  if constexpr (EO && std::is_same<T, float>::value) {
+    // FP32: the transposed derivative as three even-odd line passes, Vq[c] = sum_d DcW^T_d G[3c+d]
+    eo_pass<n, NI, 3, 0, true, kEoGeneral, TH, 1, 0, 3, 0, false>(kDcWT, G, Vq, nlines, lm);
+    __syncthreads();
+    eo_pass<n, NI, 3, 1, true, kEoGeneral, TH, 1, 0, 3, 1, true>(kDcWT, G, Vq, nlines, lm);
+    __syncthreads();
+    eo_pass<n, NI, 3, 2, true, kEoGeneral, TH, 1, 0, 3, 2, true>(kDcWT, G, Vq, nlines, lm);
     __syncthreads();
     eo_pass<n, NI, 3, 0, false, kEoCentreCol, TH>(kBW, Vq, G, nlines, lm);
     __syncthreads();
@@ -332,7 +352,7 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
     eo_pass<n, NI, 3, 2, false, kEoCentreCol, TH>(kBW, Vq, G + 3 * NI, nlines, lm);
     __syncthreads();
   } else {
-    from_points<n, NI>(sBW, sDcW, G, Vq, G + 3 * NI, nitems);
+    transposed<n, NI, TH, EO>(sBW, sDcW, kBW, G, Vq, nitems, nlines, lm);
   }
   if constexpr (std::is_same<T, float>::value) {
     if (a.vloc) {
@@ -677,19 +697,18 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
   T* Vq = A + 3 * NI;     // [3][NI]
   pdl_launch_next();
   load_tables<P>(a, sB, sDc, sD, sW, 1.0);
+  __syncthreads();
+  for (int i = threadIdx.x; i < n * n; i += blockDim.x) sDc[i] = a.Dch[i];  // physical gradients
   const long long e0 = (long long)blockIdx.x * NE;
   const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
   gather<P, NI>(a, a.u64, e0, nvalid, false, A);
   __syncthreads();
   to_points<n, NI>(sB, A, Vq, Vq, nvalid * n3);
-  const double invh = 1.0 / a.h;
   const long long cbase = (a.col.slot0 + e0) * n3;
   bool bad = false;
   for (int t = threadIdx.x; t < nvalid * n3; t += blockDim.x) {
     double H[9], Fi[9], lnJ;
     colloc_grad<n, NI>(sDc, Vq, t, H);
-#pragma unroll
-    for (int k = 0; k < 9; ++k) H[k] *= invh;
     const double Jm1 = kinematics(H, Fi, lnJ);
     bad |= !(Jm1 > -1.0);
     if (a.cache64_out) {
@@ -765,154 +784,249 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
 }
 
 // ------------------------------------------------------------------ residual
+// The passes of the on-the-fly apply with P(F) / mu in place of dP / mu: the weights, mu and h ride
+// on the transposed tables, the other h of the integral and the material factor on the scatter.  FP64 operations per point
+// bound it: with the kinematics above, P from the adjugate (P / mu = F + c A^T) and the even-odd
+// passes of odd n, Q3 48^3 takes 320 -> 165 of them.
 template <int P, bool SMALL>
 __global__ void __launch_bounds__(Shape<P, double, 0, SMALL>::THREADS) k_residual(const OpArgs a) {
   using T = double;
   constexpr int n = P + 1, n3 = n * n * n, NE = Shape<P, T, 0, SMALL>::NE, NI = NE * n3;
+  constexpr int S = kMaxN * kMaxN, TH = Shape<P, T, 0, SMALL>::THREADS;
+  constexpr bool EO = n % 2 == 1;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* sB = reinterpret_cast<T*>(smem_raw);
-  T* sDc = sB + kMaxN * kMaxN;
-  T* sD = sDc + kMaxN * kMaxN;
-  T* sW = sD + kMaxN * kMaxN;
-  T* Vq = sB + kTabSlots;  // [3][NI]
-  T* G = Vq + 3 * NI;      // [9][NI]
+  T* tab = reinterpret_cast<T*>(smem_raw);
+  const T *kB = tab + 5 * S, *kDch = kB + kEoSlots, *kBW = kDch + kEoSlots;
+  T* sF = tab + 5 * S + 4 * kEoSlots;  // [NE] h times the material factors
+  T* Vq = tab + kTabSlots;             // [3][NI] u at the points
+  T* G = Vq + 3 * NI;                  // [9][NI] gradients, then fluxes
   pdl_launch_next();
-  load_tables<P>(a, sB, sDc, sD, sW, a.h * a.h);
+  load_apply_tables<P>(a, tab, a.eoh);
   const long long e0 = (long long)blockIdx.x * NE;
   const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
+  const int nitems = nvalid * n3, nlines = nvalid * n * n;
+  for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = a.h * elem_factor(a, e0 + min(e, nvalid - 1));
   gather<P, NI>(a, a.u64, e0, nvalid, false, G);
   __syncthreads();
-  const int nitems = nvalid * n3;
-  to_points<n, NI>(sB, G, Vq, Vq, nitems);
-  const double invh = 1.0 / a.h;
+  if constexpr (EO) {
+    eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, G, Vq, nlines);
+    __syncthreads();
+    eo_pass<n, NI, 3, 1, false, kEoCentreRow, TH>(kB, Vq, G, nlines);
+    __syncthreads();
+    eo_pass<n, NI, 3, 2, false, kEoCentreRow, TH>(kB, G, Vq, nlines);
+    __syncthreads();
+    eo_pass<n, NI, 3, 0, true, kEoGeneral, TH, 3, 0>(kDch, Vq, G, nlines);
+    eo_pass<n, NI, 3, 1, true, kEoGeneral, TH, 3, 1>(kDch, Vq, G, nlines);
+    eo_pass<n, NI, 3, 2, true, kEoGeneral, TH, 3, 2>(kDch, Vq, G, nlines);
+    __syncthreads();
+  } else {
+    to_points<n, NI>(tab, G, Vq, Vq, nitems);
+  }
+  const T r2 = a.r2mu, inv_mu = 1.0 / a.mu;
   unsigned flags = 0;
   for (int t = threadIdx.x; t < nitems; t += blockDim.x) {
-    double H[9], Fi[9], lnJ;
-    colloc_grad<n, NI>(sDc, Vq, t, H);
+    T H[9], g[9];
+    if constexpr (EO) {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) H[k] *= invh;
-    const double Jm1 = kinematics(H, Fi, lnJ);
+      for (int k = 0; k < 9; ++k) H[k] = G[k * NI + t];
+    } else {
+      colloc_grad<n, NI>(tab + 4 * S, Vq, t, H);
+    }
+    const Kinematics<T> kin(H);
     // a NaN deformation gradient is a non-finite input; det F <= 0 makes P non-finite too,
     // but is reported as what it is (the Newton backtracking acts on it)
-    const bool inverted = Jm1 <= -1.0;
+    const bool inverted = kin.Jm1 <= -1.0;
     if (inverted) flags |= kStatusNonPosJ;
-    const double s = sW[t % n3] * elem_factor(a, e0 + min(t / n3, nvalid - 1));
-    double F[9], P[9];
+    if (a.model == NHMF_MODEL_SPLIT) {
+      T F[9], Fi[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) F[k] = (k % 4 == 0 ? 1.0 : 0.0) + H[k];
-    model_piola(a.model, F, Fi, lnJ, Jm1, a.mu, a.lam, P);
+      for (int k = 0; k < 9; ++k) {
+        F[k] = (k % 4 == 0 ? 1.0 : 0.0) + H[k];
+        Fi[k] = kin.A[k] * kin.invJ;
+      }
+      model_piola(a.model, F, Fi, kin.lnJ, kin.Jm1, a.mu, a.lam, g);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) g[k] *= inv_mu;
+    } else {
+      const T c = fma(r2, kin.lnJ, -1.0) * kin.invJ;
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          g[3 * i + j] = fma(c, kin.A[3 * j + i], i == j ? 1.0 + H[3 * i + j] : H[3 * i + j]);
+    }
+    bool finite = true;  // by the exponent bits: the FP64 pipe is the busy unit
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-      if (!inverted && !isfinite(P[k])) flags |= kStatusNonFinite;
-      G[k * NI + t] = s * P[k];
+      finite &= (__double2hiint(g[k]) & 0x7ff00000) != 0x7ff00000;
+      G[k * NI + t] = g[k];
     }
+    if (!inverted && !finite) flags |= kStatusNonFinite;
   }
   if (flags) atomicOr(a.status, flags);
   __syncthreads();
-  from_points<n, NI>(sB, sDc, G, Vq, G + 3 * NI, nitems);
-  scatter_add<P, NI>(a, G + 3 * NI, e0, nvalid, static_cast<double*>(a.v));
+  transposed<n, NI, TH, EO>(tab + 2 * S, tab + 3 * S, kBW, G, Vq, nitems, nlines);
+  scatter_add<P, NI>(a, G + 3 * NI, e0, nvalid, static_cast<double*>(a.v), (const T*)sF);
 }
 
 // ------------------------------------------------------------------ diagonal
 // diag(K)_{c,I} = sum_q sum_{d,l} L_{cdcl} dphi_I/dX_d dphi_I/dX_l w_q h^3 with
-// L_{cdcl} = mu delta_dl + (mu + 2 lambda (1 - ln J)) Finv[d][c] Finv[l][c].  The products
-// of 1D factors are separable, so each (d, l) pair is three transposed passes with the
-// elementwise-product tables BB, BD, DD.
+// L_{cdcl} = mu delta_dl + (mu + 2 lambda (1 - ln J)) Finv[d][c] Finv[l][c].  The products of 1D
+// factors are separable: with T0 = B.B, T1 = B.D, T2 = D.D (times w), pair (d, l) contracts
+// direction e with T_m, m the number of d, l equal to e.  x: six pairs, in place; y: the pairs of one
+// z-factor are added as they are contracted (00, 01, 11 | 02, 12 | 22); z: the three sums
+// at once.  15 line passes per component instead of 18 and the additions; the symmetric pairs'
+// factor 2 rides on the x tables, h and the material factor on the scatter.  FP64 operations per
+// point bound it.
 template <int P, bool SMALL> struct DiagCfg {
   using S = Shape<P, double, NHMF_CACHED, SMALL>;
   static constexpr int NE = SMALL ? S::NE : (S::NE / 2 > 0 ? S::NE / 2 : 1), THREADS = S::THREADS;
 };
+constexpr int kDiagFields = 21;  // 18 pair fields and u at the points
+
+// One line of NIN fields contracted and summed into `out`: y_k = sum_f sum_q tab[f][q][k] x_f[q].
+template <int n, int NIN>
+__device__ __forceinline__ void diag_line(const double* const (&tab)[NIN], const double* const (&in)[NIN], double* out,
+                                          int s) {
+  double y[n];
+#pragma unroll
+  for (int f = 0; f < NIN; ++f) {
+    double x[n];
+#pragma unroll
+    for (int q = 0; q < n; ++q) x[q] = in[f][q * s];
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+#pragma unroll
+      for (int q = 0; q < n; ++q) y[k] = f == 0 && q == 0 ? tab[f][k] * x[0] : fma(tab[f][q * n + k], x[q], y[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < n; ++k) out[k * s] = y[k];
+}
 
 template <int P, bool SMALL>
 __global__ void __launch_bounds__(DiagCfg<P, SMALL>::THREADS) k_diagonal(const OpArgs a) {
   using T = double;
-  constexpr int n = P + 1, n3 = n * n * n, NE = DiagCfg<P, SMALL>::NE, NI = NE * n3;
+  constexpr int n = P + 1, n3 = n * n * n, NE = DiagCfg<P, SMALL>::NE, NI = NE * n3, NL = NE * n * n;
+  constexpr int S = kMaxN * kMaxN, TH = DiagCfg<P, SMALL>::THREADS;
+  constexpr bool EO = n % 2 == 1;
+  static_assert(7 * S + kEoSlots + NE <= kTabSlots, "the diagonal's tables exceed the table slots");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sB = reinterpret_cast<T*>(smem_raw);
-  T* sDc = sB + kMaxN * kMaxN;
-  T* sD = sDc + kMaxN * kMaxN;
-  T* sW = sD + kMaxN * kMaxN;
-  T* sBB = sB + kTabSlots;  // 3 product tables, n*n each
-  T* sBD = sBB + kMaxN * kMaxN;
-  T* sDD = sBD + kMaxN * kMaxN;
-  T* Cq = sDD + kMaxN * kMaxN + 1;  // [20][NI]: Finv (9), ln J, and for the split model F (9), J - 1
-  T* S = Cq + 20 * NI;              // [3][NI]
-  T* tmp = S + 3 * NI;              // [3][NI]
-  T* R = tmp + 3 * NI;              // [3][NI]
+  T *sDch = sB + S, *tBB = sDch + S, *tBD = tBB + S, *tDD = tBD + S, *t2BB = tDD + S, *t2BD = t2BB + S;
+  T *kB = t2BD + S, *sF = kB + kEoSlots;
+  T* X = sB + kTabSlots;  // [18][NI]: field 3 pair + c, pairs 00, 01, 02, 11, 12, 22
+  T* Vq = X + 18 * NI;    // [3][NI]
   pdl_launch_next();
-  load_tables<P>(a, sB, sDc, sD, sW, a.h);
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
-    const int q = i / n, k = i % n;
-    sBB[i] = a.B[q * n + k] * a.B[q * n + k];
-    sBD[i] = a.B[q * n + k] * a.D[q * n + k];
-    sDD[i] = a.D[q * n + k] * a.D[q * n + k];
+    const T b = a.B[i], d = a.D[i], w = a.w[i / n];
+    sB[i] = b;
+    sDch[i] = a.Dch[i];
+    tBB[i] = w * b * b;
+    tBD[i] = w * b * d;
+    tDD[i] = w * d * d;
+    t2BB[i] = 2.0 * (w * b * b);
+    t2BD[i] = 2.0 * (w * b * d);
   }
+  for (int i = threadIdx.x; i < kEoSlots; i += blockDim.x) kB[i] = a.eo[0][i];
   const long long e0 = (long long)blockIdx.x * NE;
   const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
-  gather<P, NI>(a, a.u64, e0, nvalid, false, S);
+  const int nitems = nvalid * n3, nlines = nvalid * n * n;
+  for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = a.h * elem_factor(a, e0 + min(e, nvalid - 1));
+  gather<P, NI>(a, a.u64, e0, nvalid, false, X);
   __syncthreads();
-  const int nitems = nvalid * n3;
-  to_points<n, NI>(sB, S, tmp, tmp, nitems);
-  const double invh = 1.0 / a.h;
+  if constexpr (EO) {
+    eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, X, Vq, nlines);
+    __syncthreads();
+    eo_pass<n, NI, 3, 1, false, kEoCentreRow, TH>(kB, Vq, X, nlines);
+    __syncthreads();
+    eo_pass<n, NI, 3, 2, false, kEoCentreRow, TH>(kB, X, Vq, nlines);
+    __syncthreads();
+  } else {
+    to_points<n, NI>(sB, X, Vq, Vq, nitems);
+  }
   for (int t = threadIdx.x; t < nitems; t += blockDim.x) {
-    double H[9], Fi[9], lnJ;
-    colloc_grad<n, NI>(sDc, tmp, t, H);
-#pragma unroll
-    for (int k = 0; k < 9; ++k) H[k] *= invh;
-    const double Jm1 = kinematics(H, Fi, lnJ);
-#pragma unroll
-    for (int k = 0; k < 9; ++k) Cq[k * NI + t] = Fi[k];
-    Cq[9 * NI + t] = lnJ;
+    T H[9];
+    colloc_grad<n, NI>(sDch, Vq, t, H);
+    const Kinematics<T> kin(H);
+    const int pd[6] = {0, 0, 0, 1, 1, 2}, pl[6] = {0, 1, 2, 1, 2, 2};
     if (a.model == NHMF_MODEL_SPLIT) {
+      // L_cdcl = mu a d_dl - 2/3 mu a (F_cd Fi_lc + Fi_dc F_cl) + (2/9 mu a I1 + kappa J^2
+      //          + mu a I1/3 - kappa/2 (J^2 - 1)) Fi_dc Fi_lc
+      const T J = 1.0 + kin.Jm1, J2 = J * J, mua = a.mu * exp(-2.0 / 3.0 * kin.lnJ);
+      T I1 = 0.0, F[9], Fi[9];
 #pragma unroll
-      for (int k = 0; k < 9; ++k) Cq[(10 + k) * NI + t] = (k % 4 == 0 ? 1.0 : 0.0) + H[k];
-      Cq[19 * NI + t] = Jm1;
+      for (int k = 0; k < 9; ++k) {
+        F[k] = (k % 4 == 0 ? 1.0 : 0.0) + H[k];
+        Fi[k] = kin.A[k] * kin.invJ;
+        I1 += F[k] * F[k];
+      }
+      const T cff = 2.0 / 9.0 * mua * I1 + a.lam * J2 + mua * I1 / 3.0 - 0.5 * a.lam * (J2 - 1.0);
+#pragma unroll
+      for (int pr = 0; pr < 6; ++pr)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int d = pd[pr], l = pl[pr];
+          const T Fidc = Fi[3 * d + c], Filc = Fi[3 * l + c];
+          X[(3 * pr + c) * NI + t] = (d == l ? mua : 0.0) - 2.0 / 3.0 * mua * (F[3 * c + d] * Filc + Fidc * F[3 * c + l]) +
+                                     cff * Fidc * Filc;
+        }
+    } else {
+      const T kap = fma(2.0 * a.lam, 1.0 - kin.lnJ, a.mu) * (kin.invJ * kin.invJ);  // the adjugate enters twice
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        T f[3], kf[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          f[d] = kin.A[3 * d + c];
+          kf[d] = kap * f[d];
+        }
+#pragma unroll
+        for (int pr = 0; pr < 6; ++pr)
+          X[(3 * pr + c) * NI + t] = pd[pr] == pl[pr] ? fma(kf[pd[pr]], f[pl[pr]], a.mu) : kf[pd[pr]] * f[pl[pr]];
+      }
     }
-    for (int c = 0; c < 3; ++c) R[c * NI + t] = 0.0;
   }
   __syncthreads();
-  for (int d = 0; d < 3; ++d)
-    for (int l = d; l < 3; ++l) {
-      for (int t = threadIdx.x; t < nitems; t += blockDim.x) {
-        const double s = sW[t % n3] * (d == l ? 1.0 : 2.0) * elem_factor(a, e0 + min(t / n3, nvalid - 1));
-        if (a.model == NHMF_MODEL_SPLIT) {
-          // L_cdcl = mu a d_dl - 2/3 mu a (F_cd Fi_lc + Fi_dc F_cl) + (2/9 mu a I1 + kappa J^2
-          //          + mu a I1/3 - kappa/2 (J^2 - 1)) Fi_dc Fi_lc
-          const double lnJ = Cq[9 * NI + t], J = 1.0 + Cq[19 * NI + t], J2 = J * J;
-          const double mua = a.mu * exp(-2.0 / 3.0 * lnJ);
-          double I1 = 0.0;
-#pragma unroll
-          for (int k = 0; k < 9; ++k) I1 += Cq[(10 + k) * NI + t] * Cq[(10 + k) * NI + t];
-          const double cff = 2.0 / 9.0 * mua * I1 + a.lam * J2 + mua * I1 / 3.0 - 0.5 * a.lam * (J2 - 1.0);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const double Fidc = Cq[(3 * d + c) * NI + t], Filc = Cq[(3 * l + c) * NI + t];
-            const double Fcd = Cq[(10 + 3 * c + d) * NI + t], Fcl = Cq[(10 + 3 * c + l) * NI + t];
-            const double L = (d == l ? mua : 0.0) - 2.0 / 3.0 * mua * (Fcd * Filc + Fidc * Fcl) + cff * Fidc * Filc;
-            S[c * NI + t] = s * L;
-          }
-        } else {
-          const double kap = a.mu + 2.0 * a.lam * (1.0 - Cq[9 * NI + t]);
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const double L = (d == l ? a.mu : 0.0) + kap * Cq[(3 * d + c) * NI + t] * Cq[(3 * l + c) * NI + t];
-            S[c * NI + t] = s * L;
-          }
-        }
-      }
-      __syncthreads();
-      // direction x uses DD if d == l == 0, BD if exactly one of d, l is 0, else BB
-      const T* mx = (d == 0 && l == 0) ? sDD : ((d == 0 || l == 0) ? sBD : sBB);
-      const T* my = (d == 1 && l == 1) ? sDD : ((d == 1 || l == 1) ? sBD : sBB);
-      const T* mz = (d == 2 && l == 2) ? sDD : ((d == 2 || l == 2) ? sBD : sBB);
-      sf_pass<n, NI, 3, 0, true, false>(mx, S, tmp, nitems);
-      __syncthreads();
-      sf_pass<n, NI, 3, 1, true, false>(my, tmp, S, nitems);
-      __syncthreads();
-      sf_pass<n, NI, 3, 2, true, true>(mz, S, R, nitems);
-      __syncthreads();
+  for (int task = threadIdx.x; task < 18 * NL; task += TH) {
+    const int f = task / NL, L = task - f * NL;
+    if (L >= nlines) continue;
+    const int pr = f / 3;
+    T* x = X + f * NI + L * n;
+    const T* const tab[1] = {pr == 0 ? tDD : pr < 3 ? t2BD : pr == 4 ? t2BB : tBB};
+    const T* const in[1] = {x};
+    diag_line<n, 1>(tab, in, x, 1);
+  }
+  __syncthreads();
+  for (int task = threadIdx.x; task < 9 * NL; task += TH) {
+    const int g = task / (3 * NL), rest = task - g * 3 * NL, c = rest / NL, L = rest - c * NL;
+    if (L >= nlines) continue;
+    T* x = X + c * NI + (L % n) + (L / n) * n * n;
+    if (g == 0) {
+      const T* const tab[3] = {tBB, tBD, tDD};
+      const T* const in[3] = {x, x + 3 * NI, x + 9 * NI};
+      diag_line<n, 3>(tab, in, x, n);
+    } else if (g == 1) {
+      const T* const tab[2] = {tBB, tBD};
+      const T* const in[2] = {x + 6 * NI, x + 12 * NI};
+      diag_line<n, 2>(tab, in, x + 6 * NI, n);
+    } else {
+      const T* const tab[1] = {tBB};
+      const T* const in[1] = {x + 15 * NI};
+      diag_line<n, 1>(tab, in, x + 15 * NI, n);
     }
-  scatter_add<P, NI>(a, R, e0, nvalid, static_cast<double*>(a.v));
+  }
+  __syncthreads();
+  for (int task = threadIdx.x; task < 3 * NL; task += TH) {
+    const int c = task / NL, L = task - c * NL;
+    if (L >= nlines) continue;
+    T* x = X + c * NI + (L % (n * n)) + (L / (n * n)) * n * n * n;
+    const T* const tab[3] = {tBB, tBD, tDD};
+    const T* const in[3] = {x, x + 6 * NI, x + 15 * NI};
+    diag_line<n, 3>(tab, in, x, n * n);
+  }
+  __syncthreads();
+  scatter_add<P, NI>(a, X, e0, nvalid, static_cast<double*>(a.v), (const T*)sF);
 }
 
 // ------------------------------------------------------------------ result vector
@@ -985,6 +1099,7 @@ OpArgs base_args(nhmf_ctx* c) {
     eo_pack(a.B, n, a.eo[0]);
     eo_pack(a.Dc, n, a.eo[1]);
     eo_pack(BWt, n, a.eo[2]);
+    eo_pack(a.Dch, n, a.eoh);
     eo_pack(DcWt, n, a.eo[3]);  // DcW^T is anti-centro-symmetric like Dc (symmetric weights)
   }
   a.r2mu = 2.0 * c->prm.lambda / c->prm.mu;
@@ -1221,7 +1336,7 @@ template <int P, bool SMALL>
 nhmf_status diagonal_shape(nhmf_ctx* c, const OpArgs& a, double* d, cudaStream_t s) {
   using Sh = DiagCfg<P, SMALL>;
   constexpr int n3 = (P + 1) * (P + 1) * (P + 1);
-  const size_t smem = (kTabSlots + 3 * kMaxN * kMaxN + 1 + 29 * (size_t)Sh::NE * n3) * sizeof(double);
+  const size_t smem = (kTabSlots + kDiagFields * (size_t)Sh::NE * n3) * sizeof(double);
   return run_colours<double>(c, k_diagonal<P, SMALL>, a, Sh::NE, Sh::THREADS, smem, nullptr, d, 1.0, s, "diagonal",
                              NHMF_KIND_DIAGONAL);
 }

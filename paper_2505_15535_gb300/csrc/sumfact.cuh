@@ -93,10 +93,11 @@ struct OpArgs {
   // Tables of the tangent apply, which carry the quadrature weight, mu and h so that its
   // point code returns dP / mu unweighted:
   //   BW[q][i] = B[q][i] w_q,  DcW[m][r] = Dc[m][r] w_m / w_r mu h,  Dch = Dc / h,
-  //   eo[0..3]: even-odd coefficients of B, Dc, BW^T and DcW^T (odd n, see eo_line),
+  //   eo[0..3], eoh: even-odd coefficients of B, Dc, BW^T, DcW^T and Dch (odd n, see eo_line),
   //   r2mu = 2 lambda / mu.
   double BW[kMaxN * kMaxN], DcW[kMaxN * kMaxN], Dch[kMaxN * kMaxN];
   double eo[4][kEoSlots];
+  double eoh[kEoSlots];  // of Dch
   double r2mu;
   int reg32;  // FP32 point cache in the register kernel's [10][n^3][E] layout (see kRegMaxP)
   float BWf[kMaxN * kMaxN], DcWf[kMaxN * kMaxN], Dchf[kMaxN * kMaxN], eof[4][kEoSlots];  // FP32 copies
@@ -408,32 +409,81 @@ __device__ __forceinline__ void colloc_grad_T(const T* __restrict__ Dc, const T*
 }
 
 // ------------------------------------------------------------------ point code
-// Kinematics at a point from the physical displacement gradient H (row-major H[3c+d]):
-// J - 1 from the invariants of H (no cancellation near J = 1),
-//   J - 1 = tr H + ((tr H)^2 - tr(H^2))/2 + det H,
-// F^-1 = cof(F)^T / J, ln J = log1p(J - 1).  Returns J - 1.
+// The FP64 pipe (2 DFMA per clock and SM) bounds every FP64 kernel, so its point code counts FP64
+// instructions.  CUDA's 1 / x and log1p took about 70 of them at a point; the two below take 16.
+
+// 1 / x by Newton's iteration, third order: y0 = rcp.approx(x) (relative error below 2^-20), e = 1 -
+// x y0, y = y0 (1 + e + e^2) with error e^3 < 2^-60 before rounding.  x a normal number whose
+// reciprocal is normal.
+__device__ __forceinline__ double fast_rcp(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float fast_rcp(float x) { return 1.f / x; }
+
+// log1p(x) given J = 1 + x, table driven (P. T. P. Tang, "Table-driven implementation of the
+// logarithm function in IEEE floating-point arithmetic", ACM TOMS 16, 1990): J = 2^k m with m in
+// [0.75, 1.5), c from the table near 1 / m, r = c 2^-k (1 + x) - 1 from x itself (one rounding, so
+// small x keep their relative accuracy; c = 1 next to J = 1), |r| <= 2^-7, and log1p(x) = k ln 2 -
+// ln c + log1p(r) with the series to r^8 (next term below 2^-66).  J not positive, not finite or
+// subnormal goes to CUDA's function.
+#include "log_table.h"
+__device__ __forceinline__ double fast_log1p(double x, double J) {
+  const int hi = __double2hiint(J);
+  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log1p(x);
+  const int t = hi - 0x3fe80000, k = t >> 20, i = (t >> 13) & 127;  // m >= 0.75: exponent field of 0.75
+  double c = __ldg(&kLogTable[i][0]), l = __ldg(&kLogTable[i][1]);
+  if (k != 0) {
+    c *= __hiloint2double((1023 - k) << 20, 0);
+    l = fma((double)k, 0.69314718055994530942, l);
+  }
+  const double r = fma(c, x, c - 1.0);
+  double p = fma(r, -1.0 / 8.0, 1.0 / 7.0);
+  p = fma(r, p, -1.0 / 6.0);
+  p = fma(r, p, 1.0 / 5.0);
+  p = fma(r, p, -1.0 / 4.0);
+  p = fma(r, p, 1.0 / 3.0);
+  p = fma(r, p, -1.0 / 2.0);
+  return l + fma(r * r, p, r);
+}
+__device__ __forceinline__ float fast_log1p(float x, float) { return log1pf(x); }
+
+// Kinematics at a point from the physical displacement gradient H (row-major H[3c+d]), F = I + H:
+// the adjugate A = J F^-1, 1 / J, ln J and J - 1.  With C00 - 1 = H4 + H8 + H4 H8 - H5 H7,
+//   J - 1 = H0 + F0 (C00 - 1) + H1 C01 + H2 C02
+// has no cancellation near F = I (25 operations for A and J - 1).
+template <typename T>
+struct Kinematics {
+  T A[9], invJ, lnJ, Jm1;
+  __device__ __forceinline__ explicit Kinematics(const T H[9]) {
+    const T F0 = T(1) + H[0], F4 = T(1) + H[4], F8 = T(1) + H[8];
+    const T C = fma(-H[5], H[7], fma(H[4], F8, H[8]));  // C00 - 1
+    A[0] = T(1) + C;
+    A[1] = fma(H[2], H[7], -(H[1] * F8));
+    A[2] = fma(H[1], H[5], -(H[2] * F4));
+    A[3] = fma(H[5], H[6], -(H[3] * F8));
+    A[4] = fma(F0, F8, -(H[2] * H[6]));
+    A[5] = fma(H[2], H[3], -(F0 * H[5]));
+    A[6] = fma(H[3], H[7], -(F4 * H[6]));
+    A[7] = fma(H[1], H[6], -(F0 * H[7]));
+    A[8] = fma(F0, F4, -(H[1] * H[3]));
+    Jm1 = fma(F0, C, fma(H[1], A[3], fma(H[2], A[6], H[0])));
+    const T J = T(1) + Jm1;
+    invJ = fast_rcp(J);
+    lnJ = fast_log1p(Jm1, J);
+  }
+};
+
+// The same as F^-1 = A / J and ln J; returns J - 1.
 template <typename T>
 __device__ __forceinline__ T kinematics(const T H[9], T Fi[9], T& lnJ) {
-  const T trH = H[0] + H[4] + H[8];
-  const T trH2 = H[0] * H[0] + H[4] * H[4] + H[8] * H[8] +
-                 T(2) * (H[1] * H[3] + H[2] * H[6] + H[5] * H[7]);
-  const T detH = H[0] * (H[4] * H[8] - H[5] * H[7]) - H[1] * (H[3] * H[8] - H[5] * H[6]) +
-                 H[2] * (H[3] * H[7] - H[4] * H[6]);
-  const T Jm1 = trH + T(0.5) * (trH * trH - trH2) + detH;
-  const T F0 = T(1) + H[0], F4 = T(1) + H[4], F8 = T(1) + H[8];
-  const T F1 = H[1], F2 = H[2], F3 = H[3], F5 = H[5], F6 = H[6], F7 = H[7];
-  const T invJ = T(1) / (T(1) + Jm1);
-  Fi[0] = (F4 * F8 - F5 * F7) * invJ;
-  Fi[1] = (F2 * F7 - F1 * F8) * invJ;
-  Fi[2] = (F1 * F5 - F2 * F4) * invJ;
-  Fi[3] = (F5 * F6 - F3 * F8) * invJ;
-  Fi[4] = (F0 * F8 - F2 * F6) * invJ;
-  Fi[5] = (F2 * F3 - F0 * F5) * invJ;
-  Fi[6] = (F3 * F7 - F4 * F6) * invJ;
-  Fi[7] = (F1 * F6 - F0 * F7) * invJ;
-  Fi[8] = (F0 * F4 - F1 * F3) * invJ;
-  lnJ = log1p(Jm1);
-  return Jm1;
+  const Kinematics<T> k(H);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) Fi[i] = k.A[i] * k.invJ;
+  lnJ = k.lnJ;
+  return k.Jm1;
 }
 
 // Linearised first Piola stress at a point, scaled by s (Eq. LG: G = L : Grad du):
@@ -464,24 +514,35 @@ __device__ __forceinline__ void linearised_stress(const T Fi[9], T lnJ, const T 
 
 // The same linearised stress divided by mu and without the point weight (the tangent apply
 // carries w_q, mu and h on its transposed tables), r = 2 lambda / mu:
-//   g = dH + (1 - r ln J) Q^T + r tr(K) F^-T.
+//   g = dH + (1 - r ln J) (K F^-1)^T + r tr(K) F^-T = dH + ((c1 K + c2 I) F^-1)^T:
+// 67 operations instead of 76 with the two terms added separately.
 template <typename T>
-__device__ __forceinline__ void linearised_stress_unit(const T Fi[9], T lnJ, const T dH[9], T r, T g[9]) {
+__device__ __forceinline__ void linearised_stress_unit(const T Fi[9], T c1, T rs, const T dH[9], T g[9]) {
   T K[9];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int j = 0; j < 3; ++j)
       K[3 * i + j] = fma(Fi[3 * i + 0], dH[j], fma(Fi[3 * i + 1], dH[3 + j], Fi[3 * i + 2] * dH[6 + j]));
-  const T c1 = fma(-r, lnJ, T(1));
-  const T c2 = r * (K[0] + K[4] + K[8]);
+  const T c2 = rs * (K[0] + K[4] + K[8]);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) K[k] = k % 4 == 0 ? fma(c1, K[k], c2) : c1 * K[k];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const T Qji = fma(K[3 * j + 0], Fi[i], fma(K[3 * j + 1], Fi[3 + i], K[3 * j + 2] * Fi[6 + i]));
-      g[3 * i + j] = fma(c1, Qji, fma(c2, Fi[3 * j + i], dH[3 * i + j]));
-    }
+    for (int j = 0; j < 3; ++j)
+      g[3 * i + j] = fma(K[3 * j + 0], Fi[i], fma(K[3 * j + 1], Fi[3 + i], fma(K[3 * j + 2], Fi[6 + i], dH[3 * i + j])));
+}
+// from F^-1 and ln J
+template <typename T>
+__device__ __forceinline__ void linearised_stress_unit(const T Fi[9], T lnJ, const T dH[9], T r, T g[9]) {
+  linearised_stress_unit(Fi, fma(-r, lnJ, T(1)), r, dH, g);
+}
+// from the adjugate: F^-1 = A / J enters twice, so both coefficients carry 1 / J^2
+template <typename T>
+__device__ __forceinline__ void linearised_stress_unit(const Kinematics<T>& k, const T dH[9], T r, T g[9]) {
+  const T s = k.invJ * k.invJ;
+  linearised_stress_unit(k.A, fma(-r, k.lnJ, T(1)) * s, r * s, dH, g);
 }
 
 // Split neo-Hookean model (Eq. hypcomplex), with a = J^(-2/3), I1 = F : F:
