@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "apply32.cuh"
 #include "df64.cuh"
 #include "sumfact.cuh"
 
@@ -25,7 +26,7 @@ namespace {
 // Table slots ahead of the per-item arrays: B, Dc, D, n^3 weights and NE factors, or in the
 // apply B, Dc, BW, DcW, Dch, 3 even-odd sets and NE factors (whichever is larger).
 constexpr int kTabSlots = 3 * kMaxN * kMaxN + 128 + 32;
-static_assert(5 * kMaxN * kMaxN + 4 * kEoSlots + 32 <= kTabSlots, "apply tables exceed the table slots");
+static_assert(5 * kMaxN * kMaxN + 3 * kEoSlots + 32 <= kTabSlots, "apply tables exceed the table slots");
 
 template <int P, typename T>
 __device__ __forceinline__ void load_tables(const OpArgs& a, T* sB, T* sDc, T* sD, T* sW, double wscale) {
@@ -52,7 +53,7 @@ __device__ __forceinline__ void load_apply_tables(const OpArgs& a, T* tab, const
     tab[3 * S + i] = T(a.DcW[i]);
     tab[4 * S + i] = T(a.Dch[i]);
   }
-  for (int i = threadIdx.x; i < 4 * kEoSlots; i += blockDim.x)
+  for (int i = threadIdx.x; i < 3 * kEoSlots; i += blockDim.x)
     tab[5 * S + i] = T(deriv && i / kEoSlots == 1 ? deriv[i % kEoSlots] : a.eo[i / kEoSlots][i % kEoSlots]);
 }
 
@@ -152,17 +153,17 @@ __device__ __forceinline__ void from_points(const T* sB, const T* sDc, T* G, T* 
 
 // The transposed passes of the apply and the residual: fluxes G[3c+d] with the weighted tables BW,
 // DcW (kBW: even-odd coefficients of BW^T) to nodal values in G[3..5].
-template <int n, int NI, int TH, bool EO, typename T, typename MAP = NoLineMap>
+template <int n, int NI, int TH, bool EO, typename T>
 __device__ __forceinline__ void transposed(const T* sBW, const T* sDcW, const T* kBW, T* G, T* Vq, int nitems,
-                                           int nlines, const MAP& lm = MAP()) {
+                                           int nlines) {
   if constexpr (EO) {
     colloc_grad_T<n, NI>(sDcW, G, Vq, nitems);
     __syncthreads();
-    eo_pass<n, NI, 3, 0, false, kEoCentreCol, TH>(kBW, Vq, G, nlines, lm);
+    eo_pass<n, NI, 3, 0, false, kEoCentreCol, TH>(kBW, Vq, G, nlines);
     __syncthreads();
-    eo_pass<n, NI, 3, 1, false, kEoCentreCol, TH>(kBW, G, Vq, nlines, lm);
+    eo_pass<n, NI, 3, 1, false, kEoCentreCol, TH>(kBW, G, Vq, nlines);
     __syncthreads();
-    eo_pass<n, NI, 3, 2, false, kEoCentreCol, TH>(kBW, Vq, G + 3 * NI, nlines, lm);
+    eo_pass<n, NI, 3, 2, false, kEoCentreCol, TH>(kBW, Vq, G + 3 * NI, nlines);
     __syncthreads();
   } else {
     from_points<n, NI>(sBW, sDcW, G, Vq, G + 3 * NI, nitems);
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
   constexpr int n = P + 1, n3 = n * n * n, NE = Shape<P, T, STRAT, SMALL>::NE, NI = NE * n3;
   constexpr int S = kMaxN * kMaxN, TH = Shape<P, T, STRAT, SMALL>::THREADS;
   constexpr bool EO = n % 2 == 1;
-  static_assert(5 * S + 4 * kEoSlots + NE <= kTabSlots, "the factor table exceeds the table slots");
+  static_assert(5 * S + 3 * kEoSlots + NE <= kTabSlots, "the factor table exceeds the table slots");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
   const T* sB = tab;
@@ -191,19 +192,14 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
   const T* sBW = tab + 2 * S;
   const T* sDcW = tab + 3 * S;
   const T* sDch = tab + 4 * S;
-  const T* kB = tab + 5 * S;                    // even-odd coefficients of B, Dc, BW^T, DcW^T
+  const T* kB = tab + 5 * S;                    // even-odd coefficients of B, Dc, BW^T
   const T* kDc = kB + kEoSlots;
   const T* kBW = kDc + kEoSlots;
-  const T* kDcWT = kBW + kEoSlots;              // even-odd coefficients of DcW^T
-  T* sF = tab + 5 * S + 4 * kEoSlots;          // [NE] material factors of the block's elements
+  T* sF = tab + 5 * S + 3 * kEoSlots;          // [NE] material factors of the block's elements
   T* U = tab + kTabSlots;                       // [3][NI] ubar at the points (on the fly)
   T* Vq = U + (STRAT == NHMF_ON_THE_FLY ? 3 * NI : 0);  // [3][NI] du at the points
   T* G = Vq + 3 * NI;                           // [9][NI] gradients, then fluxes; G[0..2] gathers
 
-  // FP32: the passes' task decomposition computed once (the FP32 kernel is issue bound)
-  using LM = typename std::conditional<std::is_same<T, float>::value && NHMF_LINEMAP && EO, LineMap<n, NI, TH>,
-                                       NoLineMap>::type;
-  const LM lm{};
   pdl_launch_next();
   load_apply_tables<P>(a, tab);
   const long long e0 = (long long)blockIdx.x * NE;
@@ -219,11 +215,11 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
       gather<P, NI>(a, a.u32, e0, nvalid, false, G);
     __syncthreads();
     if constexpr (EO) {
-      eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, G, Vq, nlines, lm);
+      eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, G, Vq, nlines);
       __syncthreads();
-      eo_pass<n, NI, 3, 1, false, kEoCentreRow, TH>(kB, Vq, G, nlines, lm);
+      eo_pass<n, NI, 3, 1, false, kEoCentreRow, TH>(kB, Vq, G, nlines);
       __syncthreads();
-      eo_pass<n, NI, 3, 2, false, kEoCentreRow, TH>(kB, G, U, nlines, lm);
+      eo_pass<n, NI, 3, 2, false, kEoCentreRow, TH>(kB, G, U, nlines);
       __syncthreads();
     } else {
       to_points<n, NI>(sB, G, Vq, U, nitems);
@@ -233,16 +229,16 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
                 a.factor ? (const T*)sF : nullptr);
   __syncthreads();
   if constexpr (EO) {
-    eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, G, Vq, nlines, lm);
+    eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, G, Vq, nlines);
     __syncthreads();
-    eo_pass<n, NI, 3, 1, false, kEoCentreRow, TH>(kB, Vq, G, nlines, lm);
+    eo_pass<n, NI, 3, 1, false, kEoCentreRow, TH>(kB, Vq, G, nlines);
     __syncthreads();
-    eo_pass<n, NI, 3, 2, false, kEoCentreRow, TH>(kB, G, Vq, nlines, lm);
+    eo_pass<n, NI, 3, 2, false, kEoCentreRow, TH>(kB, G, Vq, nlines);
     __syncthreads();
     // reference gradient of du: G[3c+d] = Dc along d of du[c]
-    eo_pass<n, NI, 3, 0, true, kEoGeneral, TH, 3, 0>(kDc, Vq, G, nlines, lm);
-    eo_pass<n, NI, 3, 1, true, kEoGeneral, TH, 3, 1>(kDc, Vq, G, nlines, lm);
-    eo_pass<n, NI, 3, 2, true, kEoGeneral, TH, 3, 2>(kDc, Vq, G, nlines, lm);
+    eo_pass<n, NI, 3, 0, true, kEoGeneral, TH, 3, 0>(kDc, Vq, G, nlines);
+    eo_pass<n, NI, 3, 1, true, kEoGeneral, TH, 3, 1>(kDc, Vq, G, nlines);
+    eo_pass<n, NI, 3, 2, true, kEoGeneral, TH, 3, 2>(kDc, Vq, G, nlines);
     __syncthreads();
   } else {
     to_points<n, NI>(sB, G, Vq + 0, Vq, nitems);  // passes ping-pong via G: x G->Vq, y Vq->G, z G->Vq
@@ -337,23 +333,7 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
   }
   if (bad) atomicOr(a.status, kStatusNonPosJ);
   __syncthreads();
-  if constexpr (EO && std::is_same<T, float>::value) {
-    // FP32: the transposed derivative as three even-odd line passes, Vq[c] = sum_d DcW^T_d G[3c+d]
-    eo_pass<n, NI, 3, 0, true, kEoGeneral, TH, 1, 0, 3, 0, false>(kDcWT, G, Vq, nlines, lm);
-    __syncthreads();
-    eo_pass<n, NI, 3, 1, true, kEoGeneral, TH, 1, 0, 3, 1, true>(kDcWT, G, Vq, nlines, lm);
-    __syncthreads();
-    eo_pass<n, NI, 3, 2, true, kEoGeneral, TH, 1, 0, 3, 2, true>(kDcWT, G, Vq, nlines, lm);
-    __syncthreads();
-    eo_pass<n, NI, 3, 0, false, kEoCentreCol, TH>(kBW, Vq, G, nlines, lm);
-    __syncthreads();
-    eo_pass<n, NI, 3, 1, false, kEoCentreCol, TH>(kBW, G, Vq, nlines, lm);
-    __syncthreads();
-    eo_pass<n, NI, 3, 2, false, kEoCentreCol, TH>(kBW, Vq, G + 3 * NI, nlines, lm);
-    __syncthreads();
-  } else {
-    transposed<n, NI, TH, EO>(sBW, sDcW, kBW, G, Vq, nitems, nlines, lm);
-  }
+  transposed<n, NI, TH, EO>(sBW, sDcW, kBW, G, Vq, nitems, nlines);
   if constexpr (std::is_same<T, float>::value) {
     if (a.vloc) {
       store_local<P, NE>(a, G + 3 * NI, e0, nvalid);
@@ -571,7 +551,7 @@ __global__ void __launch_bounds__(kRegThreads, NHMF_REG_MINB) k_apply_reg(const 
         if constexpr (STRAT == NHMF_ON_THE_FLY && MODEL == NHMF_MODEL_SPLIT)
           split_stress_dP(F, Fi, lnJ, Jm1, dH, float(a.mu), float(a.lam), inv_mu, g);
         else
-          linearised_stress_unit(Fi, lnJ, dH, r2, g);
+          linearised_stress_terms(Fi, fmaf(-r2, lnJ, 1.f), r2, dH, g);
         // transposed collocation derivative with the weights, mu and h:
         //   acc[c][point on the line through q] += DcW[q][m] g
 #pragma unroll
@@ -797,7 +777,7 @@ __global__ void __launch_bounds__(Shape<P, double, 0, SMALL>::THREADS) k_residua
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
   const T *kB = tab + 5 * S, *kDch = kB + kEoSlots, *kBW = kDch + kEoSlots;
-  T* sF = tab + 5 * S + 4 * kEoSlots;  // [NE] h times the material factors
+  T* sF = tab + 5 * S + 3 * kEoSlots;  // [NE] h times the material factors
   T* Vq = tab + kTabSlots;             // [3][NI] u at the points
   T* G = Vq + 3 * NI;                  // [9][NI] gradients, then fluxes
   pdl_launch_next();
@@ -1061,6 +1041,22 @@ void eo_pack(const double* M, int n, double* k) {
   }
 }
 
+// The even-odd form of an n x n line operator M (row-major) for the FP32 column kernel.
+EoTab eo_tab(const double* M, int n) {
+  EoTab t{};
+  const int h = n / 2;
+  for (int r = 0; r < h; ++r) {
+    for (int m = 0; m < h; ++m) {
+      t.S[r][m] = float(0.5 * (M[r * n + m] + M[r * n + n - 1 - m]));
+      t.A[r][m] = float(0.5 * (M[r * n + m] - M[r * n + n - 1 - m]));
+    }
+    t.C[r] = n % 2 == 1 ? float(M[r * n + h]) : 0.f;
+    t.mid[r] = n % 2 == 1 ? float(M[h * n + r]) : 0.f;
+  }
+  t.ch = n % 2 == 1 ? float(M[h * n + h]) : 0.f;
+  return t;
+}
+
 OpArgs base_args(nhmf_ctx* c) {
   OpArgs a{};
   a.N = c->g.N;
@@ -1085,14 +1081,13 @@ OpArgs base_args(nhmf_ctx* c) {
     a.wf[q] = float(c->tab.w[q]);
   }
   // tables of the tangent apply (see OpArgs)
-  double BWt[kMaxN * kMaxN], DcWt[kMaxN * kMaxN];
+  double BWt[kMaxN * kMaxN];
   for (int q = 0; q < n; ++q)
     for (int i = 0; i < n; ++i) {
       const double wq = c->tab.w[q];
       a.BW[q * n + i] = c->tab.B[q][i] * wq;
       BWt[i * n + q] = a.BW[q * n + i];
       a.DcW[q * n + i] = c->tab.Dc[q][i] * wq / c->tab.w[i] * c->prm.mu * c->g.h;
-      DcWt[i * n + q] = a.DcW[q * n + i];
       a.Dch[q * n + i] = c->tab.Dc[q][i] / c->g.h;
     }
   if (n % 2 == 1) {
@@ -1100,16 +1095,32 @@ OpArgs base_args(nhmf_ctx* c) {
     eo_pack(a.Dc, n, a.eo[1]);
     eo_pack(BWt, n, a.eo[2]);
     eo_pack(a.Dch, n, a.eoh);
-    eo_pack(DcWt, n, a.eo[3]);  // DcW^T is anti-centro-symmetric like Dc (symmetric weights)
   }
+  if (n >= 3) {
+    double DWt[kMaxN * kMaxN], BWz[kMaxN * kMaxN], DWz[kMaxN * kMaxN];
+    for (int q = 0; q < n; ++q)
+      for (int i = 0; i < n; ++i) {
+        DWt[i * n + q] = c->tab.D[q][i] * c->tab.w[q];
+        BWz[i * n + q] = BWt[i * n + q] * c->prm.mu * c->g.h;
+        DWz[i * n + q] = DWt[i * n + q] * c->prm.mu * c->g.h;
+      }
+    a.cB = eo_tab(a.B, n);
+    a.cD = eo_tab(a.D, n);
+    a.cBT = eo_tab(BWt, n);
+    a.cDT = eo_tab(DWt, n);
+    a.cBTz = eo_tab(BWz, n);
+    a.cDTz = eo_tab(DWz, n);
+  }
+  a.invhf = float(1.0 / c->g.h);
   a.r2mu = 2.0 * c->prm.lambda / c->prm.mu;
+  a.r2muf = float(a.r2mu);
   a.reg32 = c->reg32 ? 1 : 0;
   for (int i = 0; i < kMaxN * kMaxN; ++i) {
     a.BWf[i] = float(a.BW[i]);
     a.DcWf[i] = float(a.DcW[i]);
     a.Dchf[i] = float(a.Dch[i]);
   }
-  for (int k = 0; k < 4; ++k)
+  for (int k = 0; k < 3; ++k)
     for (int i = 0; i < kEoSlots; ++i) a.eof[k][i] = float(a.eo[k][i]);
   a.status = c->status;
   a.factor = c->factor;
@@ -1264,10 +1275,20 @@ nhmf_status apply_p(nhmf_ctx* c, const void* du, void* v, bool raw, const Gather
                             STRAT == NHMF_ON_THE_FLY ? kin_smem : 0, du32, v32, g32, s);
       }
     }
-    using Sh = Shape<P, T, STRAT, false>;
-    const size_t smem = (kTabSlots + per_item * Sh::NE * (P + 1) * (P + 1) * (P + 1)) * sizeof(T);
-    auto* k = split ? k_apply<P, T, STRAT, SPLIT, false> : k_apply<P, T, STRAT, NHMF_MODEL_COMPRESSIBLE, false>;
-    return run_local<P>(c, k, a, Sh::NE, Sh::THREADS, smem, du32, v32, g32, s);
+    if constexpr (P >= 2) {
+      using Sh = ColShape<P + 1>;
+      constexpr size_t field = (size_t)Sh::NE * (P + 1) * (P + 1) * (P + 1) * sizeof(float);
+      if (split)
+        return run_local<P>(c, k_apply_col<P, STRAT, SPLIT>, a, Sh::NE, Sh::THREADS,
+                            col_fields<P + 1, STRAT, SPLIT>() * field, du32, v32, g32, s);
+      return run_local<P>(c, k_apply_col<P, STRAT, NHMF_MODEL_COMPRESSIBLE>, a, Sh::NE, Sh::THREADS,
+                          col_fields<P + 1, STRAT, NHMF_MODEL_COMPRESSIBLE>() * field, du32, v32, g32, s);
+    } else {
+      using Sh = Shape<P, T, STRAT, false>;
+      const size_t smem = (kTabSlots + per_item * Sh::NE * (P + 1) * (P + 1) * (P + 1)) * sizeof(T);
+      auto* k = split ? k_apply<P, T, STRAT, SPLIT, false> : k_apply<P, T, STRAT, NHMF_MODEL_COMPRESSIBLE, false>;
+      return run_local<P>(c, k, a, Sh::NE, Sh::THREADS, smem, du32, v32, g32, s);
+    }
   } else {
     if (small_blocks<T, Shape<P, T, STRAT, false>::NE>(c))
       return split ? apply_colours<P, T, STRAT, SPLIT, true>(c, a, per_item, s)

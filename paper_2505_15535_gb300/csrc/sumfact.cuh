@@ -31,22 +31,7 @@ template <> struct Cfg<1, double> { static constexpr int NE = 32, THREADS = 256;
 template <> struct Cfg<2, double> { static constexpr int NE = NHMF_Q2D_NE, THREADS = NHMF_Q2D_THREADS; };
 template <> struct Cfg<3, double> { static constexpr int NE = 8, THREADS = 256; };
 template <> struct Cfg<4, double> { static constexpr int NE = NHMF_Q4D_NE, THREADS = NHMF_Q4D_THREADS; };
-template <> struct Cfg<1, float> { static constexpr int NE = 32, THREADS = 256; };
-#ifndef NHMF_Q2F_NE
-#define NHMF_Q2F_NE 8
-#define NHMF_Q2F_THREADS 224
-#endif
-template <> struct Cfg<2, float> { static constexpr int NE = NHMF_Q2F_NE, THREADS = NHMF_Q2F_THREADS; };
-#ifndef NHMF_Q3F_NE
-#define NHMF_Q3F_NE 8
-#define NHMF_Q3F_THREADS 256
-#endif
-#ifndef NHMF_Q4F_NE
-#define NHMF_Q4F_NE 4
-#define NHMF_Q4F_THREADS 160
-#endif
-template <> struct Cfg<3, float> { static constexpr int NE = NHMF_Q3F_NE, THREADS = NHMF_Q3F_THREADS; };
-template <> struct Cfg<4, float> { static constexpr int NE = NHMF_Q4F_NE, THREADS = NHMF_Q4F_THREADS; };
+template <> struct Cfg<1, float> { static constexpr int NE = 32, THREADS = 256; };  // p >= 2: ColShape (apply32.cuh)
 struct df64;
 template <int P> struct Cfg<P, df64> : Cfg<P, double> {};
 template <> struct Cfg<4, df64> { static constexpr int NE = 4, THREADS = 256; };
@@ -83,6 +68,13 @@ template <int P, typename T, int STRAT> struct Shape<P, T, STRAT, true> : SmallC
 // (h+1), h = n / 2.
 constexpr int kEoSlots = 16;
 
+// One n x n line operator of the FP32 column kernel in even-odd form, M[n-1-r][n-1-m] = +-M[r][m], h =
+// n / 2: S = (M_rm + M_r,n-1-m) / 2 and A = (M_rm - M_r,n-1-m) / 2 for r, m < h, C = M_rh, and the
+// centre row of odd n: mid_m = M_hm (its even or odd half) and ch = M_hh.
+struct EoTab {
+  float S[2][2], A[2][2], C[2], mid[2], ch;
+};
+
 // Kernel arguments (by value; lives in the constant bank).
 struct OpArgs {
   int N, M, bc, model;
@@ -93,15 +85,17 @@ struct OpArgs {
   // Tables of the tangent apply, which carry the quadrature weight, mu and h so that its
   // point code returns dP / mu unweighted:
   //   BW[q][i] = B[q][i] w_q,  DcW[m][r] = Dc[m][r] w_m / w_r mu h,  Dch = Dc / h,
-  //   eo[0..3], eoh: even-odd coefficients of B, Dc, BW^T, DcW^T and Dch (odd n, see eo_line),
+  //   eo[0..2], eoh: even-odd coefficients of B, Dc, BW^T and Dch (odd n, see eo_line),
   //   r2mu = 2 lambda / mu.
   double BW[kMaxN * kMaxN], DcW[kMaxN * kMaxN], Dch[kMaxN * kMaxN];
-  double eo[4][kEoSlots];
+  double eo[3][kEoSlots];
   double eoh[kEoSlots];  // of Dch
   double r2mu;
   int reg32;  // FP32 point cache in the register kernel's [10][n^3][E] layout (see kRegMaxP)
-  float BWf[kMaxN * kMaxN], DcWf[kMaxN * kMaxN], Dchf[kMaxN * kMaxN], eof[4][kEoSlots];  // FP32 copies
+  float BWf[kMaxN * kMaxN], DcWf[kMaxN * kMaxN], Dchf[kMaxN * kMaxN], eof[3][kEoSlots];  // FP32 copies
   float Bf[kMaxN * kMaxN], Dcf[kMaxN * kMaxN], wf[kMaxN];  // FP32 copies (register kernels)
+  EoTab cB, cD, cBT, cDT, cBTz, cDTz;  // B, D and the weighted transposes; z: times mu h
+  float invhf, r2muf;                  // 1 / h, r2mu
   const double* u64;
   const float* u32;
   const void* du;
@@ -143,6 +137,12 @@ __device__ __forceinline__ float ld_policy(const float* a, unsigned long long po
 #else
   return __ldg(a);
 #endif
+}
+// The same, kept in program order (a prefetch that must not sink to its use).
+__device__ __forceinline__ float ld_policy_ordered(const float* a, unsigned long long pol) {
+  float v;
+  asm volatile("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol));
+  return v;
 }
 __device__ __forceinline__ double ld_policy(const double* a, unsigned long long pol) {
 #if NHMF_L2HINT
@@ -292,36 +292,15 @@ __device__ __forceinline__ void eo_line(const T (&k)[kEoSlots], const T (&x)[n],
   }
 }
 
-// The tasks of a pass over 3 fields with one thread per (field, line): this thread's field,
-// line and line start for each direction, computed once per kernel instead of in every pass.
-struct NoLineMap {};
-template <int n, int NI, int TH>
-struct LineMap {
-  static constexpr int NL = NI / n, ITER = (3 * NL + TH - 1) / TH;
-  int c[ITER], L[ITER], base[3][ITER];
-  __device__ __forceinline__ LineMap() {
-#pragma unroll
-    for (int it = 0; it < ITER; ++it) {
-      const int task = threadIdx.x + it * TH;
-      c[it] = task / NL;  // >= 3: no task
-      L[it] = task - c[it] * NL;
-      base[0][it] = L[it] * n;
-      base[1][it] = (L[it] % n) + (L[it] / n) * n * n;
-      base[2][it] = (L[it] % (n * n)) + (L[it] / (n * n)) * n * n * n;
-    }
-  }
-};
-
 // One 1D pass along DIR over NC fields with one thread per (field, line of n items), odd n:
-//   out[(c OS + OO)][line] (+)= M in[(c IS + IO)][line]  (+= when ACC)
+//   out[(c OS + OO)][line] = M in[c][line]
 // where M is given by its even-odd coefficients `coef` (see eo_line).
 // TH is the block size; the task loop is unrolled so that independent lines interleave (not for
 // double-float, whose unrolled lines would cost an SM its second block).
 // Lines of absent elements (line index >= nlines; they come last) are skipped.
-template <int n, int NI, int NC, int DIR, bool ANTI, int FORM, int TH, int OS = 1, int OO = 0, int IS = 1,
-          int IO = 0, bool ACC = false, typename T, typename MAP = NoLineMap>
+template <int n, int NI, int NC, int DIR, bool ANTI, int FORM, int TH, int OS = 1, int OO = 0, typename T>
 __device__ __forceinline__ void eo_pass(const T* __restrict__ coef, const T* __restrict__ in,
-                                        T* __restrict__ out, int nlines = NI / n, const MAP& map = MAP()) {
+                                        T* __restrict__ out, int nlines = NI / n) {
   constexpr int s = DIR == 0 ? 1 : (DIR == 1 ? n : n * n), NL = NI / n, ITER = (NC * NL + TH - 1) / TH;
   constexpr int UNROLL = std::is_same<T, df64>::value ? 1 : ITER;
   T k[kEoSlots];
@@ -329,33 +308,18 @@ __device__ __forceinline__ void eo_pass(const T* __restrict__ coef, const T* __r
   for (int i = 0; i < kEoSlots; ++i) k[i] = coef[i];
 #pragma unroll UNROLL
   for (int it = 0; it < ITER; ++it) {
-    int c, L, base;
-    if constexpr (std::is_same<MAP, NoLineMap>::value) {
-      const int task = threadIdx.x + it * TH;
-      if (ITER * TH != NC * NL && task >= NC * NL) break;
-      c = task / NL;
-      L = task - c * NL;
-      base = DIR == 0 ? L * n
-                      : (DIR == 1 ? (L % n) + (L / n) * n * n : (L % (n * n)) + (L / (n * n)) * n * n * n);
-    } else {
-      static_assert(NC == 3 && MAP::ITER == ITER && MAP::NL == NL, "a line map covers passes over 3 fields");
-      c = map.c[it];
-      if (ITER * TH != NC * NL && c >= NC) break;
-      L = map.L[it];
-      base = map.base[DIR][it];
-    }
+    const int task = threadIdx.x + it * TH;
+    if (ITER * TH != NC * NL && task >= NC * NL) break;
+    const int c = task / NL, L = task - c * NL;
+    const int base = DIR == 0 ? L * n
+                              : (DIR == 1 ? (L % n) + (L / n) * n * n : (L % (n * n)) + (L / (n * n)) * n * n * n);
     if (L >= nlines) continue;
     T x[n], y[n];
 #pragma unroll
-    for (int m = 0; m < n; ++m) x[m] = in[(c * IS + IO) * NI + base + m * s];
+    for (int m = 0; m < n; ++m) x[m] = in[c * NI + base + m * s];
     eo_line<n, ANTI, FORM>(k, x, y);
 #pragma unroll
-    for (int m = 0; m < n; ++m) {
-      if (ACC)
-        out[(c * OS + OO) * NI + base + m * s] += y[m];
-      else
-        out[(c * OS + OO) * NI + base + m * s] = y[m];
-    }
+    for (int m = 0; m < n; ++m) out[(c * OS + OO) * NI + base + m * s] = y[m];
   }
 }
 
@@ -532,6 +496,26 @@ __device__ __forceinline__ void linearised_stress_unit(const T Fi[9], T c1, T rs
 #pragma unroll
     for (int j = 0; j < 3; ++j)
       g[3 * i + j] = fma(K[3 * j + 0], Fi[i], fma(K[3 * j + 1], Fi[3 + i], fma(K[3 * j + 2], Fi[6 + i], dH[3 * i + j])));
+}
+// The two terms added separately: nine more operations, but none waits for the trace before the second
+// product starts.  The FP32 register kernel at two warps a scheduler is faster this way (Q2 64^3
+// cached: 97 us against 109).
+template <typename T>
+__device__ __forceinline__ void linearised_stress_terms(const T Fi[9], T c1, T rs, const T dH[9], T g[9]) {
+  T K[9];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      K[3 * i + j] = fma(Fi[3 * i + 0], dH[j], fma(Fi[3 * i + 1], dH[3 + j], Fi[3 * i + 2] * dH[6 + j]));
+  const T c2 = rs * (K[0] + K[4] + K[8]);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const T Qji = fma(K[3 * j + 0], Fi[i], fma(K[3 * j + 1], Fi[3 + i], K[3 * j + 2] * Fi[6 + i]));
+      g[3 * i + j] = fma(c1, Qji, fma(c2, Fi[3 * j + i], dH[3 * i + j]));
+    }
 }
 // from F^-1 and ln J
 template <typename T>

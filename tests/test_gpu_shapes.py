@@ -75,3 +75,28 @@ def test_chain_ordering(p, N):
     torch.cuda.synchronize()
     assert all(torch.equal(o, want[0]) for o in outs)
     prob.close()
+
+
+@pytest.mark.parametrize("p,N", [(1, 5), (2, 1), (2, 5), (2, 7), (3, 2), (3, 3), (4, 1), (4, 3)])
+@pytest.mark.parametrize("bc,model", [(0, 0), (1, 1), (2, 0)])
+def test_fp32_column_kernel(p, N, bc, model):
+    """FP32 applies on meshes that leave a block's last elements absent, with inclusions, both models
+    and strategies; values on constrained DoFs, even NaN, reach no other row."""
+    import torch
+    nhmf = lib_or_fail()
+    w = workload(p, N, bc)
+    u, du, fac = inp.draw_u(w), inp.draw_du(w), inp.inclusion_factors(N, 10.0)
+    op = Operator(Mesh(N, p), 1.0, 1.5, bc, model=model, factors=fac)
+    ref = op.apply(u, du)
+    fixed = inp.dirichlet_mask(N, p, bc).reshape(-1)
+    du[fixed] = np.nan
+    prob = nhmf.Problem(N, p, 1.0, 1.5, bc, model=model)
+    nhmf.nhmf_set_material_factors(prob.ctx, cuda(fac))
+    prob.set_linearization(cuda(u), 0 if model else nhmf.NHMF_CACHE_FP32)
+    dut = cuda(du).float()
+    for strat in (0,) if model else (0, 1):
+        v = host(prob.apply(dut, torch.full_like(dut, 7.0), nhmf.NHMF_FP32, strat))
+        assert np.isnan(v[fixed]).all()
+        free = ~fixed
+        assert np.linalg.norm(v[free] - ref[free]) <= 1e-5 * np.linalg.norm(ref[free])
+    prob.close()
