@@ -129,11 +129,11 @@ __device__ __forceinline__ void store_local(const OpArgs& a, const float* src, l
 // Forward interpolation of three components to the points: in -> out (tmp is clobbered).
 template <int n, int NI, typename T>
 __device__ __forceinline__ void to_points(const T* sB, T* in, T* tmp, T* out, int nitems) {
-  sf_pass<n, NI, 3, 0, false, false>(sB, in, tmp, nitems);
+  sf_pass<n, NI, 3, 0, false>(sB, in, tmp, nitems);
   __syncthreads();
-  sf_pass<n, NI, 3, 1, false, false>(sB, tmp, in, nitems);
+  sf_pass<n, NI, 3, 1, false>(sB, tmp, in, nitems);
   __syncthreads();
-  sf_pass<n, NI, 3, 2, false, false>(sB, in, out, nitems);
+  sf_pass<n, NI, 3, 2, false>(sB, in, out, nitems);
   __syncthreads();
 }
 
@@ -143,11 +143,11 @@ template <int n, int NI, typename T>
 __device__ __forceinline__ void from_points(const T* sB, const T* sDc, T* G, T* tmp, T* out, int nitems) {
   colloc_grad_T<n, NI>(sDc, G, tmp, nitems);
   __syncthreads();
-  sf_pass<n, NI, 3, 0, true, false>(sB, tmp, G, nitems);
+  sf_pass<n, NI, 3, 0, true>(sB, tmp, G, nitems);
   __syncthreads();
-  sf_pass<n, NI, 3, 1, true, false>(sB, G, tmp, nitems);
+  sf_pass<n, NI, 3, 1, true>(sB, G, tmp, nitems);
   __syncthreads();
-  sf_pass<n, NI, 3, 2, true, false>(sB, tmp, out, nitems);
+  sf_pass<n, NI, 3, 2, true>(sB, tmp, out, nitems);
   __syncthreads();
 }
 

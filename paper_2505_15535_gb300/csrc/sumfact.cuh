@@ -11,6 +11,7 @@
 
 #include <type_traits>
 
+#include "df64.cuh"
 #include "internal.h"
 
 namespace nhmf {
@@ -32,7 +33,6 @@ template <> struct Cfg<2, double> { static constexpr int NE = NHMF_Q2D_NE, THREA
 template <> struct Cfg<3, double> { static constexpr int NE = 8, THREADS = 256; };
 template <> struct Cfg<4, double> { static constexpr int NE = NHMF_Q4D_NE, THREADS = NHMF_Q4D_THREADS; };
 template <> struct Cfg<1, float> { static constexpr int NE = 32, THREADS = 256; };  // p >= 2: ColShape (apply32.cuh)
-struct df64;
 template <int P> struct Cfg<P, df64> : Cfg<P, double> {};
 template <> struct Cfg<4, df64> { static constexpr int NE = 4, THREADS = 256; };
 // Launch shape per strategy: Algorithm 2's point code (120 registers) keeps 256 threads at Q4
@@ -53,7 +53,6 @@ template <> struct LaunchCfg<2, double, NHMF_ON_THE_FLY> {
 // while the others idle.  The line: FP64 cached apply, small / normal blocks, Q2 12^3 40 / 87 us,
 // 24^3 142 / 146, 32^3 312 / 306; Q4 12^3 113 / 119, 32^3 1819 / 1721.  Double-float blocks take
 // less time each: Q2 16^3 50 / 75 us, 24^3 101 / 94; Q4 8^3 49 / 67, 12^3 91 / 87.
-struct df64;
 template <typename T> struct SmallRule { static constexpr int per_sm = 4; };
 template <> struct SmallRule<df64> { static constexpr int per_sm = 2; };
 template <int P> struct SmallCfg;
@@ -204,34 +203,29 @@ __device__ __forceinline__ double elem_factor(const OpArgs& a, long long e_in_co
 }
 
 // One 1D pass along direction DIR over NC arrays of NI items:
-//   out[c][t] (+)= sum_m Mat(r, m) in[c][t with coordinate r along DIR replaced by m]
+//   out[c][t] = sum_m Mat(r, m) in[c][t with coordinate r along DIR replaced by m]
 // with Mat(r, m) = mat[r][m] (TR = false) or mat[m][r] (TR = true).
 // Items t >= nitems (those of absent elements, which come last) are skipped.
-template <int n, int NI, int NC, int DIR, bool TR, bool ACC, typename T>
+template <int n, int NI, int NC, int DIR, bool TR, typename T>
 __device__ __forceinline__ void sf_pass(const T* __restrict__ mat, const T* in, T* out, int nitems = NI) {
   constexpr int s = DIR == 0 ? 1 : (DIR == 1 ? n : n * n);
   for (int t = threadIdx.x; t < nitems; t += blockDim.x) {
     const int r = (t / s) % n;
     const int base = t - r * s;
-    T acc[NC];
+    Acc<T> acc[NC];
     {
       const T c0 = TR ? mat[r] : mat[r * n];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) acc[c] = c0 * in[c * NI + base];
+      for (int c = 0; c < NC; ++c) acc[c].mul(c0, in[c * NI + base]);
     }
 #pragma unroll
     for (int m = 1; m < n; ++m) {
       const T cm = TR ? mat[m * n + r] : mat[r * n + m];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) acc[c] = fma(cm, in[c * NI + base + m * s], acc[c]);
+      for (int c = 0; c < NC; ++c) acc[c].fma(cm, in[c * NI + base + m * s]);
     }
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      if (ACC)
-        out[c * NI + t] += acc[c];
-      else
-        out[c * NI + t] = acc[c];
-    }
+    for (int c = 0; c < NC; ++c) out[c * NI + t] = acc[c].get();
   }
 }
 
@@ -258,37 +252,40 @@ __device__ __forceinline__ void eo_line(const T (&k)[kEoSlots], const T (&x)[n],
   }
 #pragma unroll
   for (int r = 0; r < h; ++r) {
-    T E;
+    Acc<T> E;
     if constexpr (FORM == kEoCentreCol) {
-      E = k[r * h] * e[0];
+      E.mul(k[r * h], e[0]);
 #pragma unroll
-      for (int m = 1; m < h; ++m) E = fma(k[r * h + m], e[m], E);
+      for (int m = 1; m < h; ++m) E.fma(k[r * h + m], e[m]);
     } else {
-      E = k[C0 + r] * x[h];
+      E.mul(k[C0 + r], x[h]);
 #pragma unroll
-      for (int m = 0; m < h; ++m) E = fma(k[r * h + m], e[m], E);
+      for (int m = 0; m < h; ++m) E.fma(k[r * h + m], e[m]);
     }
-    T yp = E, ym = ANTI ? -E : E;
+    Acc<T> yp = E, ym = E;
+    if (ANTI) ym.neg();
 #pragma unroll
     for (int m = 0; m < h; ++m) {
-      yp = fma(k[A0 + r * h + m], o[m], yp);
-      ym = fma(ANTI ? k[A0 + r * h + m] : -k[A0 + r * h + m], o[m], ym);
+      yp.fma(k[A0 + r * h + m], o[m]);
+      ym.fma(ANTI ? k[A0 + r * h + m] : -k[A0 + r * h + m], o[m]);
     }
-    y[r] = yp;
-    y[n - 1 - r] = ym;
+    y[r] = yp.get();
+    y[n - 1 - r] = ym.get();
   }
   if constexpr (ANTI) {
-    T c = k[A0 + h * h] * o[0];
+    Acc<T> c;
+    c.mul(k[A0 + h * h], o[0]);
 #pragma unroll
-    for (int m = 1; m < h; ++m) c = fma(k[A0 + h * h + m], o[m], c);
-    y[h] = c;
+    for (int m = 1; m < h; ++m) c.fma(k[A0 + h * h + m], o[m]);
+    y[h] = c.get();
   } else if constexpr (FORM == kEoCentreRow) {
     y[h] = x[h];
   } else {
-    T c = k[C0 + h] * x[h];
+    Acc<T> c;
+    c.mul(k[C0 + h], x[h]);
 #pragma unroll
-    for (int m = 0; m < h; ++m) c = fma(k[h * h + m], e[m], c);
-    y[h] = c;
+    for (int m = 0; m < h; ++m) c.fma(k[h * h + m], e[m]);
+    y[h] = c.get();
   }
 }
 
@@ -332,18 +329,19 @@ __device__ __forceinline__ void colloc_grad(const T* __restrict__ Dc, const T* v
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const T* vc = val + c * NI;
-    T gx = Dc[rx * n] * vc[bx];
-    T gy = Dc[ry * n] * vc[by];
-    T gz = Dc[rz * n] * vc[bz];
+    Acc<T> gx, gy, gz;
+    gx.mul(Dc[rx * n], vc[bx]);
+    gy.mul(Dc[ry * n], vc[by]);
+    gz.mul(Dc[rz * n], vc[bz]);
 #pragma unroll
     for (int m = 1; m < n; ++m) {
-      gx = fma(Dc[rx * n + m], vc[bx + m], gx);
-      gy = fma(Dc[ry * n + m], vc[by + m * n], gy);
-      gz = fma(Dc[rz * n + m], vc[bz + m * n * n], gz);
+      gx.fma(Dc[rx * n + m], vc[bx + m]);
+      gy.fma(Dc[ry * n + m], vc[by + m * n]);
+      gz.fma(Dc[rz * n + m], vc[bz + m * n * n]);
     }
-    g[c * 3 + 0] = gx;
-    g[c * 3 + 1] = gy;
-    g[c * 3 + 2] = gz;
+    g[c * 3 + 0] = gx.get();
+    g[c * 3 + 1] = gy.get();
+    g[c * 3 + 2] = gz.get();
   }
 }
 
@@ -358,16 +356,17 @@ __device__ __forceinline__ void colloc_grad_T(const T* __restrict__ Dc, const T*
       const T* gx = G + (3 * c + 0) * NI;
       const T* gy = G + (3 * c + 1) * NI;
       const T* gz = G + (3 * c + 2) * NI;
-      T acc = Dc[rx] * gx[bx];
-      acc = fma(Dc[ry], gy[by], acc);
-      acc = fma(Dc[rz], gz[bz], acc);
+      Acc<T> acc;
+      acc.mul(Dc[rx], gx[bx]);
+      acc.fma(Dc[ry], gy[by]);
+      acc.fma(Dc[rz], gz[bz]);
 #pragma unroll
       for (int m = 1; m < n; ++m) {
-        acc = fma(Dc[m * n + rx], gx[bx + m], acc);
-        acc = fma(Dc[m * n + ry], gy[by + m * n], acc);
-        acc = fma(Dc[m * n + rz], gz[bz + m * n * n], acc);
+        acc.fma(Dc[m * n + rx], gx[bx + m]);
+        acc.fma(Dc[m * n + ry], gy[by + m * n]);
+        acc.fma(Dc[m * n + rz], gz[bz + m * n * n]);
       }
-      y[c * NI + t] = acc;
+      y[c * NI + t] = acc.get();
     }
   }
 }
@@ -486,16 +485,27 @@ __device__ __forceinline__ void linearised_stress_unit(const T Fi[9], T c1, T rs
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
-      K[3 * i + j] = fma(Fi[3 * i + 0], dH[j], fma(Fi[3 * i + 1], dH[3 + j], Fi[3 * i + 2] * dH[6 + j]));
+    for (int j = 0; j < 3; ++j) {
+      Acc<T> k;
+      k.mul(Fi[3 * i + 2], dH[6 + j]);
+      k.fma(Fi[3 * i + 1], dH[3 + j]);
+      k.fma(Fi[3 * i + 0], dH[j]);
+      K[3 * i + j] = k.get();
+    }
   const T c2 = rs * (K[0] + K[4] + K[8]);
 #pragma unroll
   for (int k = 0; k < 9; ++k) K[k] = k % 4 == 0 ? fma(c1, K[k], c2) : c1 * K[k];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j)
-      g[3 * i + j] = fma(K[3 * j + 0], Fi[i], fma(K[3 * j + 1], Fi[3 + i], fma(K[3 * j + 2], Fi[6 + i], dH[3 * i + j])));
+    for (int j = 0; j < 3; ++j) {
+      Acc<T> q;
+      q.set(dH[3 * i + j]);
+      q.fma(K[3 * j + 2], Fi[6 + i]);
+      q.fma(K[3 * j + 1], Fi[3 + i]);
+      q.fma(K[3 * j + 0], Fi[i]);
+      g[3 * i + j] = q.get();
+    }
 }
 // The two terms added separately: nine more operations, but none waits for the trace before the second
 // product starts.  The FP32 register kernel at two warps a scheduler is faster this way (Q2 64^3
