@@ -1056,14 +1056,17 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_up_tc(const ConvArgs a, int z
 
 // Weight gradient of the stride-1 gather, tiled: G[tap][a][b] = sum_v P[v][a] Q[v + d_tap][b].
 // A block takes tiles of 128 consecutive positions of one z-plane of an x-strip in x-padded
-// row order (as k_conv_tc) along a column in z.  It stages the tile's P rows and a ring of Q
-// planes (the z - 1 .. z + 1 windows of all taps, zero outside the grid, the neighbouring
-// strip's data in the halo columns) as 16-byte channel halves, so
-// that every 8 x 8 block of a fragment is one ldmatrix: per chunk of 16 positions one
-// ldmatrix.x4.trans gives the A fragment (P^T, channels a x positions) for all the warp's
-// taps, and one per tap gives the B fragments (positions x channels b) of both n-tiles.
-// 9 warps, warp w owns taps 3w..3w+2; per-block partials reduced by k_wgrad_reduce.
-constexpr int kWgThreads = 288;
+// row order (as k_conv_tc) along a column in z.  It stages P rows and Q planes (zero outside
+// the grid, the neighbouring strip's data in the halo columns) as 16-byte channel halves, so
+// that every 8 x 8 block of a fragment is one ldmatrix.  The z-shift of a tap is taken from P and
+// its in-plane shift from Q: Q plane zq meets the P rows of planes zq - dz, so that for a
+// chunk of 16 positions a warp loads three A fragments (P^T of the three planes) and three B
+// fragments (the dx shifts of its dy) for 9 taps, 6 ldmatrix.x4 for 18 MMAs.  With the shifts
+// all on Q a warp took 4 for 6 MMAs, and the shared-memory pipe bounded the kernel.  3 warps, one
+// per dy; per-block partials are reduced by k_wgrad_reduce.
+constexpr int kWgThreads = 288;   // of the stride-2 kernel
+constexpr int kWg1Threads = 96;
+constexpr int kWg1Blocks = 4;     // per SM
 
 __device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -1081,10 +1084,11 @@ __device__ __forceinline__ void frag_channel_sums(uint32_t a0, uint32_t a1, uint
   sg += (__low2float(x0) + __high2float(x0)) + (__low2float(x2) + __high2float(x2));
   sg8 += (__low2float(x1) + __high2float(x1)) + (__low2float(x3) + __high2float(x3));
 }
-// All 9 warps: the block's 16 channel totals (per warp the 4 lanes of each channel, then the
+// All WARPS warps: the block's 16 channel totals (per warp the 4 lanes of each channel, then the
 // warps in order) to bpartial[blockIdx.x][16].  Ends with a block barrier.
+template <int WARPS>
 __device__ __forceinline__ void bias_partial_store(float sg, float sg8, float* bpartial) {
-  __shared__ float bsh[kWgThreads / 32][16];
+  __shared__ float bsh[WARPS][16];
   sg += __shfl_xor_sync(0xffffffffu, sg, 1);
   sg8 += __shfl_xor_sync(0xffffffffu, sg8, 1);
   sg += __shfl_xor_sync(0xffffffffu, sg, 2);
@@ -1098,12 +1102,12 @@ __device__ __forceinline__ void bias_partial_store(float sg, float sg8, float* b
   if (threadIdx.x < 16) {
     float t = 0.f;
 #pragma unroll
-    for (int w = 0; w < kWgThreads / 32; ++w) t += bsh[w][threadIdx.x];
+    for (int w = 0; w < WARPS; ++w) t += bsh[w][threadIdx.x];
     bpartial[blockIdx.x * 16 + threadIdx.x] = t;
   }
 }
 
-size_t wgrad_s1_smem(int W) { return 2 * 2 * 128 * 16 + 4 * 2 * (size_t)(130 + 2 * (W + 2)) * 16; }
+size_t wgrad_s1_smem(int W) { return 4 * 2 * 128 * 16 + 2 * 2 * (size_t)(130 + 2 * (W + 2)) * 16; }
 
 // P rows of a tile, asynchronously: position p0 + j = y R + xl + 1 of plane z in the x-strip
 // of W columns from x0 (zero on the pad columns, past the strip or the grid) to row j of both
@@ -1126,81 +1130,87 @@ __device__ __forceinline__ void wg_stage_rows_async(const __nv_bfloat16* __restr
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-#ifndef NHMF_WG_MINB
-#define NHMF_WG_MINB 4
-#endif
-__global__ void __launch_bounds__(kWgThreads, NHMF_WG_MINB) k_wgrad_s1(const __nv_bfloat16* __restrict__ P,
+__global__ void __launch_bounds__(kWg1Threads, kWg1Blocks) k_wgrad_s1(const __nv_bfloat16* __restrict__ P,
                                                          const __nv_bfloat16* __restrict__ Q, int m, int zc, int W,
                                                          int nstrips, float* partial, float* bpartial) {
   extern __shared__ __align__(128) unsigned char sm[];
   const int R = W + 2, L = 130 + 2 * R;
-  unsigned char* sP0 = sm;                      // [2 buffers][2 halves][128][16 B]
-  unsigned char* sQ = sm + 2 * 2 * 128 * 16;    // [4 slots][2 halves][L][16 B]
-  auto slot = [&](int plane) { return sQ + ((plane + 4) & 3) * 2 * L * 16; };  // plane >= -1
+  unsigned char* sP = sm;                    // [4 slots][2 halves][128][16 B]
+  unsigned char* sQ = sm + 4 * 2 * 128 * 16;  // [2 slots][2 halves][L][16 B]
+  auto pslot = [&](int plane) { return sP + (plane & 3) * 4096; };
+  auto qslot = [&](int plane) { return sQ + (plane & 1) * 2 * L * 16; };
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const int dyi = warp;  // dy + 1
   const int per_plane = (m * R + 127) / 128, nzc = (m + zc - 1) / zc;
   const long long nunits = (long long)per_plane * nstrips * nzc;
-  float acc[3][2][4] = {};
-  unsigned tt = 0;  // tiles done by this block; the P rows of tile tt are in buffer tt & 1
-  float bsg = 0.f, bsg8 = 0.f;  // channels g, g + 8 of P over this warp's share of the chunks (bias gradient)
-  unsigned chunk = 0;            // chunks of 16 positions done by this block; chunk % 9 adds its fragments
+  float acc[3][3][2][4] = {};  // [dz + 1][dx + 1][n-tile]
+  float bsg = 0.f, bsg8 = 0.f;  // channels g, g + 8 of P over this warp's chunks (bias gradient, dy = dz = 0)
   // ldmatrix row of this lane: matrix lane / 8, row lane % 8
   const int lm = lane >> 3, lr = lane & 7;
   for (long long unit = blockIdx.x; unit < nunits; unit += gridDim.x) {
     const int p0 = int(unit % per_plane) * 128;
     const long long rest = unit / per_plane;
     const int x0 = int(rest % nstrips) * W, zb = int(rest / nstrips) * zc, ze = min(m, zb + zc);
-    // planes z - 1 .. z + 1 of Q and the P rows of plane z are in shared memory when tile z
-    // starts; plane z + 2 and the rows of plane z + 1 are copied while tile z computes
-    for (int pl = zb - 1; pl <= zb + 1; ++pl)
-      tc_stage_async(Q, m, R, L, p0 - 1, 1 - x0, 1, pl, slot(pl), threadIdx.x, blockDim.x);
-    wg_stage_rows_async(P, m, R, p0, zb, x0, W, sP0 + (tt & 1u) * 4096);
+    const int q0 = max(zb - 1, 0), q1 = min(ze, m - 1);  // the Q planes that P planes zb .. ze - 1 meet
+    auto stage_p = [&](int z) {
+      if (z >= zb && z < ze) wg_stage_rows_async(P, m, R, p0, z, x0, W, pslot(z));
+    };
+    auto stage_q = [&](int z) { tc_stage_async(Q, m, R, L, p0 - 1, 1 - x0, 1, z, qslot(z), threadIdx.x, blockDim.x); };
+    // Q plane zq and P planes zq - 1 .. zq + 1 are in shared memory when step zq starts; Q plane
+    // zq + 1 and P plane zq + 2 are copied while it computes
+    stage_q(q0);
+    stage_p(q0);
+    stage_p(q0 + 1);
     cp_async_wait_all();
     __syncthreads();
-    for (int z = zb; z < ze; ++z, ++tt) {
-      if (z + 1 < ze) {
-        tc_stage_async(Q, m, R, L, p0 - 1, 1 - x0, 1, z + 2, slot(z + 2), threadIdx.x, blockDim.x);
-        wg_stage_rows_async(P, m, R, p0, z + 1, x0, W, sP0 + ((tt + 1) & 1u) * 4096);
-      }
-      const uint32_t sp = smem_u32(sP0 + (tt & 1u) * 4096);
+    for (int zq = q0; zq <= q1; ++zq) {
+      if (zq < q1) stage_q(zq + 1);
+      stage_p(zq + 2);
+      const uint32_t sq = smem_u32(qslot(zq));
+      bool on[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) on[d] = zq - (d - 1) >= zb && zq - (d - 1) < ze;
+#pragma unroll 4
       for (int c = 0; c < 8; ++c) {
         // A = P^T on positions 16c..16c+15: matrices (k 0-7, a lo), (k 0-7, a hi), (k 8-15, a lo), (k 8-15, a hi)
-        uint32_t a0, a1, a2, a3;
-        ldsm_x4_trans(sp + (uint32_t)(((lm & 1) * 128 + 16 * c + (lm >> 1) * 8 + lr) * 16), a0, a1, a2, a3);
+        uint32_t a[3][4];
 #pragma unroll
-        for (int jt = 0; jt < 3; ++jt) {
-          const int tap = 3 * warp + jt;
-          const int dx = tap % 3 - 1, dy = (tap / 3) % 3 - 1, dz = tap / 9 - 1;
-          const int row = R + 1 + dx + dy * R + 16 * c;  // staged row of position 16c of plane z + dz
+        for (int d = 0; d < 3; ++d)
+          if (on[d])
+            ldsm_x4_trans(smem_u32(pslot(zq - (d - 1))) + (uint32_t)(((lm & 1) * 128 + 16 * c + (lm >> 1) * 8 + lr) * 16),
+                          a[d][0], a[d][1], a[d][2], a[d][3]);
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          const int row = R + 1 + (dx - 1) + (dyi - 1) * R + 16 * c;  // staged row of position 16c
           // B: matrices (k 0-7, b lo), (k 8-15, b lo), (k 0-7, b hi), (k 8-15, b hi)
           uint32_t b0, b1, b2, b3;
-          ldsm_x4_trans(smem_u32(slot(z + dz)) + (uint32_t)(((lm >> 1) * L + row + (lm & 1) * 8 + lr) * 16), b0, b1,
-                        b2, b3);
-          mma16816(acc[jt][0], a0, a1, a2, a3, b0, b1);
-          mma16816(acc[jt][1], a0, a1, a2, a3, b2, b3);
+          ldsm_x4_trans(sq + (uint32_t)(((lm >> 1) * L + row + (lm & 1) * 8 + lr) * 16), b0, b1, b2, b3);
+#pragma unroll
+          for (int d = 0; d < 3; ++d)
+            if (on[d]) {
+              mma16816(acc[d][dx][0], a[d][0], a[d][1], a[d][2], a[d][3], b0, b1);
+              mma16816(acc[d][dx][1], a[d][0], a[d][1], a[d][2], a[d][3], b2, b3);
+            }
         }
-        // the bias gradient's share, after the MMAs have consumed the fragment
-        if (bpartial && chunk % (kWgThreads / 32) == (unsigned)warp) frag_channel_sums(a0, a1, a2, a3, bsg, bsg8);
-        ++chunk;
+        if (bpartial && dyi == 1 && on[1]) frag_channel_sums(a[1][0], a[1][1], a[1][2], a[1][3], bsg, bsg8);
       }
       cp_async_wait_all();
       __syncthreads();
     }
   }
-  if (bpartial) bias_partial_store(bsg, bsg8, bpartial);
+  if (bpartial) bias_partial_store<kWg1Threads / 32>(bsg, bsg8, bpartial);
   float* out = partial + (long long)blockIdx.x * 27 * 256;
 #pragma unroll
-  for (int jt = 0; jt < 3; ++jt) {
-    const int tap = 3 * warp + jt;
+  for (int d = 0; d < 3; ++d)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int b = 8 * h + 2 * t;
-      out[tap * 256 + g * 16 + b] = acc[jt][h][0];
-      out[tap * 256 + g * 16 + b + 1] = acc[jt][h][1];
-      out[tap * 256 + (g + 8) * 16 + b] = acc[jt][h][2];
-      out[tap * 256 + (g + 8) * 16 + b + 1] = acc[jt][h][3];
-    }
-  }
+    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int tap = 9 * d + 3 * dyi + dx, ar = g + 8 * (i >> 1), bc = 8 * h + 2 * t + (i & 1);
+          out[tap * 256 + ar * 16 + bc] = acc[d][dx][h][i];
+        }
 }
 
 // Weight gradient of the stride-2 gather (the down-convolution), tiled like k_wgrad_s1:
@@ -1315,7 +1325,7 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_s2(const __nv_bfloat16* __
       __syncthreads();
     }
   }
-  if (bpartial) bias_partial_store(bsg, bsg8, bpartial);
+  if (bpartial) bias_partial_store<kWgThreads / 32>(bsg, bsg8, bpartial);
   float* out = partial + (long long)blockIdx.x * 27 * 256;
 #pragma unroll
   for (int jt = 0; jt < 3; ++jt) {
@@ -1457,9 +1467,13 @@ void wgrad(UNet& u, int layer, int gather, const __nv_bfloat16* P, int mp, const
     const size_t smem = wgrad_s1_smem(W);
     cudaFuncSetAttribute(k_wgrad_s1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const long long per_plane = ((long long)mp * (W + 2) + 127) / 128;
-    const int zc = wave_column(per_plane * nstrips, mp, kWgBlocks, 1, 4);
-    blocks = (int)std::min<long long>(kWgBlocks, per_plane * nstrips * ((mp + zc - 1) / zc));
-    k_wgrad_s1<<<blocks, kWgThreads, smem, s>>>(P, Q, mp, zc, W, nstrips, u.partial, bpart);
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const long long slots = std::min<long long>(kWgBlocks, (long long)kWg1Blocks * std::max(nsm, 1));
+    const int zc = wave_column(per_plane * nstrips, mp, slots, 1, 4);
+    blocks = (int)std::min<long long>(slots, per_plane * nstrips * ((mp + zc - 1) / zc));
+    k_wgrad_s1<<<blocks, kWg1Threads, smem, s>>>(P, Q, mp, zc, W, nstrips, u.partial, bpart);
   } else {  // stride 2: P on the coarse grid, Q on the fine grid
     int nseg = 0;
     const int seg = wgrad_s2_seg(mp, &nseg);
