@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(ColShape<P + 1>::THREADS, ColShape<P + 1>::BLO
   static_assert(kTile % NE == 0, "a block's elements lie in one tile of vloc");
   extern __shared__ __align__(16) float F[];  // [9][n][NE][n][n], then the point state
   const int tid = threadIdx.x;
+  pdl_launch_next();
   const long long e0 = (long long)blockIdx.x * NE;
   const int nvalid = (int)min((long long)NE, a.col.count - e0);
 
@@ -262,6 +263,7 @@ __global__ void __launch_bounds__(ColShape<P + 1>::THREADS, ColShape<P + 1>::BLO
   const long long node = gi + (long long)a.M * (P * ey + cy + (long long)a.M * gk);
   const float fac = a.factor ? float(a.factor[el]) : 1.f;
   bool bad = false;
+  pdl_wait();
 
   if constexpr (STRAT == NHMF_ON_THE_FLY) {
     if (column) {

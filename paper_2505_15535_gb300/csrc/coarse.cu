@@ -166,6 +166,17 @@ struct CgArgs {
   unsigned long long* words;         // [0] += iterations, [1] |= status flags
 };
 
+// x / y rounded to T.  In FP32 the quotient's 48 good bits of one Newton step decide the rounding as
+// the FP64 division does but for ties nearer than 2^-47, at half its latency.
+template <typename T>
+__device__ __forceinline__ T quotient(double x, double y) {
+  if constexpr (sizeof(T) == 4) {
+    const float yf = float(y);
+    if (fabsf(yf) > 1e-30f && fabsf(yf) < 1e30f) return T(x * fast_rcp(y));
+  }
+  return T(x / y);
+}
+
 // Jacobi-CG from x = 0 to ||r|| <= rtol ||b||, tested every `check` iterations as pcg() does;
 // p.q <= 0 or a non-finite residual is recorded in the status word and ends the solve.  One
 // cluster; block `rank` owns rows [rank R, rank R + R).  All warps of a block form q = A p; warp 0
@@ -260,15 +271,44 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
   const int vrows = (rows * kLanes + 31) / 32 * 32;
   // The loop's exit is block-uniform (`stop`) and the same in every block (it depends on the
   // cluster's sums alone).
+  // A block whose rows all have their own lanes keeps them, and their column offsets, in registers.
+  constexpr int kPart = (kRow + kLanes - 1) / kLanes;
+  const bool own = vrows <= nthr;
+  T ar[kPart];
+  int ao[kPart];
+  if (own && rows > 0) {
+    const int row = min(tid / kLanes, rows - 1), node = (row0 + row) % M3;
+#pragma unroll
+    for (int u = 0; u < kPart; ++u) {
+      const int j = tid % kLanes + u * kLanes;
+      ar[u] = j < kRow ? A[j * Rpad + row] : T(0);
+      ao[u] = node + off[min(j, kRow - 1)];
+    }
+  }
   while (k < a.maxit && !*stop) {
-    for (int i = tid; i < vrows; i += nthr) {
-      const int row = min(i / kLanes, rows - 1), node = (row0 + row) % M3;
-      T s = T(0);
+    if (own) {
+      if (tid < vrows) {
+        T s = T(0), s1 = T(0);
+#pragma unroll
+        for (int u = 0; u < kPart; u += 2) {
+          s = fma(ar[u], p[ao[u]], s);
+          if (u + 1 < kPart) s1 = fma(ar[u + 1], p[ao[u + 1]], s1);
+        }
+        s += s1;
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (tid % kLanes == 0 && tid / kLanes < rows) q[tid / kLanes] = s;
+      }
+    } else {
+      for (int i = tid; i < vrows; i += nthr) {
+        const int row = min(i / kLanes, rows - 1), node = (row0 + row) % M3;
+        T s = T(0);
 #pragma unroll 7
-      for (int j = i % kLanes; j < kRow; j += kLanes) s = fma(A[j * Rpad + row], p[node + off[j]], s);
-      s += __shfl_xor_sync(0xffffffffu, s, 1);
-      s += __shfl_xor_sync(0xffffffffu, s, 2);
-      if (i % kLanes == 0 && i / kLanes < rows) q[row] = s;
+        for (int j = i % kLanes; j < kRow; j += kLanes) s = fma(A[j * Rpad + row], p[node + off[j]], s);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (i % kLanes == 0 && i / kLanes < rows) q[row] = s;
+      }
     }
     ++k;
     __syncthreads();
@@ -278,7 +318,7 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
     sum2(v0, v1);
     const bool ok = v0 > 0.0 && isfinite(v0);  // warp 0
     if (tid < 32) {
-      const T alpha = ok ? T(rz / v0) : T(0);
+      const T alpha = ok ? quotient<T>(rz, v0) : T(0);
       v0 = v1 = 0.0;
       for (int i = tid; i < rows; i += 32) {
         x[i] = fma(alpha, p[row0 + i], x[i]);
@@ -301,7 +341,7 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
       if (end) {
         if (tid == 0) *stop = 1;
       } else {
-        const T beta = T(v0 / rz);
+        const T beta = quotient<T>(v0, rz);
         rz = v0;
         for (int i = tid; i < rows; i += 32) set_p(i, fma(beta, p[row0 + i], q[i]));
       }

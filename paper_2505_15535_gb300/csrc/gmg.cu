@@ -7,6 +7,7 @@
 // Each level is a context of its own (same degree, material and boundary preset), so every
 // operator kernel of the library serves every level.  The 3D transfers are tensor products
 // of 1D maps applied as three passes.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -15,6 +16,7 @@
 #include "blas.h"
 #include "gmg.h"
 #include "internal.h"
+#include "sumfact.cuh"
 
 namespace nhmf {
 namespace {
@@ -34,6 +36,8 @@ __global__ void __launch_bounds__(256) k_map1d(const T* __restrict__ in, T* __re
                                                int nz, int mout, const int* __restrict__ ptr,
                                                const int* __restrict__ col, const T* __restrict__ w, bool add, int bc) {
   const int ox = dir == 0 ? mout : nx, oy = dir == 1 ? mout : ny, oz = dir == 2 ? mout : nz;
+  pdl_launch_next();
+  pdl_wait();
   const int ij = blockIdx.x * 256 + threadIdx.x, k = blockIdx.y, c = blockIdx.z;
   if (ij >= ox * oy) return;
   const int j = ij / ox, i = ij - j * ox, row = dir == 0 ? i : (dir == 1 ? j : k);
@@ -60,6 +64,8 @@ __global__ void __launch_bounds__(256) k_map1d(const T* __restrict__ in, T* __re
 template <typename T>
 __global__ void k_cheb(long long n, const T* __restrict__ b, const T* __restrict__ q, const T* __restrict__ dinv,
                        T* __restrict__ d, T* __restrict__ x, T c_old, T c_new) {
+  pdl_launch_next();
+  pdl_wait();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const T r = q ? b[i] - q[i] : b[i];
     const T di = c_old == T(0) ? c_new * dinv[i] * r : fma(c_old, d[i], c_new * dinv[i] * r);
@@ -98,6 +104,23 @@ __global__ void k_to(long long n, const double* __restrict__ x, T* __restrict__ 
 }
 
 constexpr int kB = 1216, kT = 256;
+unsigned ew_blocks(long long n) { return (unsigned)std::min<long long>(kB, (n + kT - 1) / kT); }
+
+// A launch whose blocks may be scheduled while the launch before it drains (the kernel waits for that
+// one before it reads): the V-cycle is a chain of short kernels on the coarse levels.
+template <typename KernelT, typename... Args>
+void launch_chained(KernelT kernel, dim3 grid, int threads, cudaStream_t s, Args... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, args...);  // an error is the caller's next cudaGetLastError
+}
 
 // ------------------------------------------------------------------ host helpers
 double lagrange(const double* z, int n, int i, double x) {
@@ -187,10 +210,14 @@ template <> const float* wts<float>(const Map1D& m) { return m.w32; }
 template <typename T>
 void map3d(const Map1D& m, const T* in, T* out, T* t1, T* t2, cudaStream_t s, bool add = false, int bc = NHMF_BC_NONE) {
   const int mi = m.cols, mo = m.rows;
-  auto grid = [](int ox, int oy, int oz) { return dim3((unsigned)((ox * oy + 255) / 256), (unsigned)oz, 3u); };
-  k_map1d<T><<<grid(mo, mi, mi), 256, 0, s>>>(in, t1, 0, mi, mi, mi, mo, m.ptr, m.col, wts<T>(m), false, NHMF_BC_NONE);
-  k_map1d<T><<<grid(mo, mo, mi), 256, 0, s>>>(t1, t2, 1, mo, mi, mi, mo, m.ptr, m.col, wts<T>(m), false, NHMF_BC_NONE);
-  k_map1d<T><<<grid(mo, mo, mo), 256, 0, s>>>(t2, out, 2, mo, mo, mi, mo, m.ptr, m.col, wts<T>(m), add, bc);
+  auto pass = [&](const T* src, T* dst, int dir, int nx, int ny, int nz, bool a, int b) {
+    const int ox = dir == 0 ? mo : nx, oy = dir == 1 ? mo : ny, oz = dir == 2 ? mo : nz;
+    launch_chained(k_map1d<T>, dim3((unsigned)((ox * oy + 255) / 256), (unsigned)oz, 3u), 256, s, src, dst, dir, nx, ny,
+                   nz, mo, (const int*)m.ptr, (const int*)m.col, wts<T>(m), a, b);
+  };
+  pass(in, t1, 0, mi, mi, mi, false, NHMF_BC_NONE);
+  pass(t1, t2, 1, mo, mi, mi, false, NHMF_BC_NONE);
+  pass(t2, out, 2, mo, mo, mi, add, bc);
 }
 
 }  // namespace
@@ -427,7 +454,7 @@ nhmf_status chebyshev(GmgLevel& L, int strat, const T* b, T* x, int degree, doub
     }
     // d = c_old d + c_new D^-1 (b - A x), x += d, with A x = 0 in the first step from zero
     if (first && zero_start) {
-      k_cheb<T><<<kB, kT, 0, s>>>(L.n, b, nullptr, Buf<T>::dinv(L), d, x, c_old, c_new);
+      launch_chained(k_cheb<T>, dim3(ew_blocks(L.n)), kT, s, L.n, b, (const T*)nullptr, Buf<T>::dinv(L), d, x, c_old, c_new);
     } else if constexpr (sizeof(T) == 4) {
       Gather32 g;
       g.mode = Gather32::kChebyshev;
@@ -439,7 +466,7 @@ nhmf_status chebyshev(GmgLevel& L, int strat, const T* b, T* x, int degree, doub
       if ((st = launch_apply32(L.ctx, strat, x, x, g, s)) != NHMF_OK) return st;
     } else {
       if ((st = launch_apply(L.ctx, Buf<T>::prec, strat, x, q, s)) != NHMF_OK) return st;
-      k_cheb<T><<<kB, kT, 0, s>>>(L.n, b, q, Buf<T>::dinv(L), d, x, c_old, c_new);
+      launch_chained(k_cheb<T>, dim3(ew_blocks(L.n)), kT, s, L.n, b, (const T*)q, Buf<T>::dinv(L), d, x, c_old, c_new);
     }
   }
   return cuda_check(L.ctx, cudaGetLastError(), "chebyshev");

@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
   T* G = Vq + 3 * NI;                           // [9][NI] gradients, then fluxes; G[0..2] gathers
 
   pdl_launch_next();
+  if constexpr (std::is_same<T, float>::value) pdl_wait();  // one launch: nothing of it may run ahead
   load_apply_tables<P>(a, tab);
   const long long e0 = (long long)blockIdx.x * NE;
   const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
@@ -364,6 +365,8 @@ constexpr int kRegThreads = NHMF_REG_THREADS;  // threads (= elements) per block
 template <int P, int STRAT, int MODEL>
 __global__ void __launch_bounds__(kRegThreads, NHMF_REG_MINB) k_apply_reg(const OpArgs a) {
   constexpr int n = P + 1, n3 = n * n * n;
+  pdl_launch_next();
+  pdl_wait();
   const long long ec = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (ec >= a.col.count) return;
   const Colour& col = a.col;
@@ -592,6 +595,7 @@ __global__ void __launch_bounds__(256) k_gather_local(const float* __restrict__ 
                                                      int M, int bc, const Gather32 g32) {
   constexpr int n = P + 1, n3 = n * n * n;
   static_assert(kTile == 32, "tile index by shift and mask");
+  pdl_launch_next();
   // grid: x covers the M^2 nodes of one z-plane, y the plane (32-bit index arithmetic; the
   // launcher keeps the element count below 2^31)
   const int ij = blockIdx.x * blockDim.x + threadIdx.x;
@@ -600,6 +604,7 @@ __global__ void __launch_bounds__(256) k_gather_local(const float* __restrict__ 
   const int g[3] = {ij - gj * M, gj, (int)blockIdx.y};
   const long long node = ij + (long long)M * M * blockIdx.y, M3 = (long long)M * M * M;
   const unsigned long long done_pol = l2_evict_first();  // each element-local value is read once
+  pdl_wait();
   // per direction: the element below the node (local index P), if any, then the element at or
   // above it (local index g % P); an absent element in x gets a clamped (valid) index and is
   // masked after the load
@@ -1212,13 +1217,16 @@ nhmf_status run_local(nhmf_ctx* c, KernelT kernel, OpArgs a, int NE, int threads
   }
   a.col = c->g.all;
   a.vloc = c->vloc;
-  kernel<<<(unsigned)((c->g.E + NE - 1) / NE), threads, smem, s>>>(a);
+  // both launches may start while the one before them drains (they wait for it before they read)
+  cudaError_t e = launch(kernel, dim3((unsigned)((c->g.E + NE - 1) / NE)), threads, smem, s, true, a);
+  if (e != cudaSuccess) return cuda_check(c, e, "apply");
   const dim3 gather_grid((unsigned)(((long long)c->g.M * c->g.M + 255) / 256), (unsigned)c->g.M);
   auto* gather = g32.mode == Gather32::kApply       ? k_gather_local<P, Gather32::kApply>
                  : g32.mode == Gather32::kResidual  ? k_gather_local<P, Gather32::kResidual>
                  : g32.mode == Gather32::kChebyshev ? k_gather_local<P, Gather32::kChebyshev>
                                                     : k_gather_local<P, Gather32::kPower>;
-  gather<<<gather_grid, 256, 0, s>>>(c->vloc, du, v, c->g.N, c->g.M, a.bc, g32);
+  e = launch(gather, gather_grid, 256, 0, s, true, (const float*)c->vloc, du, v, c->g.N, c->g.M, a.bc, g32);
+  if (e != cudaSuccess) return cuda_check(c, e, "apply");
   if (c->profiling) {
     cudaEventRecord(rec.b, s);
     c->prof.push_back(rec);
