@@ -16,7 +16,7 @@
 #include "blas.h"
 #include "gmg.h"
 #include "internal.h"
-#include "sumfact.cuh"
+#include "pdl.cuh"
 
 namespace nhmf {
 namespace {
@@ -105,22 +105,6 @@ __global__ void k_to(long long n, const double* __restrict__ x, T* __restrict__ 
 
 constexpr int kB = 1216, kT = 256;
 unsigned ew_blocks(long long n) { return (unsigned)std::min<long long>(kB, (n + kT - 1) / kT); }
-
-// A launch whose blocks may be scheduled while the launch before it drains (the kernel waits for that
-// one before it reads): the V-cycle is a chain of short kernels on the coarse levels.
-template <typename KernelT, typename... Args>
-void launch_chained(KernelT kernel, dim3 grid, int threads, cudaStream_t s, Args... args) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, args...);  // an error is the caller's next cudaGetLastError
-}
 
 // ------------------------------------------------------------------ host helpers
 double lagrange(const double* z, int n, int i, double x) {
@@ -212,7 +196,7 @@ void map3d(const Map1D& m, const T* in, T* out, T* t1, T* t2, cudaStream_t s, bo
   const int mi = m.cols, mo = m.rows;
   auto pass = [&](const T* src, T* dst, int dir, int nx, int ny, int nz, bool a, int b) {
     const int ox = dir == 0 ? mo : nx, oy = dir == 1 ? mo : ny, oz = dir == 2 ? mo : nz;
-    launch_chained(k_map1d<T>, dim3((unsigned)((ox * oy + 255) / 256), (unsigned)oz, 3u), 256, s, src, dst, dir, nx, ny,
+    launch(k_map1d<T>, dim3((unsigned)((ox * oy + 255) / 256), (unsigned)oz, 3u), 256, 0, s, true, src, dst, dir, nx, ny,
                    nz, mo, (const int*)m.ptr, (const int*)m.col, wts<T>(m), a, b);
   };
   pass(in, t1, 0, mi, mi, mi, false, NHMF_BC_NONE);
@@ -454,7 +438,7 @@ nhmf_status chebyshev(GmgLevel& L, int strat, const T* b, T* x, int degree, doub
     }
     // d = c_old d + c_new D^-1 (b - A x), x += d, with A x = 0 in the first step from zero
     if (first && zero_start) {
-      launch_chained(k_cheb<T>, dim3(ew_blocks(L.n)), kT, s, L.n, b, (const T*)nullptr, Buf<T>::dinv(L), d, x, c_old, c_new);
+      launch(k_cheb<T>, dim3(ew_blocks(L.n)), kT, 0, s, true, L.n, b, (const T*)nullptr, Buf<T>::dinv(L), d, x, c_old, c_new);
     } else if constexpr (sizeof(T) == 4) {
       Gather32 g;
       g.mode = Gather32::kChebyshev;
@@ -466,7 +450,7 @@ nhmf_status chebyshev(GmgLevel& L, int strat, const T* b, T* x, int degree, doub
       if ((st = launch_apply32(L.ctx, strat, x, x, g, s)) != NHMF_OK) return st;
     } else {
       if ((st = launch_apply(L.ctx, Buf<T>::prec, strat, x, q, s)) != NHMF_OK) return st;
-      launch_chained(k_cheb<T>, dim3(ew_blocks(L.n)), kT, s, L.n, b, (const T*)q, Buf<T>::dinv(L), d, x, c_old, c_new);
+      launch(k_cheb<T>, dim3(ew_blocks(L.n)), kT, 0, s, true, L.n, b, (const T*)q, Buf<T>::dinv(L), d, x, c_old, c_new);
     }
   }
   return cuda_check(L.ctx, cudaGetLastError(), "chebyshev");

@@ -1139,24 +1139,6 @@ cudaError_t prepare(KernelT kernel, size_t smem) {
   return cudaSuccess;
 }
 
-// One launch; with `pdl` by programmatic dependent launch, so that its blocks may start once every
-// block of the launch before it has started (and must not touch that launch's output before
-// pdl_wait).
-template <typename KernelT, typename... Args>
-cudaError_t launch(KernelT kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, bool pdl, Args... args) {
-  cudaLaunchAttribute attr{};
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = &attr;
-  cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 // Runs `kernel` once per colour class with NE elements per block, after k_init_rows on `out` if
 // given (null: the kernel writes no nodal vector).  The classes are chained by programmatic
 // dependent launch: everything before a class's scatter depends on no other class, so its blocks

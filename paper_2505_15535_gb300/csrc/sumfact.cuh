@@ -13,6 +13,7 @@
 
 #include "df64.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace nhmf {
 
@@ -159,12 +160,6 @@ __device__ __forceinline__ void st_policy(float* a, float v, unsigned long long 
   *a = v;
 #endif
 }
-// Programmatic dependent launch: let the stream's next launch start once every block of this one
-// has started; wait until the launches before this one are complete and their writes visible.
-// Both do nothing where a kernel is launched without the attribute.
-__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 __device__ __forceinline__ bool is_constrained(int bc, int c, int gi, int gk, int M) {
   if (bc == NHMF_BC_CLAMP_X0) return gi == 0;
   if (bc == NHMF_BC_COMPRESSION) return gk == 0 || (c == 2 && gk == M - 1);

@@ -24,6 +24,7 @@
 
 #include "blas.h"
 #include "internal.h"
+#include "pdl.cuh"
 #include "unet.h"
 
 namespace nhmf {
@@ -69,6 +70,8 @@ struct ConvArgs {
 // partials [nblocks][16] the same way.
 __global__ void __launch_bounds__(1024) k_wgrad_reduce(const float* partial, const float* bpartial, int nblocks,
                                                        float* grad_w, float* grad_b, int kind, int cin, int cout) {
+  pdl_launch_next();
+  pdl_wait();
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   __shared__ float sh[32][33];
   if (blockIdx.x == 27 * 256 / 32) {  // the bias block
@@ -106,6 +109,8 @@ __global__ void __launch_bounds__(1024) k_wgrad_reduce(const float* partial, con
 // Per-block channel sums of P [voxel][16] (the bias gradient's partials): a thread adds whole
 // 32-byte voxel rows, then the block adds its threads' sums in a fixed order.
 __global__ void __launch_bounds__(256) k_bgrad_partial(const __nv_bfloat16* P, long long nvox, float* partial) {
+  pdl_launch_next();
+  pdl_wait();
   float s[16];
 #pragma unroll
   for (int ch = 0; ch < 16; ++ch) s[ch] = 0.f;
@@ -143,6 +148,8 @@ __global__ void __launch_bounds__(256) k_bgrad_partial(const __nv_bfloat16* P, l
 
 // grad_b[ch] = sum over the partial blocks, in a fixed order (one block of 256 threads).
 __global__ void __launch_bounds__(256) k_bgrad_reduce(const float* partial, int nblocks, float* grad_b, int cout) {
+  pdl_launch_next();
+  pdl_wait();
   const int ch = threadIdx.x & 15, g = threadIdx.x >> 4;
   float r = 0.f;
   for (int b = g; b < nblocks; b += 16) r += partial[b * 16 + ch];
@@ -606,6 +613,8 @@ __device__ __forceinline__ void tma_load5(uint32_t dst, const CUtensorMap* map, 
 
 __global__ void __launch_bounds__(kTcSThreads) k_conv_tc(const ConvArgs a, const __grid_constant__ CUtensorMap map,
                                                          int zc, int W, int nstrips, unsigned* status) {
+  pdl_launch_next();
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char sm[];
   const int m = a.m_out, R = W + 2, NY = tma_ny(R);
   const uint32_t H = tma_h(R);
@@ -811,6 +820,8 @@ size_t down_tc_smem(int W) {
 
 __global__ void __launch_bounds__(kTcSThreads) k_down_tc(const ConvArgs a, int zc, int W, int nstrips,
                                                          unsigned* status) {
+  pdl_launch_next();
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char sm[];
   const int mo = a.m_out, mi = a.m_in, R = W + 2, L = R + 129;
   const uint32_t slot_bytes = 4u * 2u * (uint32_t)L * 16u;
@@ -950,6 +961,8 @@ size_t up_tc_smem(int mi) {
 }
 
 __global__ void __launch_bounds__(kTcThreads, 4) k_up_tc(const ConvArgs a, int zc, unsigned* status) {
+  pdl_launch_next();
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char sm[];
   const int mi = a.m_in, mo = a.m_out, R = mi + 1, L = 129 + R;
   unsigned char* sB = sm;
@@ -1062,7 +1075,11 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_up_tc(const ConvArgs a, int z
 // its in-plane shift from Q: Q plane zq meets the P rows of planes zq - dz, so that for a
 // chunk of 16 positions a warp loads three A fragments (P^T of the three planes) and three B
 // fragments (the dx shifts of its dy) for 9 taps, 6 ldmatrix.x4 for 18 MMAs.  With the shifts
-// all on Q a warp took 4 for 6 MMAs, and the shared-memory pipe bounded the kernel.  3 warps, one
+// all on Q a warp took 4 for 6 MMAs, and the shared-memory pipe bounded the kernel (129^3: 140 us
+// a launch, now 121); mma.sync issue bounds it, one m16n8k16 in 4.6 clocks of an SM.  So the
+// layers with three channels on one side take the MMAs of their eight-channel tile only (NT =
+// 1): the input layer has them on Q; the output layer has them on P and swaps the operands,
+// G[tap][a][b] = sum_v Q[v][b] P[v - d_tap][a] (SWAP: rows are b, tap 26 - tap).  3 warps, one
 // per dy; per-block partials are reduced by k_wgrad_reduce.
 constexpr int kWgThreads = 288;   // of the stride-2 kernel
 constexpr int kWg1Threads = 96;
@@ -1071,6 +1088,10 @@ constexpr int kWg1Blocks = 4;     // per SM
 __device__ __forceinline__ void ldsm_x4_trans(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
+}
+
+__device__ __forceinline__ void ldsm_x2_trans(uint32_t addr, uint32_t& r0, uint32_t& r1) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
 }
 
 // Bias-gradient share of an A fragment (P^T, channels x 16 positions, m16n8k16 layout): lane
@@ -1130,9 +1151,12 @@ __device__ __forceinline__ void wg_stage_rows_async(const __nv_bfloat16* __restr
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
+template <int NT, bool SWAP>
 __global__ void __launch_bounds__(kWg1Threads, kWg1Blocks) k_wgrad_s1(const __nv_bfloat16* __restrict__ P,
                                                          const __nv_bfloat16* __restrict__ Q, int m, int zc, int W,
                                                          int nstrips, float* partial, float* bpartial) {
+  pdl_launch_next();
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char sm[];
   const int R = W + 2, L = 130 + 2 * R;
   unsigned char* sP = sm;                    // [4 slots][2 halves][128][16 B]
@@ -1143,7 +1167,7 @@ __global__ void __launch_bounds__(kWg1Threads, kWg1Blocks) k_wgrad_s1(const __nv
   const int dyi = warp;  // dy + 1
   const int per_plane = (m * R + 127) / 128, nzc = (m + zc - 1) / zc;
   const long long nunits = (long long)per_plane * nstrips * nzc;
-  float acc[3][3][2][4] = {};  // [dz + 1][dx + 1][n-tile]
+  float acc[3][3][NT][4] = {};  // [dz + 1][dx + 1][n-tile]
   float bsg = 0.f, bsg8 = 0.f;  // channels g, g + 8 of P over this warp's chunks (bias gradient, dy = dz = 0)
   // ldmatrix row of this lane: matrix lane / 8, row lane % 8
   const int lm = lane >> 3, lr = lane & 7;
@@ -1183,13 +1207,17 @@ __global__ void __launch_bounds__(kWg1Threads, kWg1Blocks) k_wgrad_s1(const __nv
         for (int dx = 0; dx < 3; ++dx) {
           const int row = R + 1 + (dx - 1) + (dyi - 1) * R + 16 * c;  // staged row of position 16c
           // B: matrices (k 0-7, b lo), (k 8-15, b lo), (k 0-7, b hi), (k 8-15, b hi)
-          uint32_t b0, b1, b2, b3;
-          ldsm_x4_trans(sq + (uint32_t)(((lm >> 1) * L + row + (lm & 1) * 8 + lr) * 16), b0, b1, b2, b3);
+          uint32_t b[4];
+          if constexpr (NT == 2)
+            ldsm_x4_trans(sq + (uint32_t)(((lm >> 1) * L + row + (lm & 1) * 8 + lr) * 16), b[0], b[1], b[2], b[3]);
+          else
+            ldsm_x2_trans(sq + (uint32_t)((row + (lm & 1) * 8 + lr) * 16), b[0], b[1]);
 #pragma unroll
           for (int d = 0; d < 3; ++d)
             if (on[d]) {
-              mma16816(acc[d][dx][0], a[d][0], a[d][1], a[d][2], a[d][3], b0, b1);
-              mma16816(acc[d][dx][1], a[d][0], a[d][1], a[d][2], a[d][3], b2, b3);
+#pragma unroll
+              for (int h = 0; h < NT; ++h)
+                mma16816(acc[d][dx][h], a[d][0], a[d][1], a[d][2], a[d][3], b[2 * h], b[2 * h + 1]);
             }
         }
         if (bpartial && dyi == 1 && on[1]) frag_channel_sums(a[1][0], a[1][1], a[1][2], a[1][3], bsg, bsg8);
@@ -1205,11 +1233,14 @@ __global__ void __launch_bounds__(kWg1Threads, kWg1Blocks) k_wgrad_s1(const __nv
 #pragma unroll
     for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+      for (int h = 0; h < NT; ++h)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int tap = 9 * d + 3 * dyi + dx, ar = g + 8 * (i >> 1), bc = 8 * h + 2 * t + (i & 1);
-          out[tap * 256 + ar * 16 + bc] = acc[d][dx][h][i];
+          if constexpr (SWAP)
+            out[(26 - tap) * 256 + bc * 16 + ar] = acc[d][dx][h][i];
+          else
+            out[tap * 256 + ar * 16 + bc] = acc[d][dx][h][i];
         }
 }
 
@@ -1235,6 +1266,8 @@ size_t wgrad_s2_smem(int seg) { return 2 * 2 * (size_t)seg * 16 + kW2Slots * 2 *
 __global__ void __launch_bounds__(kWgThreads) k_wgrad_s2(const __nv_bfloat16* __restrict__ P, int mp,
                                                          const __nv_bfloat16* __restrict__ Q, int mq, int seg,
                                                          int nseg, int zc, float* partial, float* bpartial) {
+  pdl_launch_next();
+  pdl_wait();
   extern __shared__ __align__(128) unsigned char sm[];
   const int Wf = 2 * seg + 1, hs = 3 * Wf * 16;  // bytes per staged fine half
   unsigned char* sP0 = sm;                        // [2 buffers][2 halves][seg][16 B]
@@ -1371,7 +1404,7 @@ void up_tc_launch(const ConvArgs& a, unsigned* status, cudaStream_t s) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   const long long slots = 4ll * std::max(nsm, 1);  // 4 blocks per SM (launch bounds, TMEM)
-  k_up_tc<<<(int)std::min<long long>(nunits, slots), kTcThreads, smem, s>>>(a, zc, status);
+  launch(k_up_tc, dim3((unsigned)std::min<long long>(nunits, slots)), kTcThreads, smem, s, true, a, zc, status);
 }
 
 typedef CUresult (*TensorMapEncodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -1420,7 +1453,8 @@ void conv_tc_launch(const ConvArgs& a, unsigned* status, cudaStream_t s) {
   const long long slots = (long long)std::max(1, std::min(4, smem_sm / (int)(smem + 1024))) * std::max(nsm, 1);
   const int zc = wave_column(per_plane * nstrips, m, slots, 1, 4);  // z + 2 planes per column
   const long long nunits = per_plane * nstrips * ((m + zc - 1) / zc);
-  k_conv_tc<<<(int)std::min<long long>(nunits, slots), kTcSThreads, smem, s>>>(a, map, zc, W, nstrips, status);
+  launch(k_conv_tc, dim3((unsigned)std::min<long long>(nunits, slots)), kTcSThreads, smem, s, true, a, map, zc, W,
+         nstrips, status);
 }
 
 // A stride-2 convolution on tcgen05 (k_down_tc): x-strips of at most kDnStripMax coarse
@@ -1439,7 +1473,8 @@ void down_tc_launch(const ConvArgs& a, unsigned* status, cudaStream_t s) {
   const long long slots = (long long)std::max(1, std::min(4, smem_sm / (int)(smem + 1024))) * std::max(nsm, 1);
   const int zc = wave_column(per_plane * nstrips, mo, slots, 2, 3);  // 2 z + 1 planes per column
   const long long nunits = per_plane * nstrips * ((mo + zc - 1) / zc);
-  k_down_tc<<<(int)std::min<long long>(nunits, slots), kTcSThreads, smem, s>>>(a, zc, W, nstrips, status);
+  launch(k_down_tc, dim3((unsigned)std::min<long long>(nunits, slots)), kTcSThreads, smem, s, true, a, zc, W, nstrips,
+         status);
 }
 
 // out = act(conv_G(in; w) + bias + add) * mask
@@ -1456,7 +1491,7 @@ void conv(int gather, const __nv_bfloat16* in, int m_in, const __nv_bfloat16* w,
 }
 
 // Weight gradient of `layer`; with bias_from_p also its bias gradient (the channel sums of P,
-// the layer's output gradient), from the same kernel.
+// the layer's output gradient), from the same kernel (not where the operands are swapped).
 void wgrad(UNet& u, int layer, int gather, const __nv_bfloat16* P, int mp, const __nv_bfloat16* Q, int mq,
            bool bias_from_p, cudaStream_t s) {
   float* bpart = bias_from_p ? u.partial + (long long)kWgBlocks * 27 * 256 : nullptr;
@@ -1465,7 +1500,10 @@ void wgrad(UNet& u, int layer, int gather, const __nv_bfloat16* P, int mp, const
     int nstrips = 0;
     const int W = conv_strip_width(mp, &nstrips);
     const size_t smem = wgrad_s1_smem(W);
-    cudaFuncSetAttribute(k_wgrad_s1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const UNetLayer& L = u.L[layer];
+    const bool swap = L.cout <= 8;  // three output channels: the operands change sides
+    auto* kernel = swap ? k_wgrad_s1<1, true> : L.cin <= 8 ? k_wgrad_s1<1, false> : k_wgrad_s1<2, false>;
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const long long per_plane = ((long long)mp * (W + 2) + 127) / 128;
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
@@ -1473,7 +1511,8 @@ void wgrad(UNet& u, int layer, int gather, const __nv_bfloat16* P, int mp, const
     const long long slots = std::min<long long>(kWgBlocks, (long long)kWg1Blocks * std::max(nsm, 1));
     const int zc = wave_column(per_plane * nstrips, mp, slots, 1, 4);
     blocks = (int)std::min<long long>(slots, per_plane * nstrips * ((mp + zc - 1) / zc));
-    k_wgrad_s1<<<blocks, kWg1Threads, smem, s>>>(P, Q, mp, zc, W, nstrips, u.partial, bpart);
+    launch(kernel, dim3((unsigned)blocks), kWg1Threads, smem, s, true, swap ? Q : P, swap ? P : Q, mp, zc, W, nstrips,
+           u.partial, swap ? (float*)nullptr : bpart);
   } else {  // stride 2: P on the coarse grid, Q on the fine grid
     int nseg = 0;
     const int seg = wgrad_s2_seg(mp, &nseg);
@@ -1482,18 +1521,20 @@ void wgrad(UNet& u, int layer, int gather, const __nv_bfloat16* P, int mp, const
     const long long per_plane = (long long)mp * nseg;
     const int zc = (int)std::max<long long>(1, std::min<long long>(kTcZ, per_plane * mp / kTcUnits));
     blocks = (int)std::min<long long>(kWgBlocks, per_plane * ((mp + zc - 1) / zc));
-    k_wgrad_s2<<<blocks, kWgThreads, smem, s>>>(P, mp, Q, mq, seg, nseg, zc, u.partial, bpart);
+    launch(k_wgrad_s2, dim3((unsigned)blocks), kWgThreads, smem, s, true, P, mp, Q, mq, seg, nseg, zc, u.partial, bpart);
   }
   const UNetLayer& L = u.L[layer];
-  k_wgrad_reduce<<<27 * 256 / 32 + (bias_from_p ? 1 : 0), 1024, 0, s>>>(
-      u.partial, bpart, blocks, u.grads + L.woff, bias_from_p ? u.grads + L.boff : nullptr, L.kind, L.cin, L.cout);
+  launch(k_wgrad_reduce, dim3(27 * 256 / 32 + (bias_from_p ? 1 : 0)), 1024, 0, s, true, (const float*)u.partial,
+         (const float*)bpart, blocks, u.grads + L.woff, bias_from_p ? u.grads + L.boff : (float*)nullptr, L.kind, L.cin,
+         L.cout);
 }
 
 void bgrad(UNet& u, int layer, const __nv_bfloat16* P, long long nvox, cudaStream_t s) {
   const int blocks = (int)std::min<long long>(kBgBlocks, (nvox + 255) / 256);
   float* part = u.partial + (long long)kWgBlocks * 27 * 256;
-  k_bgrad_partial<<<blocks, 256, 0, s>>>(P, nvox, part);
-  k_bgrad_reduce<<<1, 256, 0, s>>>(part, blocks, u.grads + u.L[layer].boff, u.L[layer].cout);
+  launch(k_bgrad_partial, dim3((unsigned)blocks), 256, 0, s, true, P, nvox, part);
+  launch(k_bgrad_reduce, dim3(1), 256, 0, s, true, (const float*)part, blocks, u.grads + u.L[layer].boff,
+         u.L[layer].cout);
 }
 
 }  // namespace
@@ -1599,7 +1640,8 @@ void unet_backward(UNet& u, cudaStream_t s) {
   __nv_bfloat16 *dy = u.g0a, *dt0 = u.g0b, *du0 = u.g0c, *ds0 = u.g0a;
   __nv_bfloat16 *dt1 = u.g1a, *du1 = u.g1b, *ds1 = u.g1c, *dd1 = u.g1a;
   __nv_bfloat16 *dm2 = u.g2a, *dd2 = u.g2b;
-  wgrad(u, L_OUT, S1, dy, M0, u.t0, M0, true, s);
+  wgrad(u, L_OUT, S1, dy, M0, u.t0, M0, false, s);
+  bgrad(u, L_OUT, dy, u.N0, s);
   conv(S1, dy, M0, u.L[L_OUT].wb, nullptr, nullptr, u.t0, false, dt0, nullptr, M0, s, u.status);
   wgrad(u, L_T0, S1, dt0, M0, u.u0, M0, true, s);
   conv(S1, dt0, M0, u.L[L_T0].wb, nullptr, nullptr, u.u0, false, du0, nullptr, M0, s, u.status);
