@@ -669,7 +669,9 @@ __global__ void __launch_bounds__(256) k_gather_local(const float* __restrict__ 
 }
 
 // ------------------------------------------------------------------ point cache
-template <int P, bool SMALL>
+// SPATIAL: Algorithm 2's 36 values as well (compiled apart: its code takes the registers that let
+// a second and third block hide the plain cache's latencies).
+template <int P, bool SMALL, bool SPATIAL>
 __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS) k_cache(const OpArgs a) {
   using T = double;
   constexpr int n = P + 1, n3 = n * n * n, NE = Shape<P, T, NHMF_CACHED, SMALL>::NE, NI = NE * n3;
@@ -701,7 +703,7 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
       for (int k = 0; k < 9; ++k) a.cache64_out[k * a.nq + cbase + t] = Fi[k];
       a.cache64_out[9 * a.nq + cbase + t] = lnJ;
     }
-    if (a.cachesp_out) {
+    if constexpr (SPATIAL) {
       // Algorithm 2 cache from the model's P and dP only: tau = P F^T;
       // J a_ijkl = (dP[e_k (x) F_l.] F^T)_ij, J c_ijkl = J a_ijkl - delta_ik tau_jl
       double F[9];
@@ -889,7 +891,9 @@ __device__ __forceinline__ void diag_line(const double* const (&tab)[NIN], const
   for (int k = 0; k < n; ++k) out[k * s] = y[k];
 }
 
-template <int P, bool SMALL>
+// CACHED: F^-1 and ln J come from the FP64 point cache of the linearisation point (compressible
+// model), which saves a third of the operations (u's values, gradient and kinematics).
+template <int P, bool SMALL, bool CACHED>
 __global__ void __launch_bounds__(DiagCfg<P, SMALL>::THREADS) k_diagonal(const OpArgs a) {
   using T = double;
   constexpr int n = P + 1, n3 = n * n * n, NE = DiagCfg<P, SMALL>::NE, NI = NE * n3, NL = NE * n * n;
@@ -918,24 +922,40 @@ __global__ void __launch_bounds__(DiagCfg<P, SMALL>::THREADS) k_diagonal(const O
   const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
   const int nitems = nvalid * n3, nlines = nvalid * n * n;
   for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = a.h * elem_factor(a, e0 + min(e, nvalid - 1));
-  gather<P, NI>(a, a.u64, e0, nvalid, false, X);
-  __syncthreads();
-  if constexpr (EO) {
-    eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, X, Vq, nlines);
+  if constexpr (!CACHED) {
+    gather<P, NI>(a, a.u64, e0, nvalid, false, X);
     __syncthreads();
-    eo_pass<n, NI, 3, 1, false, kEoCentreRow, TH>(kB, Vq, X, nlines);
-    __syncthreads();
-    eo_pass<n, NI, 3, 2, false, kEoCentreRow, TH>(kB, X, Vq, nlines);
-    __syncthreads();
-  } else {
-    to_points<n, NI>(sB, X, Vq, Vq, nitems);
+    if constexpr (EO) {
+      eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, X, Vq, nlines);
+      __syncthreads();
+      eo_pass<n, NI, 3, 1, false, kEoCentreRow, TH>(kB, Vq, X, nlines);
+      __syncthreads();
+      eo_pass<n, NI, 3, 2, false, kEoCentreRow, TH>(kB, X, Vq, nlines);
+      __syncthreads();
+    } else {
+      to_points<n, NI>(sB, X, Vq, Vq, nitems);
+    }
   }
+  const double* cache = static_cast<const double*>(a.cache) + (a.col.slot0 + e0) * n3;
+  const unsigned long long pol = l2_evict_first();
   for (int t = threadIdx.x; t < nitems; t += blockDim.x) {
     T H[9];
-    colloc_grad<n, NI>(sDch, Vq, t, H);
-    const Kinematics<T> kin(H);
+    // the matrix f whose entries enter L twice, and the factor that makes f f the product of F^-1's
+    T f9[9], kap;
+    Kinematics<T> kin;
+    if constexpr (CACHED) {
+#pragma unroll
+      for (int k = 0; k < 9; ++k) f9[k] = ld_policy(cache + k * a.nq + t, pol);
+      kap = fma(2.0 * a.lam, 1.0 - ld_policy(cache + 9 * a.nq + t, pol), a.mu);
+    } else {
+      colloc_grad<n, NI>(sDch, Vq, t, H);
+      kin = Kinematics<T>(H);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) f9[k] = kin.A[k];
+      kap = fma(2.0 * a.lam, 1.0 - kin.lnJ, a.mu) * (kin.invJ * kin.invJ);
+    }
     const int pd[6] = {0, 0, 0, 1, 1, 2}, pl[6] = {0, 1, 2, 1, 2, 2};
-    if (a.model == NHMF_MODEL_SPLIT) {
+    if (!CACHED && a.model == NHMF_MODEL_SPLIT) {
       // L_cdcl = mu a d_dl - 2/3 mu a (F_cd Fi_lc + Fi_dc F_cl) + (2/9 mu a I1 + kappa J^2
       //          + mu a I1/3 - kappa/2 (J^2 - 1)) Fi_dc Fi_lc
       const T J = 1.0 + kin.Jm1, J2 = J * J, mua = a.mu * exp(-2.0 / 3.0 * kin.lnJ);
@@ -957,13 +977,12 @@ __global__ void __launch_bounds__(DiagCfg<P, SMALL>::THREADS) k_diagonal(const O
                                      cff * Fidc * Filc;
         }
     } else {
-      const T kap = fma(2.0 * a.lam, 1.0 - kin.lnJ, a.mu) * (kin.invJ * kin.invJ);  // the adjugate enters twice
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         T f[3], kf[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-          f[d] = kin.A[3 * d + c];
+          f[d] = f9[3 * d + c];
           kf[d] = kap * f[d];
         }
 #pragma unroll
@@ -1304,12 +1323,12 @@ nhmf_status apply_dispatch_p(nhmf_ctx* c, int prec, int strat, const void* du, v
                               : apply_p<P, float, NHMF_ON_THE_FLY>(c, du, v, raw, g32, s);
 }
 
-template <int P, bool SMALL>
+template <int P, bool SMALL, bool SPATIAL>
 nhmf_status cache_shape(nhmf_ctx* c, const OpArgs& a, cudaStream_t s) {
   using Sh = Shape<P, double, NHMF_CACHED, SMALL>;
   constexpr int n3 = (P + 1) * (P + 1) * (P + 1);
   const size_t smem = (kTabSlots + 6 * (size_t)Sh::NE * n3) * sizeof(double);
-  return run_colours<double>(c, k_cache<P, SMALL>, a, Sh::NE, Sh::THREADS, smem, nullptr, nullptr, 0.0, s,
+  return run_colours<double>(c, k_cache<P, SMALL, SPATIAL>, a, Sh::NE, Sh::THREADS, smem, nullptr, nullptr, 0.0, s,
                              "cache build", NHMF_KIND_CACHE);
 }
 
@@ -1321,8 +1340,9 @@ nhmf_status cache_p(nhmf_ctx* c, cudaStream_t s) {
   a.cache32_out = c->cache32;
   a.cachedf_out = c->cachedf;
   a.cachesp_out = c->cachesp;
-  return small_blocks<double, Shape<P, double, NHMF_CACHED, false>::NE>(c) ? cache_shape<P, true>(c, a, s)
-                                                                   : cache_shape<P, false>(c, a, s);
+  const bool small = small_blocks<double, Shape<P, double, NHMF_CACHED, false>::NE>(c);
+  if (c->cachesp) return small ? cache_shape<P, true, true>(c, a, s) : cache_shape<P, false, true>(c, a, s);
+  return small ? cache_shape<P, true, false>(c, a, s) : cache_shape<P, false, false>(c, a, s);
 }
 
 template <int P, bool SMALL>
@@ -1343,12 +1363,12 @@ nhmf_status residual_p(nhmf_ctx* c, const double* u, double* r, cudaStream_t s) 
                                                          : residual_shape<P, false>(c, a, r, s);
 }
 
-template <int P, bool SMALL>
+template <int P, bool SMALL, bool CACHED>
 nhmf_status diagonal_shape(nhmf_ctx* c, const OpArgs& a, double* d, cudaStream_t s) {
   using Sh = DiagCfg<P, SMALL>;
   constexpr int n3 = (P + 1) * (P + 1) * (P + 1);
   const size_t smem = (kTabSlots + kDiagFields * (size_t)Sh::NE * n3) * sizeof(double);
-  return run_colours<double>(c, k_diagonal<P, SMALL>, a, Sh::NE, Sh::THREADS, smem, nullptr, d, 1.0, s, "diagonal",
+  return run_colours<double>(c, k_diagonal<P, SMALL, CACHED>, a, Sh::NE, Sh::THREADS, smem, nullptr, d, 1.0, s, "diagonal",
                              NHMF_KIND_DIAGONAL);
 }
 
@@ -1357,8 +1377,12 @@ nhmf_status diagonal_p(nhmf_ctx* c, double* d, cudaStream_t s) {
   OpArgs a = base_args(c);
   a.u64 = c->ubar;
   a.v = d;
-  return small_blocks<double, DiagCfg<P, false>::NE>(c) ? diagonal_shape<P, true>(c, a, d, s)
-                                                : diagonal_shape<P, false>(c, a, d, s);
+  // the FP64 cache, where it exists, holds the current linearisation point (set_linearization)
+  a.cache = c->cache64;
+  const bool small = small_blocks<double, DiagCfg<P, false>::NE>(c);
+  if (c->cache64 && c->prm.model == NHMF_MODEL_COMPRESSIBLE)
+    return small ? diagonal_shape<P, true, true>(c, a, d, s) : diagonal_shape<P, false, true>(c, a, d, s);
+  return small ? diagonal_shape<P, true, false>(c, a, d, s) : diagonal_shape<P, false, false>(c, a, d, s);
 }
 
 }  // namespace

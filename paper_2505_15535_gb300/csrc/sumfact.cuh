@@ -415,6 +415,7 @@ __device__ __forceinline__ float fast_log1p(float x, float) { return log1pf(x); 
 template <typename T>
 struct Kinematics {
   T A[9], invJ, lnJ, Jm1;
+  __device__ __forceinline__ Kinematics() {}
   __device__ __forceinline__ explicit Kinematics(const T H[9]) {
     const T F0 = T(1) + H[0], F4 = T(1) + H[4], F8 = T(1) + H[8];
     const T C = fma(-H[5], H[7], fma(H[4], F8, H[8]));  // C00 - 1

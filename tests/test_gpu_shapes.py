@@ -40,7 +40,10 @@ def test_block_shapes(p, N, bc):
     for prec, strat in ((0, 0), (0, 1), (0, 2), (2, 1)):
         check(prob.apply(dut, torch.full_like(dut, np.nan), prec, strat), ref)
     check(prob.residual(cuda(u), torch.full_like(dut, np.nan)), op.residual_rows(u, rows))
-    check(prob.diagonal(torch.full_like(dut, np.nan)), op.diagonal_rows(u, rows))
+    diag = op.diagonal_rows(u, rows)
+    check(prob.diagonal(torch.full_like(dut, np.nan)), diag)   # from the point cache
+    prob.set_linearization(cuda(u), 0)
+    check(prob.diagonal(torch.full_like(dut, np.nan)), diag)   # from u
     prob.close()
 
 
