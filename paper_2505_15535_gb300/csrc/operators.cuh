@@ -61,14 +61,14 @@ __device__ __forceinline__ void load_apply_tables(const OpArgs& a, T* tab, const
 // optionally zeroing constrained DoFs and scaling by a per-element factor fac[e]; items of
 // absent elements are zero.
 template <int P, int NI, typename TS, typename T>
-__device__ __forceinline__ void gather(const OpArgs& a, const TS* __restrict__ src, long long e0,
+__device__ __forceinline__ void gather(const OpArgs& a, const Colour& col, const TS* __restrict__ src, long long e0,
                                        int nvalid, bool mask, T* dst, const T* fac = nullptr) {
   constexpr int n3 = (P + 1) * (P + 1) * (P + 1);
   for (int t = threadIdx.x; t < NI; t += blockDim.x) {
     const int e = t / n3;
     if (e < nvalid) {
       int gi, gj, gk;
-      item_node<P>(a, e0 + e, t % n3, gi, gj, gk);
+      item_node<P>(col, e0 + e, t % n3, gi, gj, gk);
       const long long node = gi + (long long)a.M * (gj + (long long)a.M * gk);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
@@ -100,7 +100,7 @@ __device__ __forceinline__ void scatter_add(const OpArgs& a, const T* src, long 
     const int e = t / n3;
     if (e >= nvalid) continue;
     int gi, gj, gk;
-    item_node<P>(a, e0 + e, t % n3, gi, gj, gk);
+    item_node<P>(a.col, e0 + e, t % n3, gi, gj, gk);
     const long long node = gi + (long long)a.M * (gj + (long long)a.M * gk);
 #pragma unroll
     for (int c = 0; c < 3; ++c)
@@ -203,17 +203,18 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
   pdl_launch_next();
   if constexpr (std::is_same<T, float>::value) pdl_wait();  // one launch: nothing of it may run ahead
   load_apply_tables<P>(a, tab);
+  const Colour& col = a.col;
   const long long e0 = (long long)blockIdx.x * NE;
-  const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
+  const int nvalid = (int)min((long long)NE, (long long)col.count - e0);
   const int nitems = nvalid * n3, nlines = nvalid * n * n;  // items / lines of present elements
-  for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = T(elem_factor(a, e0 + min(e, nvalid - 1)));
+  for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = T(elem_factor(a, col, e0 + min(e, nvalid - 1)));
   __syncthreads();
 
   if constexpr (STRAT == NHMF_ON_THE_FLY) {
     if (sizeof(T) == 8)
-      gather<P, NI>(a, a.u64, e0, nvalid, false, G);
+      gather<P, NI>(a, col, a.u64, e0, nvalid, false, G);
     else
-      gather<P, NI>(a, a.u32, e0, nvalid, false, G);
+      gather<P, NI>(a, col, a.u32, e0, nvalid, false, G);
     __syncthreads();
     if constexpr (EO) {
       eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, G, Vq, nlines);
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
       to_points<n, NI>(sB, G, Vq, U, nitems);
     }
   }
-  gather<P, NI>(a, static_cast<const typename Store<T>::type*>(a.du), e0, nvalid, true, G,
+  gather<P, NI>(a, col, static_cast<const typename Store<T>::type*>(a.du), e0, nvalid, true, G,
                 a.factor ? (const T*)sF : nullptr);
   __syncthreads();
   if constexpr (EO) {
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
 
   const T inv_mu = T(1.0 / a.mu), r2 = T(a.r2mu);
   const typename Store<T>::type* cache = static_cast<const typename Store<T>::type*>(a.cache);
-  const long long cbase = (a.col.slot0 + e0) * n3;
+  const long long cbase = (col.slot0 + e0) * n3;
   bool bad = false;
   for (int t = threadIdx.x; t < nitems; t += blockDim.x) {
     T dH[9], g[9];
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
           for (int k = 0; k < 9; ++k) Fi[k] = T(ld_policy(cache + k * a.nq + cbase + t, pol));
           lnJ = T(ld_policy(cache + 9 * a.nq + cbase + t, pol));
         } else {
-          const long long slot = a.col.slot0 + e0 + t / n3, q = t % n3;
+          const long long slot = col.slot0 + e0 + t / n3, q = t % n3;
           const auto* tile = cache + (slot / kTile) * (10 * n3 * kTile) + slot % kTile;
 #pragma unroll
           for (int k = 0; k < 9; ++k) Fi[k] = T(tile[(k * n3 + q) * kTile]);
@@ -453,7 +454,7 @@ __global__ void __launch_bounds__(kRegThreads, NHMF_REG_MINB) k_apply_reg(const 
           qv[c][idx(i, j, k)] = fixed ? 0.f : du[c * a.M3 + node(i, j, k)];
         }
   if (a.factor) {
-    const float fac = float(elem_factor(a, ec));
+    const float fac = float(elem_factor(a, col, ec));
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
@@ -682,16 +683,16 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
   T* sW = sD + kMaxN * kMaxN;
   T* A = sB + kTabSlots;  // [3][NI]
   T* Vq = A + 3 * NI;     // [3][NI]
-  pdl_launch_next();
   load_tables<P>(a, sB, sDc, sD, sW, 1.0);
   __syncthreads();
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) sDc[i] = a.Dch[i];  // physical gradients
-  const long long e0 = (long long)blockIdx.x * NE;
-  const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
-  gather<P, NI>(a, a.u64, e0, nvalid, false, A);
+  long long e0;
+  const Colour col = block_colour<NE>(a.N, e0);  // one launch: the classes are independent here
+  const int nvalid = (int)min((long long)NE, (long long)col.count - e0);
+  gather<P, NI>(a, col, a.u64, e0, nvalid, false, A);
   __syncthreads();
   to_points<n, NI>(sB, A, Vq, Vq, nvalid * n3);
-  const long long cbase = (a.col.slot0 + e0) * n3;
+  const long long cbase = (col.slot0 + e0) * n3;
   bool bad = false;
   for (int t = threadIdx.x; t < nvalid * n3; t += blockDim.x) {
     double H[9], Fi[9], lnJ;
@@ -751,7 +752,7 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
     }
     if (a.cache32_out) {
       // the FP32 applies run over all elements in natural order (element-local results)
-      const long long en = elem_natural(a, e0 + t / n3), q = t % n3;
+      const long long en = elem_natural(a, col, e0 + t / n3), q = t % n3;
       if (P <= kRegMaxP && a.reg32) {
         // element tiles [E/32][10][n^3][32] for the register kernel (one thread per element)
         float* tile = a.cache32_out + (en / kTile) * (10 * n3 * kTile) + en % kTile;
@@ -767,7 +768,6 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
     }
   }
   if (bad) atomicOr(a.status, kStatusNonPosJ);
-  pdl_wait();  // the last class is complete only when all are
 }
 
 // ------------------------------------------------------------------ residual
@@ -789,11 +789,12 @@ __global__ void __launch_bounds__(Shape<P, double, 0, SMALL>::THREADS) k_residua
   T* G = Vq + 3 * NI;                  // [9][NI] gradients, then fluxes
   pdl_launch_next();
   load_apply_tables<P>(a, tab, a.eoh);
+  const Colour& col = a.col;
   const long long e0 = (long long)blockIdx.x * NE;
-  const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
+  const int nvalid = (int)min((long long)NE, (long long)col.count - e0);
   const int nitems = nvalid * n3, nlines = nvalid * n * n;
-  for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = a.h * elem_factor(a, e0 + min(e, nvalid - 1));
-  gather<P, NI>(a, a.u64, e0, nvalid, false, G);
+  for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = a.h * elem_factor(a, col, e0 + min(e, nvalid - 1));
+  gather<P, NI>(a, col, a.u64, e0, nvalid, false, G);
   __syncthreads();
   if constexpr (EO) {
     eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, G, Vq, nlines);
@@ -908,22 +909,23 @@ __global__ void __launch_bounds__(DiagCfg<P, SMALL>::THREADS) k_diagonal(const O
   T* Vq = X + 18 * NI;    // [3][NI]
   pdl_launch_next();
   for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
-    const T b = a.B[i], d = a.D[i], w = a.w[i / n];
+    const T b = a.B[i], d = a.D[i], wq = a.w[i / n];
     sB[i] = b;
     sDch[i] = a.Dch[i];
-    tBB[i] = w * b * b;
-    tBD[i] = w * b * d;
-    tDD[i] = w * d * d;
-    t2BB[i] = 2.0 * (w * b * b);
-    t2BD[i] = 2.0 * (w * b * d);
+    tBB[i] = wq * b * b;
+    tBD[i] = wq * b * d;
+    tDD[i] = wq * d * d;
+    t2BB[i] = 2.0 * (wq * b * b);
+    t2BD[i] = 2.0 * (wq * b * d);
   }
   for (int i = threadIdx.x; i < kEoSlots; i += blockDim.x) kB[i] = a.eo[0][i];
+  const Colour& col = a.col;
   const long long e0 = (long long)blockIdx.x * NE;
-  const int nvalid = (int)min((long long)NE, (long long)a.col.count - e0);
+  const int nvalid = (int)min((long long)NE, (long long)col.count - e0);
   const int nitems = nvalid * n3, nlines = nvalid * n * n;
-  for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = a.h * elem_factor(a, e0 + min(e, nvalid - 1));
+  for (int e = threadIdx.x; e < NE; e += blockDim.x) sF[e] = a.h * elem_factor(a, col, e0 + min(e, nvalid - 1));
   if constexpr (!CACHED) {
-    gather<P, NI>(a, a.u64, e0, nvalid, false, X);
+    gather<P, NI>(a, col, a.u64, e0, nvalid, false, X);
     __syncthreads();
     if constexpr (EO) {
       eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, X, Vq, nlines);
@@ -936,7 +938,7 @@ __global__ void __launch_bounds__(DiagCfg<P, SMALL>::THREADS) k_diagonal(const O
       to_points<n, NI>(sB, X, Vq, Vq, nitems);
     }
   }
-  const double* cache = static_cast<const double*>(a.cache) + (a.col.slot0 + e0) * n3;
+  const double* cache = static_cast<const double*>(a.cache) + (col.slot0 + e0) * n3;
   const unsigned long long pol = l2_evict_first();
   for (int t = threadIdx.x; t < nitems; t += blockDim.x) {
     T H[9];
@@ -1158,8 +1160,8 @@ cudaError_t prepare(KernelT kernel, size_t smem) {
   return cudaSuccess;
 }
 
-// Runs `kernel` once per colour class with NE elements per block, after k_init_rows on `out` if
-// given (null: the kernel writes no nodal vector).  The classes are chained by programmatic
+// Runs `kernel` once per colour class with NE elements per block, after k_init_rows on `out`.  The
+// classes are chained by programmatic
 // dependent launch: everything before a class's scatter depends on no other class, so its blocks
 // fill the SMs that the classes before it leave idle, and it waits for those classes only before
 // it adds to `out`.  FP64 cached apply against plain launches: Q1 8^3 140 -> 30 us and Q2 16^3
@@ -1169,14 +1171,11 @@ template <typename T, typename KernelT>
 nhmf_status run_colours(nhmf_ctx* c, KernelT kernel, OpArgs a, int NE, int threads, size_t smem, const T* src, T* out,
                         T value, cudaStream_t s, const char* what, int kind) {
   if (cudaError_t e = prepare(kernel, smem); e != cudaSuccess) return cuda_check(c, e, what);
-  bool pdl = false;
-  if (out) {
-    const long long M2 = (long long)c->g.M * c->g.M;
-    const dim3 grid((unsigned)((M2 + 256 * kInitPer - 1) / (256 * kInitPer)), (unsigned)(3 * c->g.M));
-    if (cudaError_t e = launch(k_init_rows<T>, grid, 256, 0, s, false, a.bc, c->g.M, src, out, value); e != cudaSuccess)
-      return cuda_check(c, e, what);
-    pdl = !c->profiling;  // the event below lies between the two launches
-  }
+  const long long M2 = (long long)c->g.M * c->g.M;
+  const dim3 init_grid((unsigned)((M2 + 256 * kInitPer - 1) / (256 * kInitPer)), (unsigned)(3 * c->g.M));
+  if (cudaError_t e = launch(k_init_rows<T>, init_grid, 256, 0, s, false, a.bc, c->g.M, src, out, value); e != cudaSuccess)
+    return cuda_check(c, e, what);
+  bool pdl = !c->profiling;  // the event below lies between the two launches
   nhmf_ctx::Rec rec{kind, 0, nullptr, nullptr};
   if (c->profiling) {
     cudaEventCreate(&rec.a);
@@ -1328,8 +1327,22 @@ nhmf_status cache_shape(nhmf_ctx* c, const OpArgs& a, cudaStream_t s) {
   using Sh = Shape<P, double, NHMF_CACHED, SMALL>;
   constexpr int n3 = (P + 1) * (P + 1) * (P + 1);
   const size_t smem = (kTabSlots + 6 * (size_t)Sh::NE * n3) * sizeof(double);
-  return run_colours<double>(c, k_cache<P, SMALL, SPATIAL>, a, Sh::NE, Sh::THREADS, smem, nullptr, nullptr, 0.0, s,
-                             "cache build", NHMF_KIND_CACHE);
+  auto* kernel = k_cache<P, SMALL, SPATIAL>;
+  if (cudaError_t e = prepare(kernel, smem); e != cudaSuccess) return cuda_check(c, e, "cache build");
+  nhmf_ctx::Rec rec{NHMF_KIND_CACHE, 1, nullptr, nullptr};
+  if (c->profiling) {
+    cudaEventCreate(&rec.a);
+    cudaEventCreate(&rec.b);
+    cudaEventRecord(rec.a, s);
+  }
+  long long blocks = 0;
+  for (int k = 0; k < 8; ++k) blocks += (c->g.colour[k].count + Sh::NE - 1) / Sh::NE;
+  const cudaError_t e = launch(kernel, dim3((unsigned)blocks), Sh::THREADS, smem, s, false, a);
+  if (c->profiling) {
+    cudaEventRecord(rec.b, s);
+    c->prof.push_back(rec);
+  }
+  return cuda_check(c, e, "cache build");
 }
 
 template <int P>

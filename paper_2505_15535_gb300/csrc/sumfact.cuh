@@ -166,12 +166,32 @@ __device__ __forceinline__ bool is_constrained(int bc, int c, int gi, int gk, in
   return false;
 }
 
+// A block's colour class and first element in it, for a launch whose blocks (NE elements each) cover all
+// eight classes.  The classes are laid out as build_geometry (api.cu) does: class cx + 2 cy + 4 cz
+// holds the elements of these parities, slots in class order.
+template <int NE>
+__device__ __forceinline__ Colour block_colour(int N, long long& e0) {
+  Colour c;
+  c.stride = 2;
+  c.slot0 = 0;
+  long long first = 0;
+  for (int k = 0;; ++k) {
+    c.cx = k & 1, c.cy = (k >> 1) & 1, c.cz = k >> 2;
+    c.nx = (N + 1 - c.cx) / 2, c.ny = (N + 1 - c.cy) / 2, c.nz = (N + 1 - c.cz) / 2;
+    c.count = c.nx * c.ny * c.nz;
+    const long long blocks = (c.count + NE - 1) / NE;
+    if (k == 7 || blockIdx.x < first + blocks) break;
+    first += blocks;
+    c.slot0 += c.count;
+  }
+  e0 = ((long long)blockIdx.x - first) * NE;
+  return c;
+}
+
 // Global node of work item t (element t / n^3 of this block, local point/node t % n^3).
 template <int P>
-__device__ __forceinline__ void item_node(const OpArgs& a, long long e_in_colour, int q, int& gi,
-                                          int& gj, int& gk) {
+__device__ __forceinline__ void item_node(const Colour& c, long long e_in_colour, int q, int& gi, int& gj, int& gk) {
   constexpr int n = P + 1;
-  const Colour& c = a.col;
   const int ix = int(e_in_colour % c.nx);
   const int iy = int((e_in_colour / c.nx) % c.ny);
   const int iz = int(e_in_colour / ((long long)c.nx * c.ny));
@@ -180,21 +200,16 @@ __device__ __forceinline__ void item_node(const OpArgs& a, long long e_in_colour
   gk = P * (c.cz + c.stride * iz) + q / (n * n);
 }
 
-// Natural index ex + N (ey + N ez) of element e_in_colour of the launch's colour class.
-__device__ __forceinline__ long long elem_natural(const OpArgs& a, long long e_in_colour) {
-  const Colour& c = a.col;
+// Natural index ex + N (ey + N ez) of element e_in_colour of the class.
+__device__ __forceinline__ long long elem_natural(const OpArgs& a, const Colour& c, long long e_in_colour) {
   const long long ix = e_in_colour % c.nx, iy = (e_in_colour / c.nx) % c.ny, iz = e_in_colour / ((long long)c.nx * c.ny);
   const long long ex = c.cx + c.stride * ix, ey = c.cy + c.stride * iy, ez = c.cz + c.stride * iz;
   return ex + (long long)a.N * (ey + (long long)a.N * ez);
 }
 
-// Material factor of element e_in_colour of the launch's colour class (1 if homogeneous).
-__device__ __forceinline__ double elem_factor(const OpArgs& a, long long e_in_colour) {
-  if (!a.factor) return 1.0;
-  const Colour& c = a.col;
-  const long long ix = e_in_colour % c.nx, iy = (e_in_colour / c.nx) % c.ny, iz = e_in_colour / ((long long)c.nx * c.ny);
-  const long long ex = c.cx + c.stride * ix, ey = c.cy + c.stride * iy, ez = c.cz + c.stride * iz;
-  return a.factor[ex + (long long)a.N * (ey + (long long)a.N * ez)];
+// Material factor of element e_in_colour of the class (1 if homogeneous).
+__device__ __forceinline__ double elem_factor(const OpArgs& a, const Colour& c, long long e_in_colour) {
+  return a.factor ? a.factor[elem_natural(a, c, e_in_colour)] : 1.0;
 }
 
 // One 1D pass along direction DIR over NC arrays of NI items:
