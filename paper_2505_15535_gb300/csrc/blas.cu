@@ -1,8 +1,10 @@
 // Vector kernels of the Krylov solvers (Section 2.3: CG on the matrix-free operator).
 // Reductions are deterministic: a grid that depends on the length alone accumulates FP64 partial
 // sums with a fixed grid-stride order and a fixed shuffle tree; the last block to finish reduces
-// the partials in a fixed order.  Results stay on the device.
+// the partials in a fixed order.  Results stay on the device.  The kernels start while the launch
+// before them drains and wait for it before they read (pdl.cuh).
 #include "blas.h"
+#include "pdl.cuh"
 
 namespace nhmf {
 namespace {
@@ -63,6 +65,8 @@ unsigned red_blocks(long long n) {
 template <typename TX, typename TY>
 __global__ void __launch_bounds__(kRedThreads) k_dot(long long n, const TX* x, const TY* y, double* partials, double* out,
                                                      bool root, const double* den, double sign, double* quot) {
+  pdl_launch_next();
+  pdl_wait();
   double acc[1] = {0.0}, tot[1];
   for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads)
     acc[0] = fma(double(x[i]), double(y[i]), acc[0]);
@@ -78,6 +82,8 @@ template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_pcg_update(long long n, const double* rz, const double* pq, T* x, T* r,
                                                             const T* p, const T* q, const T* dinv, T* z, double* partials,
                                                             double* rz_new, double* rr, unsigned* flag) {
+  pdl_launch_next();
+  pdl_wait();
   const double pqv = *pq;
   const bool ok = pqv > 0.0 && isfinite(pqv);
   const T alpha = ok ? T(*rz / pqv) : T(0);
@@ -100,6 +106,8 @@ __global__ void __launch_bounds__(kRedThreads) k_pcg_update(long long n, const d
 // Flexible CG: *pq = p.q, *alpha = p.r / p.q.
 __global__ void __launch_bounds__(kRedThreads) k_fcg_alpha(long long n, const double* p, const double* q, const double* r,
                                                            double* partials, double* pq, double* alpha) {
+  pdl_launch_next();
+  pdl_wait();
   double acc[2] = {0.0, 0.0}, tot[2];
   for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads) {
     acc[0] = fma(p[i], q[i], acc[0]);
@@ -114,6 +122,8 @@ __global__ void __launch_bounds__(kRedThreads) k_fcg_alpha(long long n, const do
 __global__ void __launch_bounds__(kRedThreads) k_fcg_update(long long n, const double* alpha, const double* p,
                                                             const double* q, double* x, double* r, double* partials,
                                                             double* rnorm) {
+  pdl_launch_next();
+  pdl_wait();
   const double al = *alpha;
   double acc[1] = {0.0}, tot[1];
   for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads) {
@@ -128,6 +138,8 @@ __global__ void __launch_bounds__(kRedThreads) k_fcg_update(long long n, const d
 // p = z + beta p with beta = rz_new / rz_old (beta = 0 when rz_old is null).
 template <typename T>
 __global__ void k_pcg_direction(long long n, const double* rz_new, const double* rz_old, const T* z, T* p) {
+  pdl_launch_next();
+  pdl_wait();
   const T beta = rz_old ? T(*rz_new / *rz_old) : T(0);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     p[i] = rz_old ? fma(beta, p[i], z[i]) : z[i];
@@ -137,6 +149,8 @@ __global__ void k_pcg_direction(long long n, const double* rz_new, const double*
 template <typename T>
 __global__ void __launch_bounds__(kRedThreads) k_jacobi(long long n, const T* r, const T* dinv, T* z, double* partials,
                                                         double* rz, double* rr) {
+  pdl_launch_next();
+  pdl_wait();
   double acc[2] = {0.0, 0.0}, tot[2];
   for (long long i = blockIdx.x * (long long)kRedThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kRedThreads) {
     const T zi = dinv[i] * r[i];
@@ -151,6 +165,8 @@ __global__ void __launch_bounds__(kRedThreads) k_jacobi(long long n, const T* r,
 
 // y = a x + b y with scalars a = sa * (*pa) (pa may be null -> sa), same for b.
 __global__ void k_axpby(long long n, double sa, const double* pa, const double* x, double sb, const double* pb, double* y) {
+  pdl_launch_next();
+  pdl_wait();
   const double a = pa ? sa * *pa : sa;
   const double b = pb ? sb * *pb : sb;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -181,6 +197,8 @@ __global__ void k_ratio_or_zero(const double* num, const double* den, double* ou
 
 template <typename TI, typename TO>
 __global__ void k_scale_convert(long long n, const TI* x, const double* scale, bool invert, TO* y) {
+  pdl_launch_next();
+  pdl_wait();
   double s = scale ? *scale : 1.0;
   if (invert) s = s > 0.0 ? 1.0 / s : 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -202,46 +220,56 @@ __global__ void k_mul(long long n, const double* d, double* x) {
 
 constexpr int kEwBlocks = 1216;  // 8 blocks per SM for element-wise kernels
 constexpr int kEwThreads = 256;
+unsigned ew_blocks(long long n) {
+  const long long b = (n + kEwThreads - 1) / kEwThreads;
+  return (unsigned)(b < 1 ? 1 : (b > kEwBlocks ? kEwBlocks : b));
+}
+
+template <typename TX, typename TY>
+void launch_dot(long long n, const TX* x, const TY* y, double* partials, double* out, bool root, const double* den,
+                double sign, double* quot, cudaStream_t s) {
+  launch(k_dot<TX, TY>, dim3(red_blocks(n)), kRedThreads, 0, s, true, n, x, y, partials, out, root, den, sign, quot);
+}
 
 }  // namespace
 
 void dot(long long n, const double* x, const double* y, double* out, double* partials, cudaStream_t s) {
-  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, y, partials, out, false, nullptr, 0.0, nullptr);
+  launch_dot(n, x, y, partials, out, false, nullptr, 0.0, nullptr, s);
 }
 void dot(long long n, const float* x, const float* y, double* out, double* partials, cudaStream_t s) {
-  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, y, partials, out, false, nullptr, 0.0, nullptr);
+  launch_dot(n, x, y, partials, out, false, nullptr, 0.0, nullptr, s);
 }
 void dot_ratio(long long n, const double* x, const double* y, double* out, const double* den, double sign, double* quot,
                double* partials, cudaStream_t s) {
-  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, y, partials, out, false, den, sign, quot);
+  launch_dot(n, x, y, partials, out, false, den, sign, quot, s);
 }
 void norm2(long long n, const double* x, double* out, double* partials, cudaStream_t s) {
-  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, x, partials, out, true, nullptr, 0.0, nullptr);
+  launch_dot(n, x, x, partials, out, true, nullptr, 0.0, nullptr, s);
 }
 void norm2(long long n, const float* x, double* out, double* partials, cudaStream_t s) {
-  k_dot<<<red_blocks(n), kRedThreads, 0, s>>>(n, x, x, partials, out, true, nullptr, 0.0, nullptr);
+  launch_dot(n, x, x, partials, out, true, nullptr, 0.0, nullptr, s);
 }
 void fcg_alpha(long long n, const double* p, const double* q, const double* r, double* pq, double* alpha,
                double* partials, cudaStream_t s) {
-  k_fcg_alpha<<<red_blocks(n), kRedThreads, 0, s>>>(n, p, q, r, partials, pq, alpha);
+  launch(k_fcg_alpha, dim3(red_blocks(n)), kRedThreads, 0, s, true, n, p, q, r, partials, pq, alpha);
 }
 void fcg_update(long long n, const double* alpha, const double* p, const double* q, double* x, double* r, double* rnorm,
                 double* partials, cudaStream_t s) {
-  k_fcg_update<<<red_blocks(n), kRedThreads, 0, s>>>(n, alpha, p, q, x, r, partials, rnorm);
+  launch(k_fcg_update, dim3(red_blocks(n)), kRedThreads, 0, s, true, n, alpha, p, q, x, r, partials, rnorm);
 }
 
 template <typename T>
 void pcg_update(long long n, const double* rz, const double* pq, T* x, T* r, const T* p, const T* q, const T* dinv, T* z,
                 double* rz_new, double* rr, double* partials, unsigned* flag, cudaStream_t s) {
-  k_pcg_update<T><<<red_blocks(n), kRedThreads, 0, s>>>(n, rz, pq, x, r, p, q, dinv, z, partials, rz_new, rr, flag);
+  launch(k_pcg_update<T>, dim3(red_blocks(n)), kRedThreads, 0, s, true, n, rz, pq, x, r, p, q, dinv, z, partials, rz_new, rr, flag);
 }
 template <typename T>
 void pcg_direction(long long n, const double* rz_new, const double* rz_old, const T* z, T* p, cudaStream_t s) {
-  k_pcg_direction<T><<<kEwBlocks, kEwThreads, 0, s>>>(n, rz_new, rz_old, z, p);
+  launch(k_pcg_direction<T>, dim3(ew_blocks(n)), kEwThreads, 0, s, true, n, rz_new, rz_old, z, p);
 }
 template <typename T>
 void jacobi(long long n, const T* r, const T* dinv, T* z, double* rz, double* rr, double* partials, cudaStream_t s) {
-  k_jacobi<T><<<red_blocks(n), kRedThreads, 0, s>>>(n, r, dinv, z, partials, rz, rr);
+  launch(k_jacobi<T>, dim3(red_blocks(n)), kRedThreads, 0, s, true, n, r, dinv, z, partials, rz, rr);
 }
 template void pcg_update<double>(long long, const double*, const double*, double*, double*, const double*, const double*,
                                  const double*, double*, double*, double*, double*, unsigned*, cudaStream_t);
@@ -253,7 +281,7 @@ template void jacobi<double>(long long, const double*, const double*, double*, d
 template void jacobi<float>(long long, const float*, const float*, float*, double*, double*, double*, cudaStream_t);
 
 void axpby(long long n, double a, const double* pa, const double* x, double b, const double* pb, double* y, cudaStream_t s) {
-  k_axpby<<<kEwBlocks, kEwThreads, 0, s>>>(n, a, pa, x, b, pb, y);
+  launch(k_axpby, dim3(ew_blocks(n)), kEwThreads, 0, s, true, n, a, pa, x, b, pb, y);
 }
 void ratio(const double* num, const double* den, double sign, double* out, cudaStream_t s) {
   k_ratio<<<1, 32, 0, s>>>(num, den, sign, out);
@@ -265,10 +293,10 @@ void ratio_or_zero(const double* num, const double* den, double* out, cudaStream
   k_ratio_or_zero<<<1, 32, 0, s>>>(num, den, out);
 }
 void to_fp32_scaled(long long n, const double* x, const double* scale, bool invert, float* y, cudaStream_t s) {
-  k_scale_convert<double, float><<<kEwBlocks, kEwThreads, 0, s>>>(n, x, scale, invert, y);
+  launch(k_scale_convert<double, float>, dim3(ew_blocks(n)), kEwThreads, 0, s, true, n, x, scale, invert, y);
 }
 void to_fp64_scaled(long long n, const float* x, const double* scale, double* y, cudaStream_t s) {
-  k_scale_convert<float, double><<<kEwBlocks, kEwThreads, 0, s>>>(n, x, scale, false, y);
+  launch(k_scale_convert<float, double>, dim3(ew_blocks(n)), kEwThreads, 0, s, true, n, x, scale, false, y);
 }
 void jacobi_apply(long long n, const double* dinv, double* x, cudaStream_t s) {
   k_mul<<<kEwBlocks, kEwThreads, 0, s>>>(n, dinv, x);

@@ -60,6 +60,44 @@ __global__ void __launch_bounds__(256) k_map1d(const T* __restrict__ in, T* __re
   *o = add ? *o + s : s;
 }
 
+// All three passes of a transfer for one component and one output z-plane: z from global memory, then y
+// and x in shared memory ([mi][mi], then [mo][mi]).  For the coarse levels, where the three launches
+// of k_map1d cost more than the planes that neighbouring outputs read again.
+template <typename T>
+__global__ void __launch_bounds__(256) k_map3d(const T* __restrict__ in, T* __restrict__ out, int mi, int mo,
+                                               const int* __restrict__ ptr, const int* __restrict__ col,
+                                               const T* __restrict__ w, bool add, int bc) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* z = reinterpret_cast<T*>(smem_raw);
+  T* y = z + mi * mi;
+  pdl_launch_next();
+  pdl_wait();
+  const int k = blockIdx.x, c = blockIdx.y;
+  const T* src = in + (long long)c * mi * mi * mi;
+  const int z0 = ptr[k], z1 = ptr[k + 1];
+  for (int ij = threadIdx.x; ij < mi * mi; ij += 256) {
+    T s = T(0);
+    for (int e = z0; e < z1; ++e) s = fma(w[e], src[(long long)mi * mi * col[e] + ij], s);
+    z[ij] = s;
+  }
+  __syncthreads();
+  for (int ij = threadIdx.x; ij < mo * mi; ij += 256) {
+    const int j = ij / mi, i = ij - j * mi;
+    T s = T(0);
+    for (int e = ptr[j]; e < ptr[j + 1]; ++e) s = fma(w[e], z[mi * col[e] + i], s);
+    y[ij] = s;
+  }
+  __syncthreads();
+  for (int ij = threadIdx.x; ij < mo * mo; ij += 256) {
+    const int j = ij / mo, i = ij - j * mo;
+    T s = T(0);
+    for (int e = ptr[i]; e < ptr[i + 1]; ++e) s = fma(w[e], y[mi * j + col[e]], s);
+    if (bc != NHMF_BC_NONE && constrained(bc, c, i, k, mo)) s = T(0);
+    T* o = out + ((long long)c * mo + k) * mo * mo + ij;
+    *o = add ? *o + s : s;
+  }
+}
+
 // Chebyshev step: d = c_old d + c_new D^-1 (b - q), x += d (q null: q = 0).
 template <typename T>
 __global__ void k_cheb(long long n, const T* __restrict__ b, const T* __restrict__ q, const T* __restrict__ dinv,
@@ -104,6 +142,10 @@ __global__ void k_to(long long n, const double* __restrict__ x, T* __restrict__ 
 }
 
 constexpr int kB = 1216, kT = 256;
+// Nodes per direction up to which a transfer is one launch.  Above it too few planes read too much:
+// Q4 16^3 linear solve (65 nodes) 79.3 ms with three launches everywhere, 78.2 with one up to 33,
+// 89.5 up to 65; Newton step Q2 16^3 (33 nodes) 10.4, 9.9 and 9.9 ms.
+constexpr int kMap3dMax = 33;
 unsigned ew_blocks(long long n) { return (unsigned)std::min<long long>(kB, (n + kT - 1) / kT); }
 
 // ------------------------------------------------------------------ host helpers
@@ -194,6 +236,12 @@ template <> const float* wts<float>(const Map1D& m) { return m.w32; }
 template <typename T>
 void map3d(const Map1D& m, const T* in, T* out, T* t1, T* t2, cudaStream_t s, bool add = false, int bc = NHMF_BC_NONE) {
   const int mi = m.cols, mo = m.rows;
+  const size_t planes = (size_t)mi * (mi + mo) * sizeof(T);
+  if (std::max(mi, mo) <= kMap3dMax && planes <= 48 * 1024) {
+    launch(k_map3d<T>, dim3((unsigned)mo, 3u), 256, planes, s, true, in, out, mi, mo, (const int*)m.ptr,
+           (const int*)m.col, wts<T>(m), add, bc);
+    return;
+  }
   auto pass = [&](const T* src, T* dst, int dir, int nx, int ny, int nz, bool a, int b) {
     const int ox = dir == 0 ? mo : nx, oy = dir == 1 ? mo : ny, oz = dir == 2 ? mo : nz;
     launch(k_map1d<T>, dim3((unsigned)((ox * oy + 255) / 256), (unsigned)oz, 3u), 256, 0, s, true, src, dst, dir, nx, ny,

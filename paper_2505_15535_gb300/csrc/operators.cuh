@@ -1043,7 +1043,8 @@ constexpr int kInitPer = 4;  // entries per thread
 template <typename T>
 __global__ void __launch_bounds__(256) k_init_rows(int bc, int M, const T* __restrict__ src, T* __restrict__ out,
                                                    T value) {
-  pdl_launch_next();
+  pdl_wait();
+  pdl_launch_next();  // after the wait: the first class reads du, which earlier launches write, before its own
   const int c = (int)blockIdx.y / M, k = (int)blockIdx.y - c * M, M2 = M * M;
   const long long base = (long long)M2 * blockIdx.y;
 #pragma unroll
@@ -1173,7 +1174,7 @@ nhmf_status run_colours(nhmf_ctx* c, KernelT kernel, OpArgs a, int NE, int threa
   if (cudaError_t e = prepare(kernel, smem); e != cudaSuccess) return cuda_check(c, e, what);
   const long long M2 = (long long)c->g.M * c->g.M;
   const dim3 init_grid((unsigned)((M2 + 256 * kInitPer - 1) / (256 * kInitPer)), (unsigned)(3 * c->g.M));
-  if (cudaError_t e = launch(k_init_rows<T>, init_grid, 256, 0, s, false, a.bc, c->g.M, src, out, value); e != cudaSuccess)
+  if (cudaError_t e = launch(k_init_rows<T>, init_grid, 256, 0, s, true, a.bc, c->g.M, src, out, value); e != cudaSuccess)
     return cuda_check(c, e, what);
   bool pdl = !c->profiling;  // the event below lies between the two launches
   nhmf_ctx::Rec rec{kind, 0, nullptr, nullptr};
