@@ -6,9 +6,9 @@
 //   d2 = r(down(s1));  m2 = r(conv(d2));  u1 = r(up(m2) + s1);  t1 = r(conv(u1));
 //   u0 = r(up(t1) + s0);  t0 = r(conv(u0));  y = conv(t0) C->3
 // with 3x3x3 zero-padded cross-correlations: conv (stride 1), down (stride 2) and up (the
-// transposed stride-2 convolution).  Activations are channels-last [voxel][16] BF16 (32 B
-// per voxel, one DRAM sector); inputs and outputs with 3 channels are padded to 16 with
-// zero weights.  Every convolution is an implicit GEMM on the tensor cores, BF16 -> FP32:
+// transposed stride-2 convolution).  Activations are two channel halves, [2][voxel][8] BF16 (16 B
+// per voxel and half), as the kernels stage them: every staged row of a half is one contiguous
+// run.  Inputs and outputs with 3 channels are padded to 16 with zero weights.  Every convolution is an implicit GEMM on the tensor cores, BF16 -> FP32:
 //   stride-1 forward/backward-data (k_conv_tc), the stride-2 down-convolution and the up
 //   layers' backward-data (k_down_tc), and the transposed stride-2 convolution (k_up_tc):
 //   tcgen05 MMAs with accumulators in tensor memory, M = 128 positions, K = 16 input
@@ -55,10 +55,10 @@ struct ConvArgs {
   int m_in;
   const __nv_bfloat16* w;      // [27][16 co][16 ci]
   const float* bias;           // [16] or null (zero beyond cout)
-  const __nv_bfloat16* add;    // [m_out^3][16] or null, added before the ReLU
-  const __nv_bfloat16* mask;   // [m_out^3][16] or null, output zeroed where mask <= 0
+  const __nv_bfloat16* add;    // [2][m_out^3][8] or null, added before the ReLU
+  const __nv_bfloat16* mask;   // [2][m_out^3][8] or null, output zeroed where mask <= 0
   int relu;
-  __nv_bfloat16* out;          // [m_out^3][16]
+  __nv_bfloat16* out;          // [2][m_out^3][8]
   float* out_planar;           // or [3][m_out^3] FP32 (channels 0..2)
   int m_out;
 };
@@ -106,8 +106,8 @@ __global__ void __launch_bounds__(1024) k_wgrad_reduce(const float* partial, con
 }
 
 // Bias gradient: per-block channel sums of P, then a fixed-order reduction.
-// Per-block channel sums of P [voxel][16] (the bias gradient's partials): a thread adds whole
-// 32-byte voxel rows, then the block adds its threads' sums in a fixed order.
+// Per-block channel sums of P (the bias gradient's partials): a thread adds both halves of whole
+// voxels, then the block adds its threads' sums in a fixed order.
 __global__ void __launch_bounds__(256) k_bgrad_partial(const __nv_bfloat16* P, long long nvox, float* partial) {
   pdl_launch_next();
   pdl_wait();
@@ -115,8 +115,8 @@ __global__ void __launch_bounds__(256) k_bgrad_partial(const __nv_bfloat16* P, l
 #pragma unroll
   for (int ch = 0; ch < 16; ++ch) s[ch] = 0.f;
   for (long long v = (long long)blockIdx.x * 256 + threadIdx.x; v < nvox; v += (long long)gridDim.x * 256) {
-    const uint4* src = reinterpret_cast<const uint4*>(P + v * kC);
-    const uint4 q0 = src[0], q1 = src[1];
+    const uint4* src = reinterpret_cast<const uint4*>(P) + v;
+    const uint4 q0 = src[0], q1 = src[nvox];
     const uint32_t q[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
     for (int h = 0; h < 8; ++h) {
@@ -214,9 +214,9 @@ __global__ void k_input(const TS* src, long long n, const double* den, double mu
     w[0] = pack_bf16(__float2bfloat16(float(src[v]) * s), __float2bfloat16(float(src[n + v]) * s));
     w[1] = pack_bf16(__float2bfloat16(float(src[2 * n + v]) * s), __float2bfloat16(0.f));
     for (int q = 2; q < 8; ++q) w[q] = 0u;
-    uint4* dst = reinterpret_cast<uint4*>(x16 + v * kC);
+    uint4* dst = reinterpret_cast<uint4*>(x16) + v;
     dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    dst[n] = make_uint4(w[4], w[5], w[6], w[7]);
   }
 }
 
@@ -294,10 +294,10 @@ __global__ void k_loss_grad(const float* y, const float* e, long long n, int bc,
     float d[3];
     for (int c = 0; c < 3; ++c)
       d[c] = constrained_dof(bc, c, v, M) ? 0.f : s * (y[c * n + v] - e[c * n + v]);
-    uint4* dst = reinterpret_cast<uint4*>(dy16 + v * kC);
+    uint4* dst = reinterpret_cast<uint4*>(dy16) + v;
     dst[0] = make_uint4(pack_bf16(__float2bfloat16(d[0]), __float2bfloat16(d[1])),
                         pack_bf16(__float2bfloat16(d[2]), __float2bfloat16(0.f)), 0u, 0u);
-    dst[1] = make_uint4(0u, 0u, 0u, 0u);
+    dst[n] = make_uint4(0u, 0u, 0u, 0u);
   }
 }
 
@@ -432,17 +432,18 @@ __device__ __forceinline__ void tc_teardown(uint32_t tmem, uint32_t cols, bool t
 }
 
 // Skip-connection and mask rows of voxel v (32 bytes each), or zeros where absent.
-__device__ __forceinline__ void tc_load_addmask(const ConvArgs& a, long long v, uint4 (&ad)[2], uint4 (&mk)[2]) {
+__device__ __forceinline__ void tc_load_addmask(const ConvArgs& a, long long v, long long nvox, uint4 (&ad)[2],
+                                                uint4 (&mk)[2]) {
   ad[0] = ad[1] = mk[0] = mk[1] = make_uint4(0u, 0u, 0u, 0u);
   if (a.add) {
-    const uint4* ap = reinterpret_cast<const uint4*>(a.add + v * kC);
+    const uint4* ap = reinterpret_cast<const uint4*>(a.add) + v;
     ad[0] = ap[0];
-    ad[1] = ap[1];
+    ad[1] = ap[nvox];
   }
   if (a.mask) {
-    const uint4* mp = reinterpret_cast<const uint4*>(a.mask + v * kC);
+    const uint4* mp = reinterpret_cast<const uint4*>(a.mask) + v;
     mk[0] = mp[0];
-    mk[1] = mp[1];
+    mk[1] = mp[nvox];
   }
 }
 
@@ -484,9 +485,9 @@ __device__ __forceinline__ void tc_emit(const ConvArgs& a, long long v, long lon
       const __nv_bfloat162 b2 = __floats2bfloat162_rn(o[2 * h], o[2 * h + 1]);
       pk[h] = *reinterpret_cast<const uint32_t*>(&b2);
     }
-    uint4* dst = reinterpret_cast<uint4*>(a.out + v * kC);
+    uint4* dst = reinterpret_cast<uint4*>(a.out) + v;
     dst[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    dst[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+    dst[nvox] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
   }
 }
 
@@ -507,6 +508,7 @@ __device__ __forceinline__ void tc_stage_async(const __nv_bfloat16* __restrict__
   const uint32_t s = smem_u32(slot);
   const uint4* g = reinterpret_cast<const uint4*>(in);
   const bool plane_in = zz >= 0 && zz < m;
+  const long long m3 = (long long)m * m * m;  // between the channel halves
   // padded row and column of position base + j (base >= -R), stepped without division
   int yr = (base + tid + R) / R - 1, xr = (base + tid + R) % R;
   for (int j = tid; j < L; j += nthr) {
@@ -514,11 +516,11 @@ __device__ __forceinline__ void tc_stage_async(const __nv_bfloat16* __restrict__
     const uint4* src = g;  // a valid address for the zero-filled copies, which read nothing
     uint32_t bytes = 0;
     if (plane_in && y >= 0 && y < m && x >= 0 && x < m) {
-      src = g + 2 * (x + (long long)m * (y + (long long)m * zz));
+      src = g + (x + (long long)m * (y + (long long)m * zz));
       bytes = 16;
     }
     cp_async16(s + (uint32_t)j * 16u, src, bytes);
-    cp_async16(s + (uint32_t)(L + j) * 16u, src + 1, bytes);
+    cp_async16(s + (uint32_t)(L + j) * 16u, src + m3, bytes);
     xr += nthr;
     while (xr >= R) {
       xr -= R;
@@ -539,7 +541,7 @@ __device__ __forceinline__ void tc_stage_async(const __nv_bfloat16* __restrict__
 // window of the strip.  Every output receives its 27 taps in the order of the per-tap form
 // (dz, then dy, then dx) on a zeroed accumulator.
 //
-// Planes arrive by TMA (cp.async.bulk.tensor, 5-D map [z][y][x][2 halves][8 channels]): per
+// Planes arrive by TMA (cp.async.bulk.tensor, 4-D map [2 halves][z][y][x]): per
 // 16-byte channel half one box of NY whole padded rows, x from x0 - 1 to x0 + W and zero
 // outside the grid, so that staged row r of a half is padded position Yb R + r (Yb = the padded
 // row of the tile's first halo position p0 - 1).  The grid runs as x-strips of W <=
@@ -602,12 +604,12 @@ __device__ __forceinline__ bool bar_or_128(bool v) {
 }
 
 
-__device__ __forceinline__ void tma_load5(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
-                                          int c4, uint32_t bar) {
+__device__ __forceinline__ void tma_load4(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
+                                          uint32_t bar) {
   asm volatile(
-      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, "
-      "%6}], [%7];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+      "[%6];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
       : "memory");
 }
 
@@ -664,8 +666,9 @@ __global__ void __launch_bounds__(kTcSThreads) k_conv_tc(const ConvArgs a, const
       const int sl = z % kTcSlots;
       const uint32_t fb = s_full + 8u * (uint32_t)sl, dst = sA0 + (uint32_t)sl * 2u * H;
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb), "r"(box_bytes) : "memory");
-      tma_load5(dst, &map, 0, 0, x0 - 1, Yb - 1, z, fb);
-      tma_load5(dst + H, &map, 0, 1, x0 - 1, Yb - 1, z, fb);
+      // x in 8-byte units, two to a voxel half: every start is a multiple of 16 bytes
+      tma_load4(dst, &map, 2 * (x0 - 1), Yb - 1, z, 0, fb);
+      tma_load4(dst + H, &map, 2 * (x0 - 1), Yb - 1, z, 1, fb);
       fpend |= 1u << sl;
     };
     if (epi) {
@@ -706,7 +709,7 @@ __global__ void __launch_bounds__(kTcSThreads) k_conv_tc(const ConvArgs a, const
         const int o = zi - 2;
         const bool emit = o >= zb && own;
         uint4 ad[2], mk[2];
-        if (emit) tc_load_addmask(a, v0 + (long long)m * m * o, ad, mk);
+        if (emit) tc_load_addmask(a, v0 + (long long)m * m * o, nvox, ad, mk);
         fail = !wait_plane(k - 1);
         if (!fail && o >= zb) {
           uint32_t r[16];
@@ -725,7 +728,7 @@ __global__ void __launch_bounds__(kTcSThreads) k_conv_tc(const ConvArgs a, const
           tc_ld16(lanes + 16u * (uint32_t)(o - zb), r);
           if (own) {
             uint4 ad[2], mk[2];
-            tc_load_addmask(a, v0 + (long long)m * m * o, ad, mk);
+            tc_load_addmask(a, v0 + (long long)m * m * o, nvox, ad, mk);
             tc_emit(a, v0 + (long long)m * m * o, nvox, r, sbias, ad, mk);
           }
         }
@@ -788,6 +791,7 @@ __device__ __forceinline__ void dn_stage_async(const __nv_bfloat16* __restrict__
   const uint32_t s = smem_u32(slot);
   const uint4* g = reinterpret_cast<const uint4*>(in);
   const bool plane_in = f >= 0 && f < mi;
+  const long long m3 = (long long)mi * mi * mi;  // between the channel halves
   int Yr = (P0 + tid + 2 * R) / R - 2, Xr = (P0 + tid + 2 * R) % R;  // row and column of P0 + j (P0 >= -R - 1)
   for (int j = tid; j < L; j += nthr) {
     const int cx = 2 * (Xr - 1 + x0), cy = 2 * Yr;
@@ -797,11 +801,11 @@ __device__ __forceinline__ void dn_stage_async(const __nv_bfloat16* __restrict__
       const uint4* src = g;  // a valid address for the zero-filled copies
       uint32_t bytes = 0;
       if (plane_in && fx >= 0 && fx < mi && fy >= 0 && fy < mi) {
-        src = g + 2 * (fx + (long long)mi * (fy + (long long)mi * f));
+        src = g + (fx + (long long)mi * (fy + (long long)mi * f));
         bytes = 16;
       }
       cp_async16(s + (uint32_t)((2 * sp) * L + j) * 16u, src, bytes);
-      cp_async16(s + (uint32_t)((2 * sp + 1) * L + j) * 16u, src + 1, bytes);
+      cp_async16(s + (uint32_t)((2 * sp + 1) * L + j) * 16u, src + m3, bytes);
     }
     Xr += nthr;
     while (Xr >= R) {
@@ -871,7 +875,7 @@ __global__ void __launch_bounds__(kTcSThreads) k_down_tc(const ConvArgs a, int z
       tc_ld16(lanes + 16u * (uint32_t)(o - zb), r);
       if (own) {
         uint4 ad[2], mk[2];
-        tc_load_addmask(a, v0 + (long long)mo * mo * o, ad, mk);
+        tc_load_addmask(a, v0 + (long long)mo * mo * o, nvox, ad, mk);
         tc_emit(a, v0 + (long long)mo * mo * o, nvox, r, sbias, ad, mk);
       }
     };
@@ -1023,9 +1027,9 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_up_tc(const ConvArgs a, int z
         long long v;
         q[0] = q[1] = make_uint4(0u, 0u, 0u, 0u);
         if (a.add && fine(cl, v)) {
-          const uint4* src = reinterpret_cast<const uint4*>(a.add + v * kC);
+          const uint4* src = reinterpret_cast<const uint4*>(a.add) + v;
           q[0] = src[0];
-          q[1] = src[1];
+          q[1] = src[nvox];
         }
       };
       auto store = [&](int cl, const uint4 (&q)[2]) {
@@ -1035,9 +1039,9 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_up_tc(const ConvArgs a, int z
         if (fine(cl, v)) {
           uint4 mk[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
           if (a.mask) {
-            const uint4* src = reinterpret_cast<const uint4*>(a.mask + v * kC);
+            const uint4* src = reinterpret_cast<const uint4*>(a.mask) + v;
             mk[0] = src[0];
-            mk[1] = src[1];
+            mk[1] = src[nvox];
           }
           tc_emit(a, v, nvox, r, sbias, q, mk);
         }
@@ -1142,11 +1146,11 @@ __device__ __forceinline__ void wg_stage_rows_async(const __nv_bfloat16* __restr
     const uint4* src = g;
     uint32_t bytes = 0;
     if (p < m * R && xl >= 0 && xl < W && x < m) {
-      src = g + 2 * (x + (long long)m * (y + (long long)m * z));
+      src = g + (x + (long long)m * (y + (long long)m * z));
       bytes = 16;
     }
     cp_async16(s + (uint32_t)j * 16u, src, bytes);
-    cp_async16(s + (uint32_t)(128 + j) * 16u, src + 1, bytes);
+    cp_async16(s + (uint32_t)(128 + j) * 16u, src + (long long)m * m * m, bytes);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -1294,11 +1298,11 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_s2(const __nv_bfloat16* __
         const uint4* src = qg;
         uint32_t bytes = 0;
         if (fin && fy >= 0 && fy < mq && fx >= 0 && fx < mq) {
-          src = qg + 2 * (fx + (long long)mq * (fy + (long long)mq * f));
+          src = qg + (fx + (long long)mq * (fy + (long long)mq * f));
           bytes = 16;
         }
         cp_async16(d + (uint32_t)(r * Wf + i) * 16u, src, bytes);
-        cp_async16(d + (uint32_t)hs + (uint32_t)(r * Wf + i) * 16u, src + 1, bytes);
+        cp_async16(d + (uint32_t)hs + (uint32_t)(r * Wf + i) * 16u, src + (long long)mq * mq * mq, bytes);
       }
     }
   };
@@ -1309,11 +1313,11 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_s2(const __nv_bfloat16* __
       const uint4* src = pg;
       uint32_t bytes = 0;
       if (x0 + k < mp) {
-        src = pg + 2 * ((x0 + k) + (long long)mp * (cy + (long long)mp * cz));
+        src = pg + ((x0 + k) + (long long)mp * (cy + (long long)mp * cz));
         bytes = 16;
       }
       cp_async16(d + (uint32_t)k * 16u, src, bytes);
-      cp_async16(d + (uint32_t)(seg + k) * 16u, src + 1, bytes);
+      cp_async16(d + (uint32_t)(seg + k) * 16u, src + (long long)mp * mp * mp, bytes);
     }
   };
   for (long long unit = blockIdx.x; unit < nunits; unit += gridDim.x) {
@@ -1432,11 +1436,13 @@ void conv_tc_launch(const ConvArgs& a, unsigned* status, cudaStream_t s) {
   const int W = conv_strip_width(m, &nstrips), R = W + 2;
   CUtensorMap map;
   const TensorMapEncodeTiled enc = tensor_map_encoder();
-  const cuuint64_t dims[5] = {8, 2, (cuuint64_t)m, (cuuint64_t)m, (cuuint64_t)m};
-  const cuuint64_t strides[4] = {16, 32, 32ull * (cuuint64_t)m, 32ull * (cuuint64_t)m * (cuuint64_t)m};
-  const cuuint32_t box[5] = {8, 1, (cuuint32_t)R, (cuuint32_t)tma_ny(R), 1};
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  if (!enc || enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<__nv_bfloat16*>(a.in), dims, strides, box,
+  // [half][z][y][x] with a voxel half as two 8-byte units, so that a box row is one contiguous run
+  const cuuint64_t dims[4] = {2 * (cuuint64_t)m, (cuuint64_t)m, (cuuint64_t)m, 2};
+  const cuuint64_t strides[3] = {16ull * (cuuint64_t)m, 16ull * (cuuint64_t)m * (cuuint64_t)m,
+                                 16ull * (cuuint64_t)m * (cuuint64_t)m * (cuuint64_t)m};
+  const cuuint32_t box[4] = {2 * (cuuint32_t)R, (cuuint32_t)tma_ny(R), 1, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  if (!enc || enc(&map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<__nv_bfloat16*>(a.in), dims, strides, box,
                   estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
     k_flag<<<1, 1, 0, s>>>(status, kStatusTmaSetup);
