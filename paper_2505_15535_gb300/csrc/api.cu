@@ -83,7 +83,7 @@ nhmf_status create_context(const nhmf_params* prm, nhmf_ctx** out) {
   build_tables(prm->degree, &c->tab);
   long long min_colour = c->g.colour[0].count;
   for (int k = 1; k < 8; ++k) min_colour = std::min<long long>(min_colour, c->g.colour[k].count);
-  c->reg32 = prm->degree <= kRegMaxP && min_colour >= kRegMinColour;
+  c->reg32 = prm->degree == 1 || (prm->degree <= kRegMaxP && min_colour >= kRegMinColour);
   cudaGetDevice(&c->device);
   if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || c->sms < 1) c->sms = 1;
   nhmf_status st = cuda_check(c, cudaMalloc(&c->status, sizeof(unsigned)), "status alloc");

@@ -14,10 +14,16 @@ namespace nhmf {
 
 constexpr int kMaxN = 5;  // p + 1 for p <= 4
 
-// FP32 applies up to degree kRegMaxP use the one-element-per-thread register kernel (with its
-// [10][n^3][E] point-cache layout) when every colour class has at least kRegMinColour
-// elements; smaller meshes (coarse multigrid levels) and higher degrees use the shared-memory
-// kernel, whose latency per launch does not grow with the element's work.
+// FP32 applies up to degree kRegMaxP use the one-element-per-thread register kernel (with its tiled
+// point-cache layout): at p = 1 always, at p = 2 when every colour class has at least kRegMinColour
+// elements; smaller p = 2 meshes (coarse multigrid levels) and higher degrees use the column kernel,
+// whose latency per launch does not grow with the element's work.  Where the line lies:
+//   p = 1, register kernel against one thread per point (us per apply, cached and on the fly): 24^3
+//     elements 10.0 / 10.5 and 10.9 / 13.2, 32^3 10.0 / 14.0 and 9.9 / 16.6, 48^3 14.7 / 32.7 and
+//     17.8 / 41.0, 63^3 27 / 67 and 34 / 86; up to 16^3 both are launch latency (10)
+//   p = 2, register against column kernel: 40^3 on the fly 45 / 40, 56^3 108 / 104, 63^3 150 / 150;
+//     cached 48^3 46 / 54, 63^3 112 / 123, but the column kernel's rounding error is the smaller one
+//     (8.8e-8 of the norm against 1.1e-7 at 33^3), so the line is the one of the fly
 #ifndef NHMF_REG_MAXP
 #define NHMF_REG_MAXP 2
 #endif

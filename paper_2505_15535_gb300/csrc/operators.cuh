@@ -1,6 +1,7 @@
 // Matrix-free operators of compressible neo-Hookean elasticity on the GPU:
-//   k_apply         tangent application, on the fly (Algorithm 1) or from the point cache
+//   k_apply         FP64 and double-float tangent application, on the fly (Algorithm 1) or from the point cache
 //   k_apply_reg     FP32 tangent application, one element per thread in registers (p <= 2)
+//   k_apply_col     FP32 tangent application, one column of points per thread (p >= 2; apply32.cuh)
 //   k_gather_local  FP32: sums the element-local results of the apply at the nodes
 //   k_cache         point cache {F^-1, ln J} at the linearisation point (partial assembly, Section 3.2)
 //   k_residual      residual R(u) (Eq. F)
@@ -109,23 +110,6 @@ __device__ __forceinline__ void scatter_add(const OpArgs& a, const T* src, long 
   }
 }
 
-// Element-local results of the block's elements (launched on the class of all elements, so the
-// slot is the natural element index) into the element tiles of vloc, [E/32][3][n^3][32]:
-// consecutive threads write consecutive elements of one (c, q) row.
-template <int P, int NE>
-__device__ __forceinline__ void store_local(const OpArgs& a, const float* src, long long e0, int nvalid) {
-  constexpr int n3 = (P + 1) * (P + 1) * (P + 1), NI = NE * n3;
-  const long long slot = a.col.slot0 + e0;
-  const unsigned long long keep_pol = l2_evict_last();
-  for (int t = threadIdx.x; t < 3 * n3 * NE; t += blockDim.x) {
-    const int e = t % NE, cq = t / NE;
-    const long long el = slot + e;
-    if (e < nvalid)
-      st_policy(a.vloc + ((el / kTile) * 3 * n3 + cq) * kTile + el % kTile, src[(cq / n3) * NI + e * n3 + cq % n3],
-                keep_pol);
-  }
-}
-
 // Forward interpolation of three components to the points: in -> out (tmp is clobbered).
 template <int n, int NI, typename T>
 __device__ __forceinline__ void to_points(const T* sB, T* in, T* tmp, T* out, int nitems) {
@@ -201,7 +185,6 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
   T* G = Vq + 3 * NI;                           // [9][NI] gradients, then fluxes; G[0..2] gathers
 
   pdl_launch_next();
-  if constexpr (std::is_same<T, float>::value) pdl_wait();  // one launch: nothing of it may run ahead
   load_apply_tables<P>(a, tab);
   const Colour& col = a.col;
   const long long e0 = (long long)blockIdx.x * NE;
@@ -310,18 +293,12 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
           }
           const float2 z = cdf[9 * a.nq + cbase + t];
           lnJ = T(z.x, z.y);
-        } else if (sizeof(typename Store<T>::type) == 8 || P > kRegMaxP || !a.reg32) {
+        } else {
           // the cache is read once per apply: evict it first, keep du and v in L2
           const unsigned long long pol = l2_evict_first();
 #pragma unroll
           for (int k = 0; k < 9; ++k) Fi[k] = T(ld_policy(cache + k * a.nq + cbase + t, pol));
           lnJ = T(ld_policy(cache + 9 * a.nq + cbase + t, pol));
-        } else {
-          const long long slot = col.slot0 + e0 + t / n3, q = t % n3;
-          const auto* tile = cache + (slot / kTile) * (10 * n3 * kTile) + slot % kTile;
-#pragma unroll
-          for (int k = 0; k < 9; ++k) Fi[k] = T(tile[(k * n3 + q) * kTile]);
-          lnJ = T(tile[(9 * n3 + q) * kTile]);
         }
       } else {
 #pragma unroll
@@ -336,12 +313,6 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
   if (bad) atomicOr(a.status, kStatusNonPosJ);
   __syncthreads();
   transposed<n, NI, TH, EO>(sBW, sDcW, kBW, G, Vq, nitems, nlines);
-  if constexpr (std::is_same<T, float>::value) {
-    if (a.vloc) {
-      store_local<P, NE>(a, G + 3 * NI, e0, nvalid);
-      return;
-    }
-  }
   scatter_add<P, NI>(a, G + 3 * NI, e0, nvalid, static_cast<typename Store<T>::type*>(a.v));
 }
 
@@ -760,7 +731,7 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
         for (int k = 0; k < 9; ++k) tile[(k * n3 + q) * kTile] = float(Fi[k]);
         tile[(9 * n3 + q) * kTile] = float(lnJ);
       } else {
-        // layout [10][E n^3] for the shared-memory kernel
+        // layout [10][E n^3] for the column kernel
 #pragma unroll
         for (int k = 0; k < 9; ++k) a.cache32_out[k * a.nq + en * n3 + q] = float(Fi[k]);
         a.cache32_out[9 * a.nq + en * n3 + q] = float(lnJ);
@@ -1162,11 +1133,11 @@ cudaError_t prepare(KernelT kernel, size_t smem) {
 }
 
 // Runs `kernel` once per colour class with NE elements per block, after k_init_rows on `out`.  The
-// classes are chained by programmatic
-// dependent launch: everything before a class's scatter depends on no other class, so its blocks
-// fill the SMs that the classes before it leave idle, and it waits for those classes only before
-// it adds to `out`.  FP64 cached apply against plain launches: Q1 8^3 140 -> 30 us and Q2 16^3
-// 368 -> 57 us (with the small blocks), Q2 64^3 2174 -> 2072 us (the classes' last waves).  The first launch of the chain waits for all earlier work of the stream as
+// classes are chained by programmatic dependent launch: everything before a class's scatter depends
+// on no other class, so its blocks fill the SMs that the classes before it leave idle, and it waits
+// for those classes only before it adds to `out`.  FP64 cached apply against plain launches: Q1 8^3
+// 140 -> 30 us and Q2 16^3 368 -> 57 us (with the small blocks), Q2 64^3 2174 -> 2072 us (the
+// classes' last waves).  The first launch of the chain waits for all earlier work of the stream as
 // usual; each class waits for the one before it, so the last one ends after all.
 template <typename T, typename KernelT>
 nhmf_status run_colours(nhmf_ctx* c, KernelT kernel, OpArgs a, int NE, int threads, size_t smem, const T* src, T* out,
@@ -1293,10 +1264,7 @@ nhmf_status apply_p(nhmf_ctx* c, const void* du, void* v, bool raw, const Gather
       return run_local<P>(c, k_apply_col<P, STRAT, NHMF_MODEL_COMPRESSIBLE>, a, Sh::NE, Sh::THREADS,
                           col_fields<P + 1, STRAT, NHMF_MODEL_COMPRESSIBLE>() * field, du32, v32, g32, s);
     } else {
-      using Sh = Shape<P, T, STRAT, false>;
-      const size_t smem = (kTabSlots + per_item * Sh::NE * (P + 1) * (P + 1) * (P + 1)) * sizeof(T);
-      auto* k = split ? k_apply<P, T, STRAT, SPLIT, false> : k_apply<P, T, STRAT, NHMF_MODEL_COMPRESSIBLE, false>;
-      return run_local<P>(c, k, a, Sh::NE, Sh::THREADS, smem, du32, v32, g32, s);
+      return fail(c, NHMF_ERR_STATE, "apply: p = 1 without the register kernel");  // reg32 is always set there
     }
   } else {
     if (small_blocks<T, Shape<P, T, STRAT, false>::NE>(c))

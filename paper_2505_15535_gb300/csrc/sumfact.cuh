@@ -33,7 +33,6 @@ template <> struct Cfg<1, double> { static constexpr int NE = 32, THREADS = 256;
 template <> struct Cfg<2, double> { static constexpr int NE = NHMF_Q2D_NE, THREADS = NHMF_Q2D_THREADS; };
 template <> struct Cfg<3, double> { static constexpr int NE = 8, THREADS = 256; };
 template <> struct Cfg<4, double> { static constexpr int NE = NHMF_Q4D_NE, THREADS = NHMF_Q4D_THREADS; };
-template <> struct Cfg<1, float> { static constexpr int NE = 32, THREADS = 256; };  // p >= 2: ColShape (apply32.cuh)
 template <int P> struct Cfg<P, df64> : Cfg<P, double> {};
 template <> struct Cfg<4, df64> { static constexpr int NE = 4, THREADS = 256; };
 // Launch shape per strategy: Algorithm 2's point code (120 registers) keeps 256 threads at Q4

@@ -103,3 +103,25 @@ def test_fp32_column_kernel(p, N, bc, model):
         free = ~fixed
         assert np.linalg.norm(v[free] - ref[free]) <= 1e-5 * np.linalg.norm(ref[free])
     prob.close()
+
+
+@pytest.mark.parametrize("N", [1, 3, 4, 15, 17])
+@pytest.mark.parametrize("bc,model", [(0, 0), (1, 1), (2, 0)])
+def test_fp32_register_kernel_q1(N, bc, model):
+    """Q1 FP32 applies on meshes of less than one warp of elements up to several blocks, most of
+    them not a multiple of a tile; with inclusions, both models and strategies."""
+    import torch
+    nhmf = lib_or_fail()
+    w = workload(1, N, bc)
+    u, du, fac = inp.draw_u(w), inp.draw_du(w), inp.inclusion_factors(N, 10.0)
+    fixed = inp.dirichlet_mask(N, 1, bc).reshape(-1)
+    du[fixed] = 0.25  # identity rows show
+    ref = Operator(Mesh(N, 1), 1.0, 1.5, bc, model=model, factors=fac).apply(u, du)
+    prob = nhmf.Problem(N, 1, 1.0, 1.5, bc, model=model)
+    nhmf.nhmf_set_material_factors(prob.ctx, cuda(fac))
+    prob.set_linearization(cuda(u), 0 if model else nhmf.NHMF_CACHE_FP32)
+    dut = cuda(du).float()
+    for strat in (0,) if model else (0, 1):
+        v = host(prob.apply(dut, torch.full_like(dut, np.nan), nhmf.NHMF_FP32, strat))
+        assert np.linalg.norm(v - ref) <= 1e-5 * np.linalg.norm(ref)
+    prob.close()
