@@ -470,7 +470,7 @@ def run_gpu(args):
                        "l2": "flushed between timed steps (256 MB write outside the timed events)",
                        "parallelism": "replicas" if world > 1 else "single GPU"},
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": int(launches + args.steps),   # 8 colour launches + 1 Dirichlet fix per step
+            "gpu_launches": int(launches + args.steps),   # 8 colour launches + 1 that fills the rows, per step
             "clocks": clocks, "cache_build_s": cache_build_s, "variants": variants, "newton": newton,
         }
         print(json.dumps(line), flush=True)

@@ -292,9 +292,8 @@ nhmf_status nhmf_linear_solve_noalloc(nhmf_ctx* ctx, int strategy, double rtol, 
  * A 3-level convolutional U-Net on the nodal grid (16 channels, 3x3x3 convolutions, ReLU,
  * stride-2 down and transposed-convolution up paths with additive skips; 3 input and 3
  * output channels = the displacement components), BF16 weights and activations with FP32
- * accumulation on the tensor cores (tcgen05 for the stride-1 and transposed stride-2
- * convolutions, mma.sync for the stride-2 down convolution and the weight gradients), FP32
- * master weights trained by Adam.  It maps a
+ * accumulation on the tensor cores (tcgen05 for the convolutions of all three kinds, mma.sync
+ * for the weight gradients), FP32 master weights trained by Adam.  It maps a
  * residual r (scaled to unit RMS) to a correction; as a preconditioner z = N(r) scaled back
  * and zeroed on constrained DoFs.  Requires p*N divisible by 4 and at most 784.
  * Parameters: a flat FP32 array, layer by layer (in, e0, d1, e1, d2, m2, u1, t1, u0, t0,
@@ -325,9 +324,10 @@ nhmf_status nhmf_unet_train(nhmf_ctx* ctx, int epochs, double lr, double* loss_f
 
 /* Kernel timing.  While enabled, every operator call records a CUDA event pair on its
  * stream around its element kernels (FP64 and double-float: the eight colour launches, not the
- * vector memset or the Dirichlet-row fix; FP32: the element-local launch and the node gather).  nhmf_profile_read() synchronises those events, returns the summed
- * elapsed milliseconds and the number of element-kernel launches recorded for one operator
- * kind (NHMF_KIND_*), and clears that kind's record. */
+ * launch before them that fills the output's rows; the point cache: its one launch; FP32: the
+ * element-local launch and the node gather).  nhmf_profile_read() synchronises those events,
+ * returns the summed elapsed milliseconds and the number of element-kernel launches recorded for
+ * one operator kind (NHMF_KIND_*), and clears that kind's record. */
 enum { NHMF_KIND_APPLY = 0, NHMF_KIND_CACHE = 1, NHMF_KIND_RESIDUAL = 2, NHMF_KIND_DIAGONAL = 3 };
 nhmf_status nhmf_profile_enable(nhmf_ctx* ctx, int enable);
 nhmf_status nhmf_profile_read(nhmf_ctx* ctx, int kind, double* elapsed_ms, long long* launches);

@@ -8,7 +8,8 @@
 // with 3x3x3 zero-padded cross-correlations: conv (stride 1), down (stride 2) and up (the
 // transposed stride-2 convolution).  Activations are two channel halves, [2][voxel][8] BF16 (16 B
 // per voxel and half), as the kernels stage them: every staged row of a half is one contiguous
-// run.  Inputs and outputs with 3 channels are padded to 16 with zero weights.  Every convolution is an implicit GEMM on the tensor cores, BF16 -> FP32:
+// run.  Inputs and outputs with 3 channels are padded to 16 with zero weights.  Every convolution is
+// an implicit GEMM on the tensor cores, BF16 -> FP32:
 //   stride-1 forward/backward-data (k_conv_tc), the stride-2 down-convolution and the up
 //   layers' backward-data (k_down_tc), and the transposed stride-2 convolution (k_up_tc):
 //   tcgen05 MMAs with accumulators in tensor memory, M = 128 positions, K = 16 input
