@@ -32,7 +32,7 @@ __device__ __forceinline__ bool constrained(int bc, int c, int i, int k, int M) 
 // added to out if `add`, and zero on the constrained DoFs of preset `bc` on an ox^3 grid.  Grid: x
 // covers an output z-plane, y the planes, z the components.
 template <typename T>
-__global__ void __launch_bounds__(256) k_map1d(const T* __restrict__ in, T* __restrict__ out, int dir, int nx, int ny,
+__global__ void __launch_bounds__(256) k_map1d(const T* in, T* out, int dir, int nx, int ny,
                                                int nz, int mout, const int* __restrict__ ptr,
                                                const int* __restrict__ col, const T* __restrict__ w, bool add, int bc) {
   const int ox = dir == 0 ? mout : nx, oy = dir == 1 ? mout : ny, oz = dir == 2 ? mout : nz;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256) k_map1d(const T* __restrict__ in, T* __re
 // and x in shared memory ([mi][mi], then [mo][mi]).  For the coarse levels, where the three launches
 // of k_map1d cost more than the planes that neighbouring outputs read again.
 template <typename T>
-__global__ void __launch_bounds__(256) k_map3d(const T* __restrict__ in, T* __restrict__ out, int mi, int mo,
+__global__ void __launch_bounds__(256) k_map3d(const T* in, T* out, int mi, int mo,
                                                const int* __restrict__ ptr, const int* __restrict__ col,
                                                const T* __restrict__ w, bool add, int bc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -100,8 +100,7 @@ __global__ void __launch_bounds__(256) k_map3d(const T* __restrict__ in, T* __re
 
 // Chebyshev step: d = c_old d + c_new D^-1 (b - q), x += d (q null: q = 0).
 template <typename T>
-__global__ void k_cheb(long long n, const T* __restrict__ b, const T* __restrict__ q, const T* __restrict__ dinv,
-                       T* __restrict__ d, T* __restrict__ x, T c_old, T c_new) {
+__global__ void k_cheb(long long n, const T* b, const T* q, const T* dinv, T* d, T* x, T c_old, T c_new) {
   pdl_launch_next();
   pdl_wait();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {

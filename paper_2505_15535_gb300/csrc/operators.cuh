@@ -94,7 +94,7 @@ __device__ __forceinline__ double to_store(df64 x) { return to_double(x); }
 // (rows of constrained DoFs keep what k_init_rows wrote), scaled by a per-element factor fac[e].
 template <int P, int NI, typename T>
 __device__ __forceinline__ void scatter_add(const OpArgs& a, const T* src, long long e0, int nvalid,
-                                            typename Store<T>::type* __restrict__ out, const T* fac = nullptr) {
+                                            typename Store<T>::type* out, const T* fac = nullptr) {
   constexpr int n3 = (P + 1) * (P + 1) * (P + 1);
   pdl_wait();
   for (int t = threadIdx.x; t < NI; t += blockDim.x) {
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(kRegThreads, NHMF_REG_MINB) k_apply_reg(const 
             gk0 = P * (col.cz + col.stride * iz);
   const long long M = a.M;
   const long long slot = col.slot0 + ec;
-  const float* __restrict__ du = static_cast<const float*>(a.du);
+  const float* du = static_cast<const float*>(a.du);
   // this element's column of its tile in the point cache and in vloc
   float* __restrict__ vloc = a.vloc + (slot / kTile) * (3 * n3 * kTile) + slot % kTile;
   const float* __restrict__ cache =
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(kRegThreads, NHMF_REG_MINB) k_apply_reg(const 
 // step costs no further pass over A x and no launch.  v may be du in those forms: every thread
 // reads and writes its own node only.
 template <int P, int MODE>
-__global__ void __launch_bounds__(256) k_gather_local(const float* __restrict__ vloc, const float* du, float* v, int N,
+__global__ void __launch_bounds__(256) k_gather_local(const float* vloc, const float* du, float* v, int N,
                                                      int M, int bc, const Gather32 g32) {
   constexpr int n = P + 1, n3 = n * n * n;
   static_assert(kTile == 32, "tile index by shift and mask");
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(256) k_gather_local(const float* __restrict__ 
         const int q = lo[0][x] + n * (lo[1][y] + n * lo[2][z]);
         const float* src = vloc + (size_t)(e >> 5) * (3 * n3 * kTile) + q * kTile + (e & 31u);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) val[c][4 * z + 2 * y + x] = ld_policy(src + c * n3 * kTile, done_pol);
+        for (int c = 0; c < 3; ++c) val[c][4 * z + 2 * y + x] = ld_produced(src + c * n3 * kTile, done_pol);
       }
     }
 #pragma unroll
@@ -1012,8 +1012,7 @@ __global__ void __launch_bounds__(DiagCfg<P, SMALL>::THREADS) k_diagonal(const O
 // components.
 constexpr int kInitPer = 4;  // entries per thread
 template <typename T>
-__global__ void __launch_bounds__(256) k_init_rows(int bc, int M, const T* __restrict__ src, T* __restrict__ out,
-                                                   T value) {
+__global__ void __launch_bounds__(256) k_init_rows(int bc, int M, const T* src, T* out, T value) {
   pdl_wait();
   pdl_launch_next();  // after the wait: the first class reads du, which earlier launches write, before its own
   const int c = (int)blockIdx.y / M, k = (int)blockIdx.y - c * M, M2 = M * M;

@@ -14,6 +14,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // One launch; with `pdl` its blocks may start once every block of the launch before it has started
 // (and must not touch that launch's output, or anything it reads, before pdl_wait).  Every kernel
 // launched so calls pdl_wait, so that the completion of one launch is that of all before it.
+// What that launch writes is no constant of this grid's lifetime, also after the wait: it is read
+// through pointers without __restrict__ and not by ld.global.nc.
 template <typename KernelT, typename... Args>
 cudaError_t launch(KernelT kernel, dim3 grid, int threads, size_t smem, cudaStream_t s, bool pdl, Args... args) {
   cudaLaunchAttribute attr{};

@@ -143,6 +143,18 @@ __device__ __forceinline__ float ld_policy_ordered(const float* a, unsigned long
   asm volatile("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol));
   return v;
 }
+// A value that the launch before this one writes, for after pdl_wait(): that launch may still run when
+// this grid starts, so the load must not be .nc (data constant while the grid lives), and the
+// compiler has to keep it behind the wait.
+__device__ __forceinline__ float ld_produced(const float* a, unsigned long long pol) {
+  float v;
+#if NHMF_L2HINT
+  asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(pol) : "memory");
+#else
+  v = *static_cast<const volatile float*>(a);
+#endif
+  return v;
+}
 __device__ __forceinline__ double ld_policy(const double* a, unsigned long long pol) {
 #if NHMF_L2HINT
   double v;

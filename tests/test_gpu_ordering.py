@@ -1,0 +1,67 @@
+"""Launches that start while the one before them drains: FP32 applies (element kernel, then node
+gather) whose input the stream has only just written and whose output it reads at once, and multigrid
+cycles (smoothing, transfers), give bit by bit what they give with the GPU idle in between."""
+import pytest
+
+import nhmf_inputs as inp
+from tests.gpu_util import cuda, lib_or_fail
+
+pytestmark = pytest.mark.gpu
+
+
+def problem(nhmf, p, N, amp=0.05):
+    w = inp.Workload("order", N, p, 1.0, 1.5, 1, "scaled", amp, "normal", 1.0, 4300 + N, 4400 + N)
+    prob = nhmf.Problem.from_workload(w)
+    prob.set_linearization(cuda(inp.draw_u(w)), nhmf.NHMF_CACHE_FP64 | nhmf.NHMF_CACHE_FP32)
+    return prob, cuda(inp.draw_du(w))
+
+
+@pytest.mark.parametrize("strat", [0, 1])
+@pytest.mark.parametrize("p,N", [(1, 9), (1, 40), (2, 12), (2, 64), (3, 11), (4, 10)])
+def test_fp32_applies_back_to_back(p, N, strat):
+    import torch
+    nhmf = lib_or_fail()
+    prob, d = problem(nhmf, p, N)
+    d = d.float()
+    want, x = [], d.clone()
+    for _ in range(3):
+        y = prob.apply(x, torch.empty_like(x), nhmf.NHMF_FP32, strat)
+        torch.cuda.synchronize()
+        want.append(y)
+        x = 0.5 * y
+    torch.cuda.synchronize()
+    v = torch.empty_like(d)
+    for _ in range(20):
+        x = d
+        for k in range(3):
+            prob.apply(x, v, nhmf.NHMF_FP32, strat)   # the same output, and so the same scratch, each time
+            y = v.clone()
+            assert torch.equal(y, want[k])
+            x = 0.5 * y
+    # applies with nothing in between: each one's gather and the next one's element kernel share vloc
+    outs = [torch.empty_like(d) for _ in range(12)]
+    prob.apply(d, outs[0], nhmf.NHMF_FP32, strat)
+    for a, b in zip(outs, outs[1:]):
+        prob.apply(a, b, nhmf.NHMF_FP32, strat)
+    torch.cuda.synchronize()
+    x = d
+    for out in outs:
+        y = prob.apply(x, torch.empty_like(x), nhmf.NHMF_FP32, strat)
+        torch.cuda.synchronize()
+        assert torch.equal(y, out)
+        x = out
+    prob.close()
+
+
+@pytest.mark.parametrize("p,N", [(1, 16), (2, 8), (3, 12)])
+def test_multigrid_repeats(p, N):
+    import torch
+    nhmf = lib_or_fail()
+    prob, b = problem(nhmf, p, N, 0.01)
+    first = None
+    for _ in range(6):
+        x = torch.empty_like(b)
+        it = prob.linear_solve(b, x, solver=nhmf.NHMF_SOLVER_MIXED_GMG, linear_rtol=1e-10)
+        assert first is None or (torch.equal(x, first[0]) and it == first[1])
+        first = first or (x, it)
+    prob.close()
