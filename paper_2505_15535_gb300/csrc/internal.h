@@ -92,10 +92,12 @@ struct SolverWork {
   double* host = nullptr;      // pinned host scalars, kHostSlots of them
   cudaStream_t stream = nullptr;  // the solvers' own stream (graph capture needs a non-legacy stream)
   cudaEvent_t ev_in = nullptr, ev_out = nullptr;
-  // CUDA graphs of `check_every` CG iterations, keyed by the buffers they were captured with
+  // CUDA graphs of `check_every` CG iterations, keyed by everything the captured launches carry that
+  // can change between solves: the buffers, and the context's caches and material factors
   struct Graph {
     cudaGraphExec_t exec = nullptr;
-    const void* key[16] = {};
+    static constexpr int kKeys = 19;
+    const void* key[kKeys] = {};
   } graph[2];  // [0] FP64, [1] FP32
 };
 }  // namespace nhmf

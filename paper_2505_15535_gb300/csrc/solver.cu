@@ -136,10 +136,12 @@ cudaGraphExec_t chunk_graph(Ctx& x, int strat, T* sol, T* r, T* z, T* p, T* q, c
                             double* rz1, double* pq, double* rr, int chunk) {
   nhmf_ctx* c = x.c;
   SolverWork::Graph& G = x.w.graph[sizeof(T) == 4 ? 1 : 0];
-  const void* key[16] = {sol, r, z, p, q, dinv, rz0, rz1, pq, rr, (const void*)(long long)chunk,
-                         (const void*)(long long)strat, c->ubar, c->ubar32, c->cache64, c->cache32};
+  constexpr int kKeys = SolverWork::Graph::kKeys;
+  const void* key[kKeys] = {sol, r, z, p, q, dinv, rz0, rz1, pq, rr, (const void*)(long long)chunk,
+                            (const void*)(long long)strat, c->ubar, c->ubar32, c->cache64, c->cache32,
+                            c->cachesp, c->factor, c->vloc};
   bool same = G.exec != nullptr;
-  for (int i = 0; i < 16 && same; ++i) same = G.key[i] == key[i];
+  for (int i = 0; i < kKeys && same; ++i) same = G.key[i] == key[i];
   if (same) return G.exec;
   if (G.exec) {
     cudaGraphExecDestroy(G.exec);
@@ -165,7 +167,7 @@ cudaGraphExec_t chunk_graph(Ctx& x, int strat, T* sol, T* r, T* z, T* p, T* q, c
     return nullptr;
   }
   G.exec = exec;
-  for (int i = 0; i < 16; ++i) G.key[i] = key[i];
+  for (int i = 0; i < kKeys; ++i) G.key[i] = key[i];
   return exec;
 }
 
