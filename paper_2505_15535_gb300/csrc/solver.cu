@@ -73,9 +73,13 @@ nhmf_status ensure_work(nhmf_ctx* c) {
     if (cudaMalloc(p, n * sizeof(float)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "solver work alloc");
   if (cudaMalloc(&w.sc, 64 * sizeof(double)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "solver scalars");
   if (cudaMalloc(&w.partials, kPartialSlots * sizeof(double)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "partials");
-  cudaMemset(w.partials, 0, kPartialSlots * sizeof(double));
   if (cudaMallocHost(&w.host, kHostSlots * sizeof(double)) != cudaSuccess) return fail(c, NHMF_ERR_OOM, "pinned scalar");
-  cudaMemset(w.sc, 0, 64 * sizeof(double));
+  // cleared on the default stream, which the solvers' stream does not wait for by itself: the
+  // reductions' counter has to be zero before their first use (as has a multigrid level's status
+  // word, cleared when its context was created just before)
+  if (cudaMemset(w.partials, 0, kPartialSlots * sizeof(double)) != cudaSuccess ||
+      cudaMemset(w.sc, 0, 64 * sizeof(double)) != cudaSuccess || cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
+    return fail(c, NHMF_ERR_CUDA, "solver scalars");
   if (cudaStreamCreateWithFlags(&w.stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&w.ev_in, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&w.ev_out, cudaEventDisableTiming) != cudaSuccess)

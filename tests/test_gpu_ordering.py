@@ -65,3 +65,25 @@ def test_multigrid_repeats(p, N):
         assert first is None or (torch.equal(x, first[0]) and it == first[1])
         first = first or (x, it)
     prob.close()
+
+
+@pytest.mark.parametrize("solver", ["NHMF_SOLVER_JACOBI_CG", "NHMF_SOLVER_MIXED_GMG"])
+def test_first_solve_beside_a_busy_default_stream(solver):
+    """A context's first solve clears its reduction scratch and builds its hierarchy; on a side stream
+    this is ordered although the default stream is still busy with something else."""
+    import torch
+    nhmf = lib_or_fail()
+    results = []
+    for busy in (False, True, True):
+        prob, b = problem(nhmf, 2, 6, 0.01)
+        x = torch.empty_like(b)
+        side = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        if busy:
+            torch.cuda._sleep(400_000_000)   # about 0.2 s
+        with torch.cuda.stream(side):
+            it = prob.linear_solve(b, x, solver=getattr(nhmf, solver), linear_rtol=1e-10)
+        torch.cuda.synchronize()
+        results.append((it, x))
+        prob.close()
+    assert all(it == results[0][0] and torch.equal(x, results[0][1]) for it, x in results[1:])
