@@ -26,7 +26,7 @@ namespace cg = cooperative_groups;
 constexpr int kRow = 81;             // entries of a matrix row: 27 neighbours x 3 components
 constexpr int kCgThreads = 512;
 constexpr int kLanes = 4;            // lanes per row
-constexpr size_t kCgSmemMax = 220 * 1024;
+constexpr size_t kCgSmemMax = 220 * 1024;  // most dynamic shared memory of a block
 
 struct ElemArgs {
   int N, model;
@@ -411,11 +411,12 @@ size_t cg_smem(int n, int M, int R, int Rpad, bool rows) {
          (n + 2 * pad + 4 * (size_t)R + (rows ? (size_t)kRow * Rpad : 0)) * sizeof(T);
 }
 
+// The kernel's limits belong to the device, not to one hierarchy: every set-up sets the same ones, so
+// that none lowers what another one, alive beside it, launches with.
 template <typename T>
-cudaError_t allow(int blocks, size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_coarse_cg<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && blocks > 8)
-    e = cudaFuncSetAttribute(k_coarse_cg<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+cudaError_t allow() {
+  cudaError_t e = cudaFuncSetAttribute(k_coarse_cg<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCgSmemMax);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_coarse_cg<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   return e;
 }
 
@@ -443,7 +444,7 @@ bool cluster_fits(const CoarseSolve& C, int n, int M) {
   bool in_smem;
   const cudaLaunchConfig_t cfg = cg_config<T>(C, n, M, &attr, &in_smem, nullptr);
   int clusters = 0;
-  const bool ok = allow<T>(C.blocks, cfg.dynamicSmemBytes) == cudaSuccess &&
+  const bool ok = allow<T>() == cudaSuccess &&
                   cudaOccupancyMaxActiveClusters(&clusters, k_coarse_cg<T>, &cfg) == cudaSuccess && clusters > 0;
   if (!ok) cudaGetLastError();
   return ok;
