@@ -8,11 +8,13 @@
 // direction and the partial sums through distributed shared memory.  The host neither launches
 // nor reads anything per iteration.
 //
-// What bounds it: latency.  An iteration is an 81-term row product, two reductions and two divisions in
-// one warp (rows are spread over blocks at about 200 per block) and two barriers of the block or
-// three of the cluster, against 70 us for the same iteration as six launches.
+// What bounds it: latency.  An iteration is an 81-term row product, two FP64 reductions and two
+// divisions in one warp (about 45 dependent FP64 operations; rows are spread over blocks at about 200
+// per block) and two barriers of the block or three of the cluster, against 70 us for the same
+// iteration as six launches.  The sums are FP64 also in the FP32 solve: as pairs of FP32 numbers they
+// took 1.4 us less an iteration (linear solve Q4 16^3 77.3 ms against 85.4), but had four bits fewer
+// and FP32's exponent range, which the squares of a stiff material's system leave.
 #include <algorithm>
-#include <cmath>
 #include <cooperative_groups.h>
 
 #include "gmg.h"
@@ -129,9 +131,9 @@ __global__ void __launch_bounds__(64) k_coarse_elements(const ElemArgs a) {
 // Rows of the constrained operator P_f K P_f + P_D from the element matrices, in the solve's layout
 // [block][81 entries][Rpad rows]: entry 3 nb + k of row (c, node) is the coupling to component
 // k of neighbour nb = (dx + 1) + 3 (dy + 1) + 9 (dz + 1); 0 outside the mesh.  An entry sums its
-// elements in increasing order.  The FP32 copy holds 2^-k times the entries.
+// elements in increasing order.
 __global__ void k_coarse_rows(const double* __restrict__ Ke, int N, int bc, int R, int Rpad, int blocks,
-                              double down, double* __restrict__ A64, float* __restrict__ A32) {
+                              double* __restrict__ A64, float* __restrict__ A32) {
   const int M = N + 1, M3 = M * M * M, n = 3 * M3;
   const int id = blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= blocks * kRow * Rpad) return;
@@ -153,7 +155,7 @@ __global__ void k_coarse_rows(const double* __restrict__ Ke, int N, int bc, int 
     }
   }
   A64[id] = v;
-  A32[id] = float(v * down);
+  A32[id] = float(v);
 }
 
 template <typename T>
@@ -161,65 +163,27 @@ struct CgArgs {
   const T *A, *b, *dinv;
   T* x;
   int n, M, R, Rpad, in_smem;        // DoFs, nodes per direction, rows per block and their padding
-  T up, down;                        // 2^k and 2^-k of the scaled system (see scale_exponent)
   double rtol;
   int maxit, check;
   unsigned long long* words;         // [0] += iterations, [1] |= status flags
 };
 
-// The solve's scalars: sums of products over the rows, kept by warp 0.  In FP64 a plain sum.  In FP32 the
-// products of two FP32 numbers and their sum in double-float arithmetic: the exact products by
-// FMA, the sum by TwoSum with its errors (49 bits; the step lengths made from it are FP32
-// numbers), because an iteration in FP64 is a chain of about 45 operations of that slow pipe, 3.7
-// us against 1.
-template <typename T> struct Sum;
-template <> struct Sum<double> {
-  double v = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { v = fma(a, b, v); }
-  __device__ __forceinline__ void add(const Sum& o) { v += o.v; }
-  __device__ __forceinline__ Sum from(int lane_xor) const {
-    Sum o;
-    o.v = __shfl_xor_sync(0xffffffffu, v, lane_xor);
-    return o;
+// x / y rounded to T, the step lengths from the FP64 sums.  In FP32 by the reciprocal (two units in the
+// last of 53 bits before the rounding to 24) where it is in range: half the latency of a division.
+template <typename T>
+__device__ __forceinline__ T quotient(double x, double y) {
+  if constexpr (sizeof(T) == 4) {
+    const double m = fabs(y);
+    if (m > 0x1p-1000 && m < 0x1p1000) return T(x * fast_rcp(y));
   }
-  __device__ __forceinline__ double value() const { return v; }
-  __device__ __forceinline__ bool positive() const { return v > 0.0 && isfinite(v); }
-  __device__ __forceinline__ bool finite() const { return isfinite(v); }
-  __device__ __forceinline__ static double quotient(const Sum& x, const Sum& y) { return x.v / y.v; }
-};
-template <> struct Sum<float> {
-  float s = 0.f, l = 0.f;
-  __device__ __forceinline__ void add(float a, float b) {
-    float t;
-    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
-    s = two_sum(s, p, t);
-    l = __fadd_rn(l, __fadd_rn(t, e));
-  }
-  __device__ __forceinline__ void add(const Sum& o) {
-    float t;
-    s = two_sum(s, o.s, t);
-    l = __fadd_rn(__fadd_rn(l, o.l), t);
-  }
-  __device__ __forceinline__ Sum from(int lane_xor) const {
-    Sum o;
-    o.s = __shfl_xor_sync(0xffffffffu, s, lane_xor);
-    o.l = __shfl_xor_sync(0xffffffffu, l, lane_xor);
-    return o;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)l; }
-  __device__ __forceinline__ bool positive() const { return s > 0.f && isfinite(s); }
-  __device__ __forceinline__ bool finite() const { return isfinite(s); }
-  // x / y from the quotient of the high parts and one correction by the remainder
-  __device__ __forceinline__ static float quotient(const Sum& x, const Sum& y) {
-    const float q = x.s / y.s, r = fmaf(-q, y.s, x.s) + fmaf(-q, y.l, x.l);
-    return q + r / y.s;
-  }
-};
+  return T(x / y);
+}
 
 // Jacobi-CG from x = 0 to ||r|| <= rtol ||b||, tested every `check` iterations as pcg() does;
 // p.q <= 0 or a non-finite residual is recorded in the status word and ends the solve.  One
 // cluster; block `rank` owns rows [rank R, rank R + R).  All warps of a block form q = A p; warp 0
-// alone does the vector updates, the sums and the scalars, so that a reduction is five shuffles.
+// alone does the vector updates, the sums and the scalars, so that a reduction is five shuffles
+// and the divisions are issued once.
 template <typename T>
 __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
   extern __shared__ __align__(16) unsigned char sm[];
@@ -227,7 +191,7 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
   const int rank = (int)cl.block_rank(), nblk = (int)cl.num_blocks(), tid = threadIdx.x, nthr = blockDim.x;
   const int M = a.M, M3 = M * M * M, pad = M * M + M + 1, R = a.R, Rpad = a.Rpad;
   const int row0 = rank * R, rows = max(0, min(R, a.n - row0));
-  Sum<T>* part = reinterpret_cast<Sum<T>*>(sm);      // [2][16][2] sums of the cluster's blocks, double buffered
+  double* part = reinterpret_cast<double*>(sm);      // [2][16][2] sums of the cluster's blocks, double buffered
   int* stop = reinterpret_cast<int*>(part + 64);     // [1] (+ 1)
   int* off = stop + 2;                               // [81] (+ 1)
   T* p = reinterpret_cast<T*>(off + 82) + pad;       // [n], `pad` zeros on either side
@@ -254,15 +218,15 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
   int buf = 0;
   // Sums of warp 0's two values over the cluster, in a fixed order, in warp 0 of every block; with
   // more than one block every thread has to call it.
-  auto sum2 = [&](Sum<T>& v0, Sum<T>& v1) {
+  auto sum2 = [&](double& v0, double& v1) {
     if (tid < 32) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        v0.add(v0.from(o));
-        v1.add(v1.from(o));
+        v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
       }
       if (nblk > 1 && tid < nblk) {
-        Sum<T>* dst = cl.map_shared_rank(part, tid) + 32 * buf + 2 * rank;
+        double* dst = cl.map_shared_rank(part, tid) + 32 * buf + 2 * rank;
         dst[0] = v0;
         dst[1] = v1;
       }
@@ -270,26 +234,23 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
     if (nblk == 1) return;
     cl.sync();
     if (tid < 32) {
-      v0 = v1 = Sum<T>();
-      if (tid < nblk) {
-        v0 = part[32 * buf + 2 * tid];
-        v1 = part[32 * buf + 2 * tid + 1];
-      }
+      v0 = tid < nblk ? part[32 * buf + 2 * tid] : 0.0;
+      v1 = tid < nblk ? part[32 * buf + 2 * tid + 1] : 0.0;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
-        v0.add(v0.from(o));
-        v1.add(v1.from(o));
+        v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+        v1 += __shfl_xor_sync(0xffffffffu, v1, o);
       }
     }
     buf ^= 1;
   };
-  auto sum1 = [&](Sum<T>& v) {
+  auto sum1 = [&](double& v) {
     if (nblk > 1) {
-      Sum<T> unused;
+      double unused = 0.0;
       sum2(v, unused);
     } else if (tid < 32) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v.add(v.from(o));
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     }
   };
   // p over the whole cluster: own row i gets v
@@ -297,21 +258,21 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
     for (int k = 0; k < nblk; ++k) (nblk == 1 ? p : cl.map_shared_rank(p, k))[row0 + i] = v;
   };
   barrier();  // every block's arrays exist and are initialised
-  Sum<T> v0, v1;
+  double v0 = 0.0, v1 = 0.0;
   if (tid < 32)
     for (int i = tid; i < rows; i += 32) {
-      const T bi = a.b[row0 + i], d = a.dinv[row0 + i] * a.up, zi = d * bi;
+      const T bi = a.b[row0 + i], d = a.dinv[row0 + i], zi = d * bi;
       x[i] = T(0);
       r[i] = bi;
       di[i] = d;
-      v0.add(bi, zi);
-      v1.add(bi, bi);
+      v0 = fma(double(bi), double(zi), v0);
+      v1 = fma(double(bi), double(bi), v1);
       set_p(i, zi);
     }
   sum2(v0, v1);
-  Sum<T> rz = v0;
-  const double bn = sqrt(v1.value());
-  unsigned flag = v1.finite() ? 0u : kStatusNonFinite;
+  double rz = v0;
+  const double bn = sqrt(v1);
+  unsigned flag = isfinite(v1) ? 0u : kStatusNonFinite;
   if (tid == 0 && (!(bn > 0.0) || flag)) *stop = 1;  // the same in every block
   barrier();                                         // also orders the writes of p before the reads below
   int k = 0;
@@ -359,21 +320,21 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
     }
     ++k;
     __syncthreads();
-    v0 = v1 = Sum<T>();
+    v0 = v1 = 0.0;
     if (tid < 32)
-      for (int i = tid; i < rows; i += 32) v0.add(p[row0 + i], q[i]);
+      for (int i = tid; i < rows; i += 32) v0 = fma(double(p[row0 + i]), double(q[i]), v0);
     sum1(v0);
-    const bool ok = v0.positive();  // warp 0
+    const bool ok = v0 > 0.0 && isfinite(v0);  // warp 0
     if (tid < 32) {
-      const T alpha = ok ? Sum<T>::quotient(rz, v0) : T(0);
-      v0 = Sum<T>();
+      const T alpha = ok ? quotient<T>(rz, v0) : T(0);
+      v0 = 0.0;
       for (int i = tid; i < rows; i += 32) {
         x[i] = fma(alpha, p[row0 + i], x[i]);
         const T ri = fma(-alpha, q[i], r[i]), zi = di[i] * ri;
         r[i] = ri;
         q[i] = zi;
-        v0.add(ri, zi);
-        v1.add(ri, ri);
+        v0 = fma(double(ri), double(zi), v0);
+        v1 = fma(double(ri), double(ri), v1);
       }
     }
     sum2(v0, v1);
@@ -382,20 +343,20 @@ __global__ void __launch_bounds__(kCgThreads) k_coarse_cg(const CgArgs<T> a) {
       if (!ok) {
         flag = kStatusBreakdown;
       } else if (k % a.check == 0 || k == a.maxit) {
-        if (!v1.finite()) flag = kStatusNonFinite;
-        end = flag || sqrt(v1.value()) <= a.rtol * bn;
+        if (!isfinite(v1)) flag = kStatusNonFinite;
+        end = flag || sqrt(v1) <= a.rtol * bn;
       }
       if (end) {
         if (tid == 0) *stop = 1;
       } else {
-        const T beta = Sum<T>::quotient(v0, rz);
+        const T beta = quotient<T>(v0, rz);
         rz = v0;
         for (int i = tid; i < rows; i += 32) set_p(i, fma(beta, p[row0 + i], q[i]));
       }
     }
     barrier();
   }
-  for (int i = tid; i < rows; i += nthr) a.x[row0 + i] = x[i] * a.down;
+  for (int i = tid; i < rows; i += nthr) a.x[row0 + i] = x[i];
   if (rank == 0 && tid == 0) {
     a.words[0] += (unsigned long long)k;
     a.words[1] |= flag;
@@ -481,14 +442,6 @@ void coarse_free(Gmg& G) {
   G.coarse = CoarseSolve{};
 }
 
-namespace {
-// The FP32 solve runs on 2^-k A and 2^k x, with 2^k near the size of A's diagonal, so that its sums of
-// products stay inside the FP32 range for every material; powers of two change no digit.
-int scale_exponent(const nhmf_ctx* c) {
-  return std::max(-120, std::min(120, std::ilogb(c->prm.mu * c->g.h)));
-}
-}  // namespace
-
 nhmf_status coarse_assemble(Gmg& G, cudaStream_t s) {
   GmgLevel& L = G.L[0];
   const CoarseSolve& C = G.coarse;
@@ -511,8 +464,7 @@ nhmf_status coarse_assemble(Gmg& G, cudaStream_t s) {
   a.Ke = C.Ke;
   k_coarse_elements<<<(unsigned)c->g.E, 64, 0, s>>>(a);
   const int entries = C.blocks * kRow * C.Rpad;
-  k_coarse_rows<<<(entries + 255) / 256, 256, 0, s>>>(C.Ke, a.N, c->prm.bc, C.R, C.Rpad, C.blocks,
-                                                      std::ldexp(1.0, -scale_exponent(c)), C.A64, C.A32);
+  k_coarse_rows<<<(entries + 255) / 256, 256, 0, s>>>(C.Ke, a.N, c->prm.bc, C.R, C.Rpad, C.blocks, C.A64, C.A32);
   return cuda_check(L.ctx, cudaGetLastError(), "coarse matrix");
 }
 
@@ -529,9 +481,6 @@ nhmf_status coarse_cg(Gmg& G, const T* b, T* x, double rtol, int maxit, int chec
   a.M = L.M;
   a.R = C.R;
   a.Rpad = C.Rpad;
-  const int k = sizeof(T) == 4 ? scale_exponent(L.ctx) : 0;
-  a.up = T(std::ldexp(1.0, k));
-  a.down = T(std::ldexp(1.0, -k));
   a.rtol = rtol;
   a.maxit = maxit;
   a.check = check;
