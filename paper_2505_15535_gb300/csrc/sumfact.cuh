@@ -397,27 +397,23 @@ __device__ __forceinline__ void colloc_grad_T(const T* __restrict__ Dc, const T*
 // instructions.  CUDA's 1 / x and log1p took about 70 of them at a point; the two below take 16.
 
 // 1 / x by Newton's iteration, third order: y0 = rcp.approx(x) (relative error below 2^-20), e = 1 -
-// x y0, y = y0 (1 + e + e^2) with error e^3 < 2^-60 before rounding.  x a normal number whose
-// reciprocal is normal.
+// x y0, y = y0 (1 + e + e^2) with error e^3 < 2^-60 before rounding.  x and its reciprocal are
+// normal numbers.
 __device__ __forceinline__ double fast_rcp(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ float fast_rcp(float x) { return 1.f / x; }
 
 // log1p(x) given J = 1 + x, table driven (P. T. P. Tang, "Table-driven implementation of the
 // logarithm function in IEEE floating-point arithmetic", ACM TOMS 16, 1990): J = 2^k m with m in
 // [0.75, 1.5), c from the table near 1 / m, r = c 2^-k (1 + x) - 1 from x itself (one rounding, so
 // small x keep their relative accuracy; c = 1 next to J = 1), |r| <= 2^-7, and log1p(x) = k ln 2 -
-// ln c + log1p(r) with the series to r^8 (next term below 2^-66).  J not positive, not finite or
-// subnormal goes to CUDA's function.
+// ln c + log1p(r) with the series to r^8 (next term below 2^-66).  J in [2^-1000, 2^1000].
 #include "log_table.h"
 __device__ __forceinline__ double fast_log1p(double x, double J) {
-  const int hi = __double2hiint(J);
-  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log1p(x);
-  const int t = hi - 0x3fe80000, k = t >> 20, i = (t >> 13) & 127;  // m >= 0.75: exponent field of 0.75
+  const int t = __double2hiint(J) - 0x3fe80000, k = t >> 20, i = (t >> 13) & 127;  // m >= 0.75: exponent field of 0.75
   double c = __ldg(&kLogTable[i][0]), l = __ldg(&kLogTable[i][1]);
   if (k != 0) {
     c *= __hiloint2double((1023 - k) << 20, 0);
@@ -432,12 +428,16 @@ __device__ __forceinline__ double fast_log1p(double x, double J) {
   p = fma(r, p, -1.0 / 2.0);
   return l + fma(r * r, p, r);
 }
-__device__ __forceinline__ float fast_log1p(float x, float) { return log1pf(x); }
+
+// J in [2^-500, 2^500): positive, and 1 / J^2 is a normal number too.
+__device__ __forceinline__ bool ordinary(double J) { return (unsigned)(__double2hiint(J) - (523 << 20)) < 1000u << 20; }
 
 // Kinematics at a point from the physical displacement gradient H (row-major H[3c+d]), F = I + H:
 // the adjugate A = J F^-1, 1 / J, ln J and J - 1.  With C00 - 1 = H4 + H8 + H4 H8 - H5 H7,
 //   J - 1 = H0 + F0 (C00 - 1) + H1 C01 + H2 C02
-// has no cancellation near F = I (25 operations for A and J - 1).
+// has no cancellation near F = I (25 operations for A and J - 1).  F^-1 = A invJ always.  In FP64, where
+// J is not ordinary (not positive, not finite, or so large that the point code's 1 / J^2 would
+// underflow while F^-1 is still an ordinary number), A is F^-1 itself and invJ is 1.
 template <typename T>
 struct Kinematics {
   T A[9], invJ, lnJ, Jm1;
@@ -456,8 +456,21 @@ struct Kinematics {
     A[8] = fma(F0, F4, -(H[1] * H[3]));
     Jm1 = fma(F0, C, fma(H[1], A[3], fma(H[2], A[6], H[0])));
     const T J = T(1) + Jm1;
-    invJ = fast_rcp(J);
-    lnJ = fast_log1p(Jm1, J);
+    if constexpr (sizeof(T) == 8) {
+      if (ordinary(J)) {
+        invJ = fast_rcp(J);
+        lnJ = fast_log1p(Jm1, J);
+      } else {
+        const T inv = 1.0 / J;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) A[k] *= inv;
+        invJ = 1.0;
+        lnJ = log1p(Jm1);
+      }
+    } else {
+      invJ = T(1) / J;
+      lnJ = log1pf(Jm1);
+    }
   }
 };
 
