@@ -1114,25 +1114,32 @@ __device__ __forceinline__ void frag_channel_sums(uint32_t a0, uint32_t a1, uint
   sg += (__low2float(x0) + __high2float(x0)) + (__low2float(x2) + __high2float(x2));
   sg8 += (__low2float(x1) + __high2float(x1)) + (__low2float(x3) + __high2float(x3));
 }
-// All WARPS warps: the block's 16 channel totals (per warp the 4 lanes of each channel, then the
-// warps in order) to bpartial[blockIdx.x][16].  Ends with a block barrier.
-template <int WARPS>
-__device__ __forceinline__ void bias_partial_store(float sg, float sg8, float* bpartial) {
-  __shared__ float bsh[WARPS][16];
-  sg += __shfl_xor_sync(0xffffffffu, sg, 1);
-  sg8 += __shfl_xor_sync(0xffffffffu, sg8, 1);
-  sg += __shfl_xor_sync(0xffffffffu, sg, 2);
-  sg8 += __shfl_xor_sync(0xffffffffu, sg8, 2);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if ((lane & 3) == 0) {
-    bsh[warp][lane >> 2] = sg;
-    bsh[warp][(lane >> 2) + 8] = sg8;
+// The bias gradient of a block is kBiasSums running sums per lane and channel, chunk j of 16 positions
+// in sum j % kBiasSums: so many short FP32 chains, whatever the number of warps that hold them.
+constexpr int kBiasSums = 9;
+// All warps, K sums each (sum i of the thread is number row[i]): the block's 16 channel totals (per
+// sum the 4 lanes of each channel, then the sums in order) to bpartial[blockIdx.x][16].  Ends with
+// a block barrier.
+template <int K>
+__device__ __forceinline__ void bias_partial_store(float (&sg)[K], float (&sg8)[K], const int (&row)[K], float* bpartial) {
+  __shared__ float bsh[kBiasSums][16];
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < K; ++i) {
+    sg[i] += __shfl_xor_sync(0xffffffffu, sg[i], 1);
+    sg8[i] += __shfl_xor_sync(0xffffffffu, sg8[i], 1);
+    sg[i] += __shfl_xor_sync(0xffffffffu, sg[i], 2);
+    sg8[i] += __shfl_xor_sync(0xffffffffu, sg8[i], 2);
+    if ((lane & 3) == 0) {
+      bsh[row[i]][lane >> 2] = sg[i];
+      bsh[row[i]][(lane >> 2) + 8] = sg8[i];
+    }
   }
   __syncthreads();
   if (threadIdx.x < 16) {
     float t = 0.f;
 #pragma unroll
-    for (int w = 0; w < WARPS; ++w) t += bsh[w][threadIdx.x];
+    for (int w = 0; w < kBiasSums; ++w) t += bsh[w][threadIdx.x];
     bpartial[blockIdx.x * 16 + threadIdx.x] = t;
   }
 }
@@ -1177,7 +1184,11 @@ __global__ void __launch_bounds__(kWg1Threads, kWg1Blocks) k_wgrad_s1(const __nv
   const int per_plane = (m * R + 127) / 128, nzc = (m + zc - 1) / zc;
   const long long nunits = (long long)per_plane * nstrips * nzc;
   float acc[3][3][NT][4] = {};  // [dz + 1][dx + 1][n-tile]
-  float bsg = 0.f, bsg8 = 0.f;  // channels g, g + 8 of P over this warp's chunks (bias gradient, dy = dz = 0)
+  // channels g, g + 8 of P over this warp's chunks (bias gradient): chunk j goes to warp j % 3, whose
+  // three sums take its chunks in turn (the next one's sum is always [0])
+  static_assert(kBiasSums == 3 * (kWg1Threads / 32), "three sums a warp");
+  float bsg[3] = {}, bsg8[3] = {};
+  int turn = 0, added = 0;
   // ldmatrix row of this lane: matrix lane / 8, row lane % 8
   const int lm = lane >> 3, lr = lane & 7;
   for (long long unit = blockIdx.x; unit < nunits; unit += gridDim.x) {
@@ -1229,13 +1240,27 @@ __global__ void __launch_bounds__(kWg1Threads, kWg1Blocks) k_wgrad_s1(const __nv
                 mma16816(acc[d][dx][h], a[d][0], a[d][1], a[d][2], a[d][3], b[2 * h], b[2 * h + 1]);
             }
         }
-        if (bpartial && dyi == 1 && on[1]) frag_channel_sums(a[1][0], a[1][1], a[1][2], a[1][3], bsg, bsg8);
+        if (bpartial && on[1]) {
+          if (turn == warp) {
+            float s0 = bsg[0], s8 = bsg8[0];
+            frag_channel_sums(a[1][0], a[1][1], a[1][2], a[1][3], s0, s8);
+            bsg[0] = bsg[1], bsg[1] = bsg[2], bsg[2] = s0;
+            bsg8[0] = bsg8[1], bsg8[1] = bsg8[2], bsg8[2] = s8;
+            ++added;
+          }
+          turn = turn == 2 ? 0 : turn + 1;
+        }
       }
       cp_async_wait_all();
       __syncthreads();
     }
   }
-  if (bpartial) bias_partial_store<kWg1Threads / 32>(bsg, bsg8, bpartial);
+  if (bpartial) {
+    int row[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) row[i] = warp + 3 * ((added + i) % 3);
+    bias_partial_store<3>(bsg, bsg8, row, bpartial);
+  }
   float* out = partial + (long long)blockIdx.x * 27 * 256;
 #pragma unroll
   for (int d = 0; d < 3; ++d)
@@ -1290,8 +1315,9 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_s2(const __nv_bfloat16* __
   const long long nunits = (long long)mp * nseg * nzc;
   float acc[3][2][4] = {};
   unsigned tt = 0;  // coarse planes done by this block; the P rows of plane tt are in buffer tt & 1
-  float bsg = 0.f, bsg8 = 0.f;  // channels g, g + 8 of P over this warp's share of the chunks (bias gradient)
-  unsigned chunk = 0;            // chunks of 16 positions done by this block; chunk % 9 adds its fragments
+  static_assert(kBiasSums == kWgThreads / 32, "one sum a warp");
+  float bsg[1] = {}, bsg8[1] = {};  // channels g, g + 8 of P over this warp's share of the chunks (bias gradient)
+  unsigned chunk = 0;               // chunks of 16 positions done by this block; warp chunk % 9 adds its fragments
   // fine rows 2 cy - 1 .. 2 cy + 1 of fine plane f over fine x 2 x0 - 1 .. 2 x0 + 2 seg - 1
   auto stage_fine = [&](int f, int cy, int x0) {
     const uint32_t d = smem_u32(slot(f));
@@ -1360,14 +1386,17 @@ __global__ void __launch_bounds__(kWgThreads) k_wgrad_s2(const __nv_bfloat16* __
           mma16816(acc[jt][1], a0, a1, a2, a3, b2, b3);
         }
         // the bias gradient's share, after the MMAs have consumed the fragment
-        if (bpartial && chunk % (kWgThreads / 32) == (unsigned)warp) frag_channel_sums(a0, a1, a2, a3, bsg, bsg8);
+        if (bpartial && chunk % kBiasSums == (unsigned)warp) frag_channel_sums(a0, a1, a2, a3, bsg[0], bsg8[0]);
         ++chunk;
       }
       cp_async_wait_all();
       __syncthreads();
     }
   }
-  if (bpartial) bias_partial_store<kWgThreads / 32>(bsg, bsg8, bpartial);
+  if (bpartial) {
+    const int row[1] = {warp};
+    bias_partial_store<1>(bsg, bsg8, row, bpartial);
+  }
   float* out = partial + (long long)blockIdx.x * 27 * 256;
 #pragma unroll
   for (int jt = 0; jt < 3; ++jt) {
