@@ -413,25 +413,26 @@ bool cluster_fits(const CoarseSolve& C, int n, int M) {
 
 }  // namespace
 
-bool coarse_setup(Gmg& G) {
+void coarse_setup(Gmg& G) {
   GmgLevel& L = G.L[0];
   CoarseSolve& C = G.coarse;
-  if (cudaMalloc(&C.words, 2 * sizeof(unsigned long long)) != cudaSuccess) return false;
-  if (L.ctx->g.p != 1 || L.ctx->g.N > kCoarseMaxN) return true;
+  if (L.ctx->g.p != 1 || L.ctx->g.N > kCoarseMaxN) return;
   const int n = (int)L.n, M = L.M;
   // about 200 rows per block (the FP64 reductions), at most one cluster of 16
   C.blocks = 1;
   while (C.blocks < 16 && (n + C.blocks - 1) / C.blocks > 200) C.blocks *= 2;
   C.R = (n + C.blocks - 1) / C.blocks;
   C.Rpad = (C.R + 31 - 8) / 32 * 32 + 8;  // = 8 mod 32: the four lanes of a row read distinct banks
-  if (!cluster_fits<double>(C, n, M) || !cluster_fits<float>(C, n, M)) {
-    C.blocks = 0;  // the level is solved by pcg() on its operator
-    return true;
-  }
   const size_t entries = (size_t)C.blocks * kRow * C.Rpad;
-  return cudaMalloc(&C.Ke, (size_t)L.ctx->g.E * 576 * sizeof(double)) == cudaSuccess &&
-         cudaMalloc(&C.A64, entries * sizeof(double)) == cudaSuccess &&
-         cudaMalloc(&C.A32, entries * sizeof(float)) == cudaSuccess;
+  if (cluster_fits<double>(C, n, M) && cluster_fits<float>(C, n, M) &&
+      cudaMalloc(&C.words, 2 * sizeof(unsigned long long)) == cudaSuccess &&
+      cudaMalloc(&C.Ke, (size_t)L.ctx->g.E * 576 * sizeof(double)) == cudaSuccess &&
+      cudaMalloc(&C.A64, entries * sizeof(double)) == cudaSuccess &&
+      cudaMalloc(&C.A32, entries * sizeof(float)) == cudaSuccess)
+    return;
+  // no room on the chip or in memory (28 MB at 15^3): pcg() solves the level on its operator
+  cudaGetLastError();
+  coarse_free(G);
 }
 
 void coarse_free(Gmg& G) {

@@ -370,10 +370,7 @@ nhmf_status gmg_build(nhmf_ctx* c) {
       return fail(c, NHMF_ERR_OOM, "gmg: transfer maps");
     }
   }
-  if (!coarse_setup(G)) {
-    gmg_free(c);
-    return fail(c, NHMF_ERR_OOM, "gmg: coarse matrix");
-  }
+  coarse_setup(G);
   return NHMF_OK;
 }
 

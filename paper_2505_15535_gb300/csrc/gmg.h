@@ -86,7 +86,8 @@ template <typename T>
 void gmg_restrict(GmgLevel& F, GmgLevel& C, const T* r_fine, T* r_coarse, cudaStream_t s);
 template <typename T>
 void gmg_prolong_add(GmgLevel& F, GmgLevel& C, const T* e_coarse, T* x_fine, cudaStream_t s);
-bool coarse_setup(Gmg& G);
+// Memory and cluster shape of the coarsest level's solve; where they cannot be had, blocks stays 0.
+void coarse_setup(Gmg& G);
 void coarse_free(Gmg& G);
 // The coarsest operator's matrix at its level's linearisation point.
 nhmf_status coarse_assemble(Gmg& G, cudaStream_t s);
