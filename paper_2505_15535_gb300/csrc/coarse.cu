@@ -430,7 +430,7 @@ void coarse_setup(Gmg& G) {
       cudaMalloc(&C.A64, entries * sizeof(double)) == cudaSuccess &&
       cudaMalloc(&C.A32, entries * sizeof(float)) == cudaSuccess)
     return;
-  // no room on the chip or in memory (28 MB at 15^3): pcg() solves the level on its operator
+  // no room on the chip or in memory (18 MB at 13^3): pcg() solves the level on its operator
   cudaGetLastError();
   coarse_free(G);
 }

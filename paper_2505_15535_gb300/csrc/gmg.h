@@ -29,7 +29,11 @@ struct GmgLevel {
 };
 
 // The coarsest level's matrix and solve (coarse.cu).
-constexpr int kCoarseMaxN = 15;  // elements per direction up to which the level is a matrix
+// Elements per direction up to which the level is a matrix; above it the rows no longer stay in shared
+// memory and pcg() on the operator is as fast or faster.  Solves of a one-level hierarchy, matrix /
+// operator, in ms: FP64 7^3 2.8 / 7.6, 9^3 3.5 / 10.5, 11^3 6.4 / 11.9, 13^3 10.5 / 14.6, 15^3 17.3 / 17.6;
+// FP32 7^3 1.6 / 3.3, 9^3 1.9 / 4.4, 11^3 3.3 / 5.2, 13^3 4.6 / 5.6, 15^3 8.4 / 6.8.
+constexpr int kCoarseMaxN = 13;
 struct CoarseSolve {
   int blocks = 0;            // blocks of the solve's cluster; 0: the level is solved by pcg() on its operator
   int R = 0, Rpad = 0;       // rows per block, padded
