@@ -87,3 +87,39 @@ def test_first_solve_beside_a_busy_default_stream(solver):
         results.append((it, x))
         prob.close()
     assert all(it == results[0][0] and torch.equal(x, results[0][1]) for it, x in results[1:])
+
+
+@pytest.mark.parametrize("p,N", [(1, 9), (2, 6), (4, 5)])
+def test_applies_in_a_callers_capture(p, N):
+    """A caller's captured stream may hold anything before an apply: a copy, a memset, an event of
+    another stream.  The graph replays with the inputs of the moment."""
+    import torch
+    nhmf = lib_or_fail()
+    prob, d = problem(nhmf, p, N)
+    for prec, dt in ((nhmf.NHMF_FP64, torch.float64), (nhmf.NHMF_FP32, torch.float32)):
+        src = d.to(dt)
+        x, v, y, z = (torch.empty_like(src) for _ in range(4))
+        prob.apply(src, v, prec, 1)   # every kernel is loaded
+        torch.cuda.synchronize()
+        graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        with torch.cuda.graph(graph):
+            x.copy_(src)
+            prob.apply(x, v, prec, 1)      # behind a copy
+            y.zero_()
+            prob.apply(v, y, prec, 0)      # behind a memset of its own output
+            cur = torch.cuda.current_stream()
+            side.wait_stream(cur)
+            with torch.cuda.stream(side):
+                z.copy_(y)
+            cur.wait_stream(side)
+            prob.apply(z, v, prec, 1)      # behind another stream's event
+        for scale in (1.0, -2.0):
+            src.copy_(scale * d.to(dt))
+            graph.replay()
+            torch.cuda.synchronize()
+            a = prob.apply(src, torch.empty_like(src), prec, 1)
+            b = prob.apply(a, torch.empty_like(src), prec, 0)
+            c = prob.apply(b, torch.empty_like(src), prec, 1)
+            torch.cuda.synchronize()
+            assert torch.equal(y, b) and torch.equal(v, c), (prec, scale)
+    prob.close()
