@@ -173,7 +173,7 @@ __global__ void k_axpby(long long n, double sa, const double* pa, const double* 
     y[i] = b == 0.0 ? a * x[i] : fma(a, x[i], b * y[i]);
 }
 
-// out = num / den (device scalars), with a sign.
+// z = noise in [-1, 1) from a hash of the index and the seed.
 __global__ void k_noise(long long n, double* z, unsigned long long seed) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     unsigned long long v = (unsigned long long)i + seed * 0x9E3779B97F4A7C15ull;
@@ -182,10 +182,6 @@ __global__ void k_noise(long long n, double* z, unsigned long long seed) {
     v ^= v >> 31;
     z[i] = double(v >> 11) * 0x1.0p-52 - 1.0;
   }
-}
-
-__global__ void k_ratio(const double* num, const double* den, double sign, double* out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *out = sign * (*num / *den);
 }
 
 __global__ void k_ratio_or_zero(const double* num, const double* den, double* out) {
@@ -211,11 +207,6 @@ __global__ void k_reciprocal(long long n, const double* d, double* dinv64, float
     if (dinv64) dinv64[i] = v;
     if (dinv32) dinv32[i] = float(v);
   }
-}
-
-__global__ void k_mul(long long n, const double* d, double* x) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    x[i] *= d[i];
 }
 
 constexpr int kEwBlocks = 1216;  // 8 blocks per SM for element-wise kernels
@@ -283,9 +274,6 @@ template void jacobi<float>(long long, const float*, const float*, float*, doubl
 void axpby(long long n, double a, const double* pa, const double* x, double b, const double* pb, double* y, cudaStream_t s) {
   launch(k_axpby, dim3(ew_blocks(n)), kEwThreads, 0, s, true, n, a, pa, x, b, pb, y);
 }
-void ratio(const double* num, const double* den, double sign, double* out, cudaStream_t s) {
-  k_ratio<<<1, 32, 0, s>>>(num, den, sign, out);
-}
 void fill_noise(long long n, double* z, unsigned long long seed, cudaStream_t s) {
   k_noise<<<kRedBlocks, kRedThreads, 0, s>>>(n, z, seed);
 }
@@ -297,9 +285,6 @@ void to_fp32_scaled(long long n, const double* x, const double* scale, bool inve
 }
 void to_fp64_scaled(long long n, const float* x, const double* scale, double* y, cudaStream_t s) {
   launch(k_scale_convert<float, double>, dim3(ew_blocks(n)), kEwThreads, 0, s, true, n, x, scale, false, y);
-}
-void jacobi_apply(long long n, const double* dinv, double* x, cudaStream_t s) {
-  k_mul<<<kEwBlocks, kEwThreads, 0, s>>>(n, dinv, x);
 }
 void reciprocal(long long n, const double* d, double* dinv64, float* dinv32, cudaStream_t s) {
   k_reciprocal<<<kEwBlocks, kEwThreads, 0, s>>>(n, d, dinv64, dinv32);

@@ -196,9 +196,8 @@ nhmf_status launch_apply(nhmf_ctx* c, int precision, int strategy, const void* d
 nhmf_status launch_apply32(nhmf_ctx* c, int strategy, const float* du, float* v, const Gather32& g32, cudaStream_t s);
 // nhmf_set_linearization without reading the status word: the caller does (asynchronous).
 nhmf_status set_linearization_async(nhmf_ctx* c, const double* u, int mask, cudaStream_t s);
-// On every constrained DoF: out = src (mode 0) or out = value (mode 1).
-nhmf_status fix_rows64(nhmf_ctx* c, const double* src, double* out, int mode, double value, cudaStream_t s);
-nhmf_status fix_rows32(nhmf_ctx* c, const float* src, float* out, int mode, float value, cudaStream_t s);
+// out = src on every constrained DoF.
+nhmf_status fix_rows64(nhmf_ctx* c, const double* src, double* out, cudaStream_t s);
 nhmf_status launch_cache_build(nhmf_ctx* c, cudaStream_t s);
 nhmf_status launch_residual(nhmf_ctx* c, const double* u, double* r, cudaStream_t s);
 nhmf_status launch_diagonal(nhmf_ctx* c, double* d, cudaStream_t s);

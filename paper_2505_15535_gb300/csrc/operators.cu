@@ -7,17 +7,13 @@ namespace nhmf {
 namespace {
 
 // ------------------------------------------------------------------ Dirichlet rows
-// mode 0: out[d] = src[d]; mode 1: out[d] = value, on every constrained DoF.
-template <typename T>
-__global__ void k_fix_constrained(int bc, int M, long long M3, const T* src, T* out, int mode, T value) {
+// out[d] = src[d] on every constrained DoF.
+__global__ void k_fix_constrained(int bc, int M, long long M3, const double* src, double* out) {
   const long long f = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long M2 = (long long)M * M;
   if (f >= M2) return;
   const int x = int(f % M), y = int(f / M);
-  auto fix = [&](int c, long long node) {
-    const long long d = c * M3 + node;
-    out[d] = mode == 0 ? src[d] : value;
-  };
+  auto fix = [&](int c, long long node) { out[c * M3 + node] = src[c * M3 + node]; };
   if (bc == NHMF_BC_CLAMP_X0) {
     const long long node = (long long)M * (x + (long long)M * y);  // (0, x, y)
     for (int c = 0; c < 3; ++c) fix(c, node);
@@ -35,17 +31,6 @@ __global__ void k_to_fp32(const double* x, float* y, long long n) {
     y[i] = float(x[i]);
 }
 
-template <typename T>
-nhmf_status fix_rows(nhmf_ctx* c, const T* src, T* out, int mode, T value, cudaStream_t s) {
-  if (c->prm.bc == NHMF_BC_NONE) return NHMF_OK;
-  const long long M2 = (long long)c->g.M * c->g.M;
-  k_fix_constrained<T><<<(unsigned)((M2 + 255) / 256), 256, 0, s>>>(c->prm.bc, c->g.M, c->g.M3, src, out, mode, value);
-  return cuda_check(c, cudaGetLastError(), "dirichlet rows");
-}
-
-}  // namespace
-
-namespace {
 nhmf_status apply(nhmf_ctx* c, int prec, int strat, const void* du, void* v, bool raw, const Gather32& g32,
                   cudaStream_t s) {
   switch (c->g.p) {
@@ -96,12 +81,11 @@ nhmf_status launch_diagonal(nhmf_ctx* c, double* d, cudaStream_t s) {
   return fail(c, NHMF_ERR_ARG, "degree out of range");
 }
 
-nhmf_status fix_rows64(nhmf_ctx* c, const double* src, double* out, int mode, double value, cudaStream_t s) {
-  return fix_rows<double>(c, src, out, mode, value, s);
-}
-
-nhmf_status fix_rows32(nhmf_ctx* c, const float* src, float* out, int mode, float value, cudaStream_t s) {
-  return fix_rows<float>(c, src, out, mode, value, s);
+nhmf_status fix_rows64(nhmf_ctx* c, const double* src, double* out, cudaStream_t s) {
+  if (c->prm.bc == NHMF_BC_NONE) return NHMF_OK;
+  const long long M2 = (long long)c->g.M * c->g.M;
+  k_fix_constrained<<<(unsigned)((M2 + 255) / 256), 256, 0, s>>>(c->prm.bc, c->g.M, c->g.M3, src, out);
+  return cuda_check(c, cudaGetLastError(), "dirichlet rows");
 }
 
 nhmf_status launch_to_fp32(const double* x, float* y, long long n, cudaStream_t s) {

@@ -24,22 +24,10 @@
 namespace nhmf {
 namespace {
 
-// Table slots ahead of the per-item arrays: B, Dc, D, n^3 weights and NE factors, or in the
-// apply B, Dc, BW, DcW, Dch, 3 even-odd sets and NE factors (whichever is larger).
+// Table slots ahead of the per-item arrays, the most of any kernel: B, Dc, BW, DcW, Dch, 3 even-odd sets
+// and NE factors in the apply, 7 tables, an even-odd set and NE factors in the diagonal.
 constexpr int kTabSlots = 3 * kMaxN * kMaxN + 128 + 32;
 static_assert(5 * kMaxN * kMaxN + 3 * kEoSlots + 32 <= kTabSlots, "apply tables exceed the table slots");
-
-template <int P, typename T>
-__device__ __forceinline__ void load_tables(const OpArgs& a, T* sB, T* sDc, T* sD, T* sW, double wscale) {
-  constexpr int n = P + 1;
-  for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
-    sB[i] = T(a.B[i]);
-    sDc[i] = T(a.Dc[i]);
-    sD[i] = T(a.D[i]);
-  }
-  for (int q = threadIdx.x; q < n * n * n; q += blockDim.x)
-    sW[q] = T(a.w[q % n] * a.w[(q / n) % n] * a.w[q / (n * n)] * wscale);
-}
 
 // The apply's tables: B and Dc (forward), BW and DcW (transposed, carrying w, mu, h), Dch and
 // the even-odd coefficient sets, laid out as in k_apply.
@@ -160,9 +148,6 @@ __device__ __forceinline__ void transposed(const T* sBW, const T* sDcW, const T*
 // dP / mu without any scaling.  For odd n (Q2, Q4) every non-accumulating pass (forward B,
 // forward collocation derivative, transposed B) runs one thread per line in even-odd form, and
 // the gradient of du reaches the point code through shared memory.
-#ifndef NHMF_LINEMAP
-#define NHMF_LINEMAP 1
-#endif
 template <int P, typename T, int STRAT, int MODEL, bool SMALL>
 __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(const OpArgs a) {
   constexpr int n = P + 1, n3 = n * n * n, NE = Shape<P, T, STRAT, SMALL>::NE, NI = NE * n3;
@@ -194,10 +179,7 @@ __global__ void __launch_bounds__(Shape<P, T, STRAT, SMALL>::THREADS) k_apply(co
   __syncthreads();
 
   if constexpr (STRAT == NHMF_ON_THE_FLY) {
-    if (sizeof(T) == 8)
-      gather<P, NI>(a, col, a.u64, e0, nvalid, false, G);
-    else
-      gather<P, NI>(a, col, a.u32, e0, nvalid, false, G);
+    gather<P, NI>(a, col, a.u64, e0, nvalid, false, G);
     __syncthreads();
     if constexpr (EO) {
       eo_pass<n, NI, 3, 0, false, kEoCentreRow, TH>(kB, G, Vq, nlines);
@@ -649,14 +631,13 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
   constexpr int n = P + 1, n3 = n * n * n, NE = Shape<P, T, NHMF_CACHED, SMALL>::NE, NI = NE * n3;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sB = reinterpret_cast<T*>(smem_raw);
-  T* sDc = sB + kMaxN * kMaxN;
-  T* sD = sDc + kMaxN * kMaxN;
-  T* sW = sD + kMaxN * kMaxN;
+  T* sDch = sB + kMaxN * kMaxN;
   T* A = sB + kTabSlots;  // [3][NI]
   T* Vq = A + 3 * NI;     // [3][NI]
-  load_tables<P>(a, sB, sDc, sD, sW, 1.0);
-  __syncthreads();
-  for (int i = threadIdx.x; i < n * n; i += blockDim.x) sDc[i] = a.Dch[i];  // physical gradients
+  for (int i = threadIdx.x; i < n * n; i += blockDim.x) {
+    sB[i] = a.B[i];
+    sDch[i] = a.Dch[i];  // physical gradients
+  }
   long long e0;
   const Colour col = block_colour<NE>(a.N, e0);  // one launch: the classes are independent here
   const int nvalid = (int)min((long long)NE, (long long)col.count - e0);
@@ -667,7 +648,7 @@ __global__ void __launch_bounds__(Shape<P, double, NHMF_CACHED, SMALL>::THREADS)
   bool bad = false;
   for (int t = threadIdx.x; t < nvalid * n3; t += blockDim.x) {
     double H[9], Fi[9], lnJ;
-    colloc_grad<n, NI>(sDc, Vq, t, H);
+    colloc_grad<n, NI>(sDch, Vq, t, H);
     const double Jm1 = kinematics(H, Fi, lnJ);
     bad |= !(Jm1 > -1.0);
     if (a.cache64_out) {
@@ -1075,7 +1056,6 @@ OpArgs base_args(nhmf_ctx* c) {
       a.Bf[q * n + i] = float(c->tab.B[q][i]);
       a.Dcf[q * n + i] = float(c->tab.Dc[q][i]);
     }
-    a.wf[q] = float(c->tab.w[q]);
   }
   // tables of the tangent apply (see OpArgs)
   double BWt[kMaxN * kMaxN];

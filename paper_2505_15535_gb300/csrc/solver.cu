@@ -830,7 +830,7 @@ static nhmf_status solve_impl(nhmf_ctx* c, const nhmf_solve_opts* o, double* u, 
         if ((st = launch_apply(c, NHMF_FP64, o->strategy, w.d, w.t, x.s, true)) != NHMF_OK) return st;
         axpby(x.n, -1.0, nullptr, w.t, 1.0, nullptr, w.b, x.s);        // b -= K d
       }
-      if ((st = fix_rows64(c, w.d, w.b, 0, 0.0, x.s)) != NHMF_OK) return st;  // b_D = d_D
+      if ((st = fix_rows64(c, w.d, w.b, x.s)) != NHMF_OK) return st;  // b_D = d_D
       if ((st = norm(x, w.b, TMP, &bnh)) != NHMF_OK) return st;
       if (ref < 0.0) ref = bnh;
       if (dn == 0.0 && (bnh <= o->newton_rtol * ref || bnh == 0.0)) {

@@ -90,9 +90,9 @@ struct OpArgs {
   double eo[3][kEoSlots];
   double eoh[kEoSlots];  // of Dch
   double r2mu;
-  int reg32;  // FP32 point cache in the register kernel's [10][n^3][E] layout (see kRegMaxP)
+  int reg32;  // FP32 point cache in the register kernel's tiles [E/32][10][n^3][32] (see kRegMaxP)
   float BWf[kMaxN * kMaxN], DcWf[kMaxN * kMaxN], Dchf[kMaxN * kMaxN], eof[3][kEoSlots];  // FP32 copies
-  float Bf[kMaxN * kMaxN], Dcf[kMaxN * kMaxN], wf[kMaxN];  // FP32 copies (register kernels)
+  float Bf[kMaxN * kMaxN], Dcf[kMaxN * kMaxN];  // FP32 copies (register kernels)
   EoTab cB, cD, cBT, cDT, cBTz, cDTz;  // B, D and the weighted transposes; z: times mu h
   float invhf, r2muf;                  // 1 / h, r2mu
   const double* u64;
