@@ -21,6 +21,9 @@
 namespace nhmf {
 namespace {
 
+// Elements and threads of a block, and blocks an SM.  Five at Q3 for both models: four, with which the
+// split model's on-the-fly instance does not spill (88 bytes at five), measure the same (on the fly,
+// five / four: 47^3 172.1 / 171.4 us, split 189.8 / 189.4; 36^3 74.9 / 74.6, split 86.0 / 84.4).
 template <int n> struct ColShape;
 template <> struct ColShape<3> { static constexpr int NE = 16, THREADS = 160, BLOCKS = 4; };
 template <> struct ColShape<4> { static constexpr int NE = 8, THREADS = 128, BLOCKS = 5; };

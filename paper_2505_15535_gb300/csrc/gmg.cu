@@ -143,7 +143,8 @@ __global__ void k_to(long long n, const double* __restrict__ x, T* __restrict__ 
 constexpr int kB = 1216, kT = 256;
 // Nodes per direction up to which a transfer is one launch.  Above it too few planes read too much:
 // Q4 16^3 linear solve (65 nodes) 79.3 ms with three launches everywhere, 78.2 with one up to 33,
-// 89.5 up to 65; Newton step Q2 16^3 (33 nodes) 10.4, 9.9 and 9.9 ms.
+// 89.5 up to 65; Newton step Q2 16^3 (33 nodes) 10.4, 9.9 and 9.9 ms.  In between, one up to 33 / up to
+// 64: Q3 16^3 (49 nodes) 7.24 / 7.54 ms, Q4 12^3 (49) 11.6 / 12.1, Q2 24^3 (49) 7.44 / 7.58.
 constexpr int kMap3dMax = 33;
 unsigned ew_blocks(long long n) { return (unsigned)std::min<long long>(kB, (n + kT - 1) / kT); }
 

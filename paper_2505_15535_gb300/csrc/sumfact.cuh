@@ -50,9 +50,18 @@ template <> struct LaunchCfg<2, double, NHMF_ON_THE_FLY> {
 // Block shapes: the launch shape above, and for the FP64 and double-float kernels (issue bound
 // within an SM) small blocks of one to four elements for meshes whose normal blocks would not give
 // every SM `per_sm` of them: a block of 27 Q2 elements keeps one SM's FP64 pipe busy for 34 us
-// while the others idle.  The line: FP64 cached apply, small / normal blocks, Q2 12^3 40 / 87 us,
-// 24^3 142 / 146, 32^3 312 / 306; Q4 12^3 113 / 119, 32^3 1819 / 1721.  Double-float blocks take
-// less time each: Q2 16^3 50 / 75 us, 24^3 101 / 94; Q4 8^3 49 / 67, 12^3 91 / 87.
+// while the others idle.  The line, small / normal blocks in us just below it and just above (Q1
+// 24^3, 34^3; Q2 20^3, 28^3; Q3 14^3, 18^3; Q4 10^3, 14^3):
+//   cached       43/44 88/93    81/107 206/203   78/100 148/177   70/96 167/187
+//   on the fly   58/60 138/146  125/140 319/316  114/142 229/238  100/131 247/281
+//   Algorithm 2  53/54 129/134  112/124 287/298  100/119 195/219  93/107 207/215
+//   residual     63/69 112/114  102/126 225/213  99/127 172/176   90/114 186/191
+//   point cache  50/51 87/88    88/79 176/167    77/89 124/126    72/80 131/145
+// and far below it Q2 8^3 takes 0.35 to 0.66 of the normal blocks' time.  The diagonal, whose normal
+// blocks hold half the elements, has its line there too (Q2 16^3 54/77, 20^3 87/90; Q3 8^3 0.97) and
+// loses up to 17 % to it at Q1 and Q3 (24^3 44/38, 14^3 87/78).  Double-float blocks take less time
+// each: Q2 16^3 44/69, 20^3 56/75, 28^3 122/112; Q3 14^3 48/58, 18^3 88/74; Q4 12^3 66/72, 14^3 94/86;
+// at Q1 the normal blocks are 5 to 20 % faster at every size.
 template <typename T> struct SmallRule { static constexpr int per_sm = 4; };
 template <> struct SmallRule<df64> { static constexpr int per_sm = 2; };
 template <int P> struct SmallCfg;

@@ -1085,7 +1085,8 @@ __global__ void __launch_bounds__(kTcThreads, 4) k_up_tc(const ConvArgs a, int z
 // chunk of 16 positions a warp loads three A fragments (P^T of the three planes) and three B
 // fragments (the dx shifts of its dy) for 9 taps, 6 ldmatrix.x4 for 18 MMAs.  With the shifts
 // all on Q a warp took 4 for 6 MMAs, and the shared-memory pipe bounded the kernel (129^3: 140 us
-// a launch, now 121); mma.sync issue bounds it, one m16n8k16 in 4.6 clocks of an SM.  So the
+// a launch, now 118); mma.sync bounds it, one m16n8k16 in 4.9 clocks of an SM (the tensor pipe is active
+// in 62 % of them, and the stall is the wait for an MMA's result).  So the
 // layers with three channels on one side take the MMAs of their eight-channel tile only (NT =
 // 1): the input layer has them on Q; the output layer has them on P and swaps the operands,
 // G[tap][a][b] = sum_v Q[v][b] P[v - d_tap][a] (SWAP: rows are b, tap 26 - tap).  3 warps, one
