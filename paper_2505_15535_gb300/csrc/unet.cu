@@ -1433,9 +1433,18 @@ int tc_column(long long per_plane, int m) {
   return (int)std::max<long long>(1, std::min<long long>(kTcZ, per_plane * m / kTcUnits));
 }
 
+// The limit of dynamic shared memory belongs to the kernel on its device: the same one for every grid,
+// so that a network on a smaller grid does not lower it under another host thread's launch.  The most
+// any kernel takes (the stride-2 weight gradient, 82 KB) lies below it on every grid.
+constexpr int kSmemLimit = 100 * 1024;
+template <typename KernelT>
+void allow_smem(KernelT* kernel) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit);
+}
+
 void up_tc_launch(const ConvArgs& a, unsigned* status, cudaStream_t s) {
   const size_t smem = up_tc_smem(a.m_in);
-  cudaFuncSetAttribute(k_up_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_up_tc);
   const long long mi = a.m_in, per_plane = (mi * (mi + 1) + 127) / 128;
   const int zc = tc_column(per_plane, (int)mi);
   const long long nunits = per_plane * ((mi + zc - 1) / zc);
@@ -1484,7 +1493,7 @@ void conv_tc_launch(const ConvArgs& a, unsigned* status, cudaStream_t s) {
     return;
   }
   const size_t smem = conv_tc_smem(m);
-  cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_conv_tc);
   cudaFuncSetAttribute(k_conv_tc, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   const long long per_plane = ((long long)m * R + 127) / 128;
   int dev = 0, nsm = 0, smem_sm = 0;  // of the current device (attribute queries are cheap)
@@ -1504,7 +1513,7 @@ void down_tc_launch(const ConvArgs& a, unsigned* status, cudaStream_t s) {
   const int mo = a.m_out;
   const int nstrips = (mo + kDnStripMax - 1) / kDnStripMax, W = (mo + nstrips - 1) / nstrips;
   const size_t smem = down_tc_smem(W);
-  cudaFuncSetAttribute(k_down_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_down_tc);
   cudaFuncSetAttribute(k_down_tc, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   const long long per_plane = ((long long)mo * (W + 2) + 127) / 128;
   int dev = 0, nsm = 0, smem_sm = 0;
@@ -1544,7 +1553,7 @@ void wgrad(UNet& u, int layer, int gather, const __nv_bfloat16* P, int mp, const
     const UNetLayer& L = u.L[layer];
     const bool swap = L.cout <= 8;  // three output channels: the operands change sides
     auto* kernel = swap ? k_wgrad_s1<1, true> : L.cin <= 8 ? k_wgrad_s1<1, false> : k_wgrad_s1<2, false>;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(kernel);
     const long long per_plane = ((long long)mp * (W + 2) + 127) / 128;
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
@@ -1558,7 +1567,7 @@ void wgrad(UNet& u, int layer, int gather, const __nv_bfloat16* P, int mp, const
     int nseg = 0;
     const int seg = wgrad_s2_seg(mp, &nseg);
     const size_t smem = wgrad_s2_smem(seg);
-    cudaFuncSetAttribute(k_wgrad_s2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_wgrad_s2);
     const long long per_plane = (long long)mp * nseg;
     const int zc = (int)std::max<long long>(1, std::min<long long>(kTcZ, per_plane * mp / kTcUnits));
     blocks = (int)std::min<long long>(kWgBlocks, per_plane * ((mp + zc - 1) / zc));
